@@ -320,7 +320,8 @@ int stag_cg_solve_batched_mixed(int n, stag_lattice *lats, stag_field *xs, const
  * each after 2 warm-ups, CUDA events on the lattice stream):
  *   STAG_TUNE_DSLASH  the Dslash: block 64, 128, 256 or 512 threads, in two
  *                     register variants (regs 1: the compiler's choice,
- *                     2: at most 64 registers, 1024 resident threads per SM)
+ *                     2: capped for 768 to 1024 resident threads per SM, by
+ *                     format)
  *                     and, for STAG_F16 on 12-real links with Lt a multiple
  *                     of 4 and at least 8, regs 3: two sites (x, y, z, t)
  *                     and (x, y, z, t + Lt/2) per thread in packed FP32x2

@@ -253,6 +253,7 @@ static inline DslashArgs dslash_args(stag_lattice lat, int prec, int out_par, co
         for (int k = 0; k < 4; k++)
             a.bc_neg[k] = lat->bc[k] < 0 ? 1 : 0;
     }
+    a.keep = link_keep_sites(prec, a.compressed);
     return a;
 }
 
@@ -339,8 +340,7 @@ static inline cudaError_t enqueue_m_pap(stag_lattice lat, int prec, const void *
     cudaError_t e = launch_dslash(prec, EPI_M_PART, a, block, s);
     if (e != cudaSuccess)
         return e;
-    const int n = pair16_used(prec, EPI_M_PART, a) ? dslash_pair16_grid(lat->geom, block) : dslash_grid(lat->geom, block);
-    return launch_pap_finish(lat->partial, n, lat->sc, skip_if_done, s, gate);
+    return launch_pap_finish(lat->partial, dslash_blocks(prec, EPI_M_PART, a, block), lat->sc, skip_if_done, s, gate);
 }
 
 // Source normalisation (stag_api.cu): when the exponent k of b's largest

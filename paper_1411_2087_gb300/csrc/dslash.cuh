@@ -47,11 +47,12 @@ struct DslashArgs {
     int c0b, cnb;           // with cn > 0: also sites c0b .. c0b+cnb-1 (cnb = 0: none)
     float inv_c[2];         // 1/c1, 1/c3: the reconstruction divides by s = c eta b
     int bc_neg[4];          // boundary sign of direction mu is -1
+    int keep;               // links of checkerboard sites below keep stay in L2, the others are evicted first
     int regs;               // EPI_NONE, EPI_M_PART: REGS_* (autotuned)
 };
 
 // register variant of the stencil (DslashArgs::regs): the launcher's
-// measured default, the compiler's free choice, at most 64 registers, or
+// measured default, the compiler's free choice, capped (kCapThreads), or
 // (16-bit stencil, EPI_NONE and EPI_M_PART) two sites per thread in packed
 // FP32x2 arithmetic with the loads through a shared-memory ring
 // (stencil16_pair_async) where pair16_applies, else the default
@@ -83,8 +84,8 @@ STAG_HD int hop_wraps(int v, int s, int L) {
 // the nine entries of one link of kind `kind` (compression mask CM): either
 // stored whole, or rows 0 and 1 of the 12-real layout with row 2 rebuilt
 // (inv_s = 1/(c eta b) of that link)
-template <int P, int CM>
-STAG_D void load_link(const void *G, int kind, int S, int idx, float ls, float inv_s,
+template <int P, int CM, int LD>
+STAG_D void load_link(const void *G, int kind, int S, int idx, float ls, float inv_s, l2pol pol,
                       cplx<typename Fmt<P>::R> L[9]) {
     using F = Fmt<P>;
     using E = typename F::Elem;
@@ -92,7 +93,7 @@ STAG_D void load_link(const void *G, int kind, int S, int idx, float ls, float i
     if constexpr (CM != 0) {
         const char *kb = (const char *)G + link_kind_offset(P, CM, kind, (size_t)S);
         if ((CM >> (kind >> 2)) & 1) {
-            C12<P>::load(kb, S, idx, ls, L);
+            C12<P>::template load<LD>(kb, S, idx, ls, pol, L);
             reconstruct_row2(L, inv_s);
             return;
         }
@@ -106,7 +107,7 @@ STAG_D void load_link(const void *G, int kind, int S, int idx, float ls, float i
     }
 #pragma unroll
     for (int e = 0; e < 9; e++)
-        L[e] = F::unpack_link(ld_stream(Lp + e * S), ls);
+        L[e] = F::unpack_link(ld_link<LD>(Lp + e * S, pol), ls);
 }
 
 }  // namespace stag
@@ -117,69 +118,70 @@ namespace stag {
 
 // acc += D psi at checkerboard site c of parity par (links with compression
 // mask CM)
-template <int P, int CM = 0>
+template <int P, int CM, int LD>
 STAG_D void dslash_site(const Geom &g, int par, int c, const void *__restrict__ Gout,
                         const void *__restrict__ Gin, const typename Fmt<P>::Elem *__restrict__ in,
                         const DslashArgs &a, cplx<typename Fmt<P>::R> acc[3]) {
     using R = typename Fmt<P>::R;
     if constexpr (P == P_F16) {
         // raw integer units (stencil16.cuh)
-        stencil16_site<CM>(g, par, c, Gout, Gin, in, a, acc);
-        return;
-    }
-    const int S = g.stride;
-    int x[4];
-    cb_coords(g, c, par, x);
+        stencil16_site<CM, LD>(g, par, c, Gout, Gin, in, a, acc);
+    } else {
+        const int S = g.stride;
+        int x[4];
+        cb_coords(g, c, par, x);
+        const LinkPolicy<LD> pol(a.keep);
 #pragma unroll
-    for (int mu = 0; mu < 4; mu++) {
-        // Kogut-Susskind phase of direction mu at x (equal at x - s mu)
-        int esum = 0;
+        for (int mu = 0; mu < 4; mu++) {
+            // Kogut-Susskind phase of direction mu at x (equal at x - s mu)
+            int esum = 0;
 #pragma unroll
-        for (int nu = 0; nu < mu; nu++)
-            esum += x[nu];
+            for (int nu = 0; nu < mu; nu++)
+                esum += x[nu];
 #pragma unroll
-        for (int h = 0; h < 2; h++) {
-            const int s = h ? 3 : 1;
-            const int kind = 4 * h + mu;
-            const float ls = a.link_scale[h];
-            // forward: + L(x) psi(x + s mu)
-            {
-                const int j = cb_hop(g, c, x, mu, +s);
-                cplx<R> v[3];
-                load_vec<P>(in, S, j, v);
-                float inv_s = 0.f;
-                if ((CM >> h) & 1) {
-                    const int flip = (esum + (a.bc_neg[mu] ? hop_wraps(x[mu], s, g.L[mu]) : 0)) & 1;
-                    inv_s = flip ? -a.inv_c[h] : a.inv_c[h];
+            for (int h = 0; h < 2; h++) {
+                const int s = h ? 3 : 1;
+                const int kind = 4 * h + mu;
+                const float ls = a.link_scale[h];
+                // forward: + L(x) psi(x + s mu)
+                {
+                    const int j = cb_hop(g, c, x, mu, +s);
+                    cplx<R> v[3];
+                    load_vec<P>(in, S, j, v);
+                    float inv_s = 0.f;
+                    if ((CM >> h) & 1) {
+                        const int flip = (esum + (a.bc_neg[mu] ? hop_wraps(x[mu], s, g.L[mu]) : 0)) & 1;
+                        inv_s = flip ? -a.inv_c[h] : a.inv_c[h];
+                    }
+                    cplx<R> L[9];
+                    load_link<P, CM, LD>(Gout, kind, S, c, ls, inv_s, pol.of(c), L);
+#pragma unroll
+                    for (int r = 0; r < 3; r++)
+#pragma unroll
+                        for (int b = 0; b < 3; b++)
+                            cmac(acc[r], L[3 * r + b], v[b]);
                 }
-                cplx<R> L[9];
-                load_link<P, CM>(Gout, kind, S, c, ls, inv_s, L);
-#pragma unroll
-                for (int r = 0; r < 3; r++)
+                // backward: - L(x - s mu)^+ psi(x - s mu)
+                {
+                    const int j = cb_hop(g, c, x, mu, -s);
+                    cplx<R> v[3];
+                    load_vec<P>(in, S, j, v);
 #pragma unroll
                     for (int b = 0; b < 3; b++)
-                        cmac(acc[r], L[3 * r + b], v[b]);
-            }
-            // backward: - L(x - s mu)^+ psi(x - s mu)
-            {
-                const int j = cb_hop(g, c, x, mu, -s);
-                cplx<R> v[3];
-                load_vec<P>(in, S, j, v);
+                        v[b] = cneg(v[b]);
+                    float inv_s = 0.f;
+                    if ((CM >> h) & 1) {
+                        const int flip = (esum + (a.bc_neg[mu] ? hop_wraps(x[mu], -s, g.L[mu]) : 0)) & 1;
+                        inv_s = flip ? -a.inv_c[h] : a.inv_c[h];
+                    }
+                    cplx<R> L[9];
+                    load_link<P, CM, LD>(Gin, kind, S, j, ls, inv_s, pol.of(j), L);
 #pragma unroll
-                for (int b = 0; b < 3; b++)
-                    v[b] = cneg(v[b]);
-                float inv_s = 0.f;
-                if ((CM >> h) & 1) {
-                    const int flip = (esum + (a.bc_neg[mu] ? hop_wraps(x[mu], -s, g.L[mu]) : 0)) & 1;
-                    inv_s = flip ? -a.inv_c[h] : a.inv_c[h];
+                    for (int r = 0; r < 3; r++)
+#pragma unroll
+                        for (int b = 0; b < 3; b++)
+                            cmac_conj(acc[r], L[3 * b + r], v[b]);
                 }
-                cplx<R> L[9];
-                load_link<P, CM>(Gin, kind, S, j, ls, inv_s, L);
-#pragma unroll
-                for (int r = 0; r < 3; r++)
-#pragma unroll
-                    for (int b = 0; b < 3; b++)
-                        cmac_conj(acc[r], L[3 * b + r], v[b]);
             }
         }
     }
@@ -276,6 +278,10 @@ STAG_D void dslash_reduce(const DslashArgs &a, T dot, double *smem) {
     }
 }
 
+// the link loads of the one-site kernels (link_keep_sites has the figures):
+// the double-float kernel runs on lattices whose links are many times the L2
+template <int P> constexpr int kLinkLoad = P == P_F32 ? LD_KEEP : LD_STREAM;
+
 template <int P, int EPI, int BLOCK, int CM>
 STAG_D void dslash_body(const DslashArgs &a) {
     using F = Fmt<P>;
@@ -295,7 +301,7 @@ STAG_D void dslash_body(const DslashArgs &a) {
     red_t<R> dot = red_zero<red_t<R>>();
     if (i < n1 + n2) {
         cplx<R> acc[3] = {czero<R>(), czero<R>(), czero<R>()};
-        dslash_site<P, CM>(a.g, a.out_par, c, a.links_out, a.links_in, (const E *)a.in, a, acc);
+        dslash_site<P, CM, kLinkLoad<P>>(a.g, a.out_par, c, a.links_out, a.links_in, (const E *)a.in, a, acc);
         dot = dslash_epilogue<P, EPI>(a, c, acc);
     }
     dslash_reduce<EPI, BLOCK>(a, dot, smem);
@@ -334,24 +340,36 @@ STAG_D void pair16_body(const DslashArgs &a) {
     dslash_reduce<EPI, BLOCK>(a, dot, smem);
 }
 
-// One launch of the stencil.  The capped form asks for at least 1024 resident
-// threads per SM (at most 64 registers).  Left free, the compiler gives the
-// uncompressed FP32 kernels so few registers (32-44) that too few loads are
-// in flight; the launcher picks the capped form for those and for the
-// 16-bit ones (kCapped) and the free one for the rest.
+// One launch of the stencil.  The capped form asks for kCapThreads resident
+// threads per SM.  Left free, the compiler gives the uncompressed FP32
+// kernels so few registers (40) that too few loads are in flight; the
+// launcher picks the capped form for FP32 and 16-bit links (kCapped) and the
+// free one for the rest.  The free double-float kernel asks for 768 (80
+// registers, as many as it takes unasked, but ordered for it: a plain-CG
+// iteration at 32^3x64 929 -> 852 us).
 template <int P, int EPI, int BLOCK, int CM = 0>
-__global__ void __launch_bounds__(BLOCK) dslash_kernel(DslashArgs a) {
+__global__ void __launch_bounds__(BLOCK, P == P_DF64 ? (768 + BLOCK - 1) / BLOCK : 0) dslash_kernel(DslashArgs a) {
     dslash_body<P, EPI, BLOCK, CM>(a);
 }
+
+// by measurement of 1024, 896, 768, 640 and 512 (an iteration of mixed CG at
+// 24^3x48 and 32^3x64): FP32 full links 166, 463 us at 1024 against 158, 462
+// at 896, 12-real three-link links 146, 406 against 141, 406; all links
+// 12-real 128, 358 against 124, 355 at 768 (free: 133, 364); 16-bit 12-real
+// 113, 287 against 107, 277 at 768, three-link only 103, 263 against 105,
+// 272 at 896, full 108, 283 against 107, 283
+template <int P, int CM>
+constexpr int kCapThreads = P == P_F32 ? (CM == 3 ? 768 : 896) : P == P_F16 && CM == 3 ? 768 : 1024;
 
 template <int P, int EPI, int BLOCK, int CM>
-__global__ void __launch_bounds__(BLOCK, 1024 / BLOCK) dslash_kernel_capped(DslashArgs a) {
+__global__ void __launch_bounds__(BLOCK, (kCapThreads<P, CM> + BLOCK - 1) / BLOCK) dslash_kernel_capped(DslashArgs a) {
     dslash_body<P, EPI, BLOCK, CM>(a);
 }
 
-// whether a launch of precision prec and epilogue epi runs the pair form
-STAG_HD bool pair16_used(int prec, int epi, const DslashArgs &a) {
-    return prec == P_F16 && a.regs == REGS_PAIR &&
+// whether a launch of precision prec, epilogue epi and block size block
+// runs the pair form
+STAG_HD bool pair16_used(int prec, int epi, const DslashArgs &a, int block) {
+    return prec == P_F16 && a.regs == REGS_PAIR && pair16_ring(block, a.compressed) > 0 &&
            (epi == EPI_NONE || epi == EPI_M_PART) &&
            a.c0 == 0 && (a.cn == 0 || a.cn == a.g.Vh) && a.cnb == 0 && pair16_applies(a.g);
 }

@@ -1,21 +1,16 @@
 // Launcher template of the Dslash kernels; each precision is instantiated in
 // its own translation unit (dslash_<prec>.cu) so that they compile in parallel.
 #pragma once
-#include "dslash.cuh"
+#include "dslash_split.cuh"
 #include "kernels.h"
 
 namespace stag {
 
-// Which kernels run under the register cap by default (before tuning), by
-// measurement (48^3x96, kernel times inside the mixed solves).  Left free,
-// the compiler gives these 32-44 registers and keeps too few stencil loads
-// in flight:
-//   FP32 uncompressed          D_oe 947 -> 901 us, M with partials 954 -> 913 us
-//   16-bit, one site           M with <p, Mp> partials 635 -> 557 us (full links)
-// FP32 on 12-real links (56-62 registers free) and the FP64 and double-float
-// kernels (HBM-bound at their free choice) keep the compiler's choice.
-template <int P, int EPI, int CM>
-constexpr bool kCapped = P == P_F16 || (P == P_F32 && CM != 3);
+// Which kernels run under the register cap by default (before tuning):
+// FP32 and 16-bit (the figures are at kCapThreads).  The FP64 kernel is
+// bound by the FP64 pipe and keeps the compiler's choice.
+template <int P>
+constexpr bool kCapped = P == P_F16 || P == P_F32;
 
 // The plain stencil and the M stencil with <p, Mp> partials (the solvers'
 // two kernels per iteration) are instantiated in both register variants, so
@@ -24,23 +19,50 @@ template <int P, int EPI, int BLOCK, int CM>
 static void launch_one(int grid, const DslashArgs &a, cudaStream_t s) {
     constexpr bool tunable = EPI == EPI_NONE || EPI == EPI_M_PART;
     const bool capped = tunable && a.regs != REGS_DEFAULT && a.regs != REGS_PAIR ? a.regs == REGS_CAPPED
-                                                                                 : kCapped<P, EPI, CM>;
+                                                                                 : kCapped<P>;
     if constexpr (tunable) {
         if (capped)
             dslash_kernel_capped<P, EPI, BLOCK, CM><<<grid, BLOCK, 0, s>>>(a);
         else
             dslash_kernel<P, EPI, BLOCK, CM><<<grid, BLOCK, 0, s>>>(a);
-    } else if constexpr (kCapped<P, EPI, CM>) {
+    } else if constexpr (kCapped<P>) {
         dslash_kernel_capped<P, EPI, BLOCK, CM><<<grid, BLOCK, 0, s>>>(a);
     } else {
         dslash_kernel<P, EPI, BLOCK, CM><<<grid, BLOCK, 0, s>>>(a);
     }
 }
 
+// the split form with NG warps per block
+template <int P, int NG, int CM>
+static cudaError_t launch_split_g(int epi, const DslashArgs &a, cudaStream_t s) {
+    const int grid = dslash_blocks(P, epi, a, 0), block = 32 * NG;
+    if (grid == 0)
+        return cudaSuccess;
+    switch (epi) {
+    case EPI_NONE: dslash_split_kernel<P, EPI_NONE, NG, CM><<<grid, block, 0, s>>>(a); break;
+    case EPI_M: dslash_split_kernel<P, EPI_M, NG, CM><<<grid, block, 0, s>>>(a); break;
+    case EPI_M_PAP: dslash_split_kernel<P, EPI_M_PAP, NG, CM><<<grid, block, 0, s>>>(a); break;
+    case EPI_RESID: dslash_split_kernel<P, EPI_RESID, NG, CM><<<grid, block, 0, s>>>(a); break;
+    case EPI_RESID_STORE: dslash_split_kernel<P, EPI_RESID_STORE, NG, CM><<<grid, block, 0, s>>>(a); break;
+    case EPI_M_PART: dslash_split_kernel<P, EPI_M_PART, NG, CM><<<grid, block, 0, s>>>(a); break;
+    default: return cudaErrorInvalidValue;
+    }
+    return cudaGetLastError();
+}
+
+template <int P, int CM>
+static cudaError_t launch_split(int epi, const DslashArgs &a, cudaStream_t s) {
+    switch (split_warps(P, a.compressed, a.g)) {
+    case 4: return launch_split_g<P, 4, CM>(epi, a, s);
+    case 8: return launch_split_g<P, 8, CM>(epi, a, s);
+    default: return cudaErrorInvalidValue;
+    }
+}
+
 template <int P, int BLOCK, int CM>
 static cudaError_t launch_p_b_c(int epi, const DslashArgs &a, cudaStream_t s) {
     if constexpr (P == P_F16 && pair16_ring<BLOCK, CM>() > 0) {
-        if (pair16_used(P, epi, a)) {
+        if (pair16_used(P, epi, a, BLOCK)) {
             const int grid = dslash_pair16_grid(a.g, BLOCK);
             if (epi == EPI_NONE)
                 dslash_pair16_kernel<EPI_NONE, BLOCK, CM><<<grid, BLOCK, 0, s>>>(a);
@@ -49,8 +71,7 @@ static cudaError_t launch_p_b_c(int epi, const DslashArgs &a, cudaStream_t s) {
             return cudaGetLastError();
         }
     }
-    const int n = (a.cn ? a.cn : a.g.Vh) + (a.cn ? a.cnb : 0);
-    const int grid = (n + BLOCK - 1) / BLOCK;
+    const int grid = dslash_blocks(P, epi, a, BLOCK);
     if (grid == 0)
         return cudaSuccess;
     switch (epi) {
@@ -84,6 +105,17 @@ static cudaError_t launch_p_b(int epi, const DslashArgs &a, cudaStream_t s) {
 }
 
 template <int P> cudaError_t launch_dslash_p(int epi, const DslashArgs &a, int block, cudaStream_t s) {
+    if constexpr (P != P_F16) {
+        if (split_warps(P, a.compressed, a.g) > 0) {
+            if constexpr (P == P_F32) {
+                if (a.compressed == 2)
+                    return launch_split<P, 2>(epi, a, s);
+                if (a.compressed == 3)
+                    return launch_split<P, 3>(epi, a, s);
+            }
+            return a.compressed ? cudaErrorInvalidValue : launch_split<P, 0>(epi, a, s);
+        }
+    }
     switch (block) {
     case 64: return launch_p_b<P, 64>(epi, a, s);
     case 128: return launch_p_b<P, 128>(epi, a, s);

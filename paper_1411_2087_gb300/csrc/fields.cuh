@@ -22,6 +22,73 @@ enum Prec { P_F64 = 0, P_F32 = 1, P_F16 = 2, P_DF64 = 3 };
 // cache hints: links stream through once (evict-first); colour vectors are
 // gathered 16 times per launch and should stay in L1/L2.
 template <class T> STAG_D T ld_stream(const T *p) { return __ldcs(p); }
+
+// How a kernel loads its links (the loads' LD parameter):
+//   LD_STREAM  streaming loads (ld.global.cs)
+//   LD_KEEP    past L1, with an L2 policy per site: links below a site index
+//              stay in L2 for the next launch on the same lattice, the others
+//              are evicted first
+enum { LD_STREAM = 0, LD_KEEP = 1 };
+typedef unsigned long long l2pol;  // an L2 cache policy
+template <int LD> struct LinkPolicy {
+    l2pol first = 0, normal = 0;
+    int keep = 0;
+    STAG_D explicit LinkPolicy(int keep_sites) {
+        if (LD == LD_KEEP) {
+            asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(first));
+            asm("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(normal));
+            keep = keep_sites;
+        }
+    }
+    STAG_D l2pol of(int site) const { return LD == LD_KEEP && site < keep ? normal : first; }
+};
+template <int LD> STAG_D float4 ld_link(const float4 *p, l2pol pol) {
+    if (LD == LD_STREAM)
+        return ld_stream(p);
+    float4 v;
+    asm("ld.global.nc.L1::no_allocate.L2::cache_hint.v4.f32 {%0, %1, %2, %3}, [%4], %5;"
+        : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p), "l"(pol));
+    return v;
+}
+template <int LD> STAG_D double2 ld_link(const double2 *p, l2pol pol) {
+    if (LD == LD_STREAM)
+        return ld_stream(p);
+    double2 v;
+    asm("ld.global.nc.L1::no_allocate.L2::cache_hint.v2.f64 {%0, %1}, [%2], %3;"
+        : "=d"(v.x), "=d"(v.y) : "l"(p), "l"(pol));
+    return v;
+}
+template <int LD> STAG_D float2 ld_link(const float2 *p, l2pol pol) {
+    if (LD == LD_STREAM)
+        return ld_stream(p);
+    float2 v;
+    asm("ld.global.nc.L1::no_allocate.L2::cache_hint.v2.f32 {%0, %1}, [%2], %3;"
+        : "=f"(v.x), "=f"(v.y) : "l"(p), "l"(pol));
+    return v;
+}
+template <int LD> STAG_D int4 ld_link(const int4 *p, l2pol pol) {
+    if (LD == LD_STREAM)
+        return ld_stream(p);
+    int4 v;
+    asm("ld.global.nc.L1::no_allocate.L2::cache_hint.v4.s32 {%0, %1, %2, %3}, [%4], %5;"
+        : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p), "l"(pol));
+    return v;
+}
+template <int LD> STAG_D int2 ld_link(const int2 *p, l2pol pol) {
+    if (LD == LD_STREAM)
+        return ld_stream(p);
+    int2 v;
+    asm("ld.global.nc.L1::no_allocate.L2::cache_hint.v2.s32 {%0, %1}, [%2], %3;"
+        : "=r"(v.x), "=r"(v.y) : "l"(p), "l"(pol));
+    return v;
+}
+template <int LD> STAG_D int ld_link(const int *p, l2pol pol) {
+    if (LD == LD_STREAM)
+        return ld_stream(p);
+    int v;
+    asm("ld.global.nc.L1::no_allocate.L2::cache_hint.s32 %0, [%1], %2;" : "=r"(v) : "l"(p), "l"(pol));
+    return v;
+}
 template <class T> STAG_D T ld_keep(const T *p) { return __ldg(p); }
 
 template <int P> struct Fmt;
@@ -101,11 +168,11 @@ template <int P> struct C12;
 
 template <> struct C12<P_F32> {
     STAG_HD static size_t kind_bytes(size_t S) { return 3 * S * 16; }
-    STAG_D static void load(const char *kind_base, int S, int idx, float, cplx<float> L[6]) {
+    template <int LD> STAG_D static void load(const char *kind_base, int S, int idx, float, l2pol pol, cplx<float> L[6]) {
         const float4 *p = (const float4 *)kind_base;
 #pragma unroll
         for (int k = 0; k < 3; k++) {
-            const float4 v = ld_stream(p + k * S + idx);
+            const float4 v = ld_link<LD>(p + k * S + idx, pol);
             L[2 * k] = cplx<float>{v.x, v.y};
             L[2 * k + 1] = cplx<float>{v.z, v.w};
         }
@@ -121,9 +188,9 @@ template <> struct C12<P_F16> {
     STAG_D static cplx<float> q(int v, float scale) {
         return cplx<float>{(float)(short)(v & 0xffff) * scale, (float)(v >> 16) * scale};
     }
-    STAG_D static void load(const char *kind_base, int S, int idx, float scale, cplx<float> L[6]) {
-        const int4 a = ld_stream((const int4 *)kind_base + idx);
-        const int2 b = ld_stream((const int2 *)(kind_base + (size_t)16 * S) + idx);
+    template <int LD> STAG_D static void load(const char *kind_base, int S, int idx, float scale, l2pol pol, cplx<float> L[6]) {
+        const int4 a = ld_link<LD>((const int4 *)kind_base + idx, pol);
+        const int2 b = ld_link<LD>((const int2 *)(kind_base + (size_t)16 * S) + idx, pol);
         L[0] = q(a.x, scale);
         L[1] = q(a.y, scale);
         L[2] = q(a.z, scale);
@@ -167,12 +234,12 @@ struct L16 {
             return (short2 *)(kb + 16 * S) + idx * 4 + (e - 4);
         return (short2 *)(kb + 32 * S) + idx;
     }
-    STAG_D static void load(const char *kb, size_t S, int idx, int w[9]) {
-        const int4 a = ld_stream((const int4 *)kb + idx);
-        const int4 b = ld_stream((const int4 *)(kb + 16 * S) + idx);
+    template <int LD> STAG_D static void load(const char *kb, size_t S, int idx, l2pol pol, int w[9]) {
+        const int4 a = ld_link<LD>((const int4 *)kb + idx, pol);
+        const int4 b = ld_link<LD>((const int4 *)(kb + 16 * S) + idx, pol);
         w[0] = a.x, w[1] = a.y, w[2] = a.z, w[3] = a.w;
         w[4] = b.x, w[5] = b.y, w[6] = b.z, w[7] = b.w;
-        w[8] = ld_stream((const int *)(kb + 32 * S) + idx);
+        w[8] = ld_link<LD>((const int *)(kb + 32 * S) + idx, pol);
     }
 };
 

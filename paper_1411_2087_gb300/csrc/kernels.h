@@ -12,7 +12,15 @@ struct DslashArgs;
 // the default block size.
 cudaError_t launch_dslash(int prec, int epi, const DslashArgs &a, int block, cudaStream_t s);
 int dslash_default_block(int prec);
-int dslash_grid(const Geom &g, int block);
+// blocks of that launch: the partials that EPI_M_PART writes (at most
+// dslash_max_blocks of a lattice)
+int dslash_blocks(int prec, int epi, const DslashArgs &a, int block);
+inline size_t dslash_max_blocks(long long Vh) { return (size_t)(Vh + 31) / 32; }
+// warps per 32 sites of the split form (dslash_split.cuh) on this lattice;
+// 0: one thread per site
+int split_warps(int prec, int compressed, const Geom &g);
+// DslashArgs::keep of a solver's launches
+int link_keep_sites(int prec, int compressed);
 
 // CG vector kernels (grid = ceil(Vh / CG_BLOCK))
 constexpr int CG_BLOCK = 256;

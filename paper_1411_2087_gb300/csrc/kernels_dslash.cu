@@ -1,5 +1,5 @@
 // Dispatch of the Dslash launchers over precisions.
-#include "dslash.cuh"
+#include "dslash_split.cuh"
 #include "kernels.h"
 
 namespace stag {
@@ -15,7 +15,45 @@ int dslash_default_block(int prec) {
     return 128;
 }
 
-int dslash_grid(const Geom &g, int block) { return (g.Vh + block - 1) / block; }
+// Where the split form (dslash_split.cuh) is the faster one, by measurement
+// (microseconds of one plain-CG iteration, or of D_oe and D_eo in FP32;
+// split against one thread per site, at sites per parity):
+//   double-float  2048: 24.5 / 55, 46080: 58 / 69, 128000: 125 / 148,
+//                 331776: 298 / 305, 1048576: 891 / 894, 3538944: 2930 / 2898
+//   FP64          2048: 34 / 60, 20736: 74 / 97, 32768: 94 / 97, 46080: 126 / 140,
+//                 96000: 229 / 221, 1048576: 2230 / 2128; single calls lose 4 % at 50000
+//   FP32 full     65536: 23 / 28, 80000: 29 / 30, 96000: 36 / 33
+//   FP32 12-real  20736: 12 / 14 (all), 12 / 16 (three-link); 32768: 16.5 / 15, 16.5 / 16.5
+// Eight warps per 32 sites on the smallest lattices (double float, 2048
+// sites: 24.5 against 27; 10368: 31.6 against 34; 20736: 41.6 against 39.6).
+// The 16-bit stencil has no split form.
+int split_warps(int prec, int compressed, const Geom &g) {
+    const int most = prec == P_DF64 ? 400000 : prec == P_F64 ? 36000 : prec != P_F32 ? 0 : compressed ? 24576 : 85000;
+    return g.Vh > most ? 0 : g.Vh <= 16384 ? 8 : 4;
+}
+
+// Links kept in L2 from one launch to the next in a solve (each launch reads
+// every link of both parities): the rest is evicted first, so that the kept
+// ones and the vectors stay.  32 MB of the 129 MB L2 measured best or equal
+// (an iteration of plain CG in double float at 46080 sites per parity 65 ->
+// 58 us, at 80000 93.5 -> 87; of mixed CG in FP32 on 12-real links at 80000
+// 59.9 -> 52.8, 128000: 69 -> 66; 64 MB and more were slower again).  A
+// single Dslash call keeps none (stag_dslash_*: its caller may well be
+// working on several lattices in turn; three of them at 120960 sites on
+// 12-real links: 28.8 against 27.8 us a pair of calls).  The kernels that
+// load with LD_STREAM ignore it.
+int link_keep_sites(int prec, int compressed) {
+    const size_t site = 2 * link_parity_bytes(prec, compressed, 256) / 256;  // both parities' links
+    return (int)((32u << 20) / site);
+}
+
+int dslash_blocks(int prec, int epi, const DslashArgs &a, int block) {
+    if (pair16_used(prec, epi, a, block))
+        return dslash_pair16_grid(a.g, block);
+    const int n = (a.cn ? a.cn : a.g.Vh) + (a.cn ? a.cnb : 0);
+    const int sites = split_warps(prec, a.compressed, a.g) > 0 ? SPLIT_SITES : block;
+    return (n + sites - 1) / sites;
+}
 
 cudaError_t launch_dslash(int prec, int epi, const DslashArgs &a, int block, cudaStream_t s) {
     if (block <= 0)

@@ -282,8 +282,8 @@ extern "C" int stag_ddr_create(stag_lattice lat, const stag_comm *comm, stag_ddr
         e = cudaMalloc(&d->sc, sizeof(CgScalars));
     if (e == cudaSuccess)
         e = cudaMalloc(&d->dd, sizeof(DdScal));
-    if (e == cudaSuccess)  // the split M Dslash: up to three launches of blocks of 64 or more
-        e = cudaMalloc(&d->partial, sizeof(double) * ((size_t)lat->Vh / 64 + 4));
+    if (e == cudaSuccess)  // the M Dslash over the slab's parts: up to three launches
+        e = cudaMalloc(&d->partial, sizeof(double) * (dslash_max_blocks(lat->Vh) + 4));
     if (e == cudaSuccess)
         e = cudaMallocHost(&d->hval, sizeof(double));
     if (e == cudaSuccess)
@@ -370,7 +370,7 @@ static int slab_range(stag_ddr d, int prec, int out_par, int epi, const void *in
     }
     CUDA_TRY(launch_dslash(prec, epi, a, block, lat->stream));
     if (np)
-        *np += (a.cn + a.cnb + block - 1) / block;
+        *np += dslash_blocks(prec, epi, a, block);
     return STAG_OK;
 }
 

@@ -1393,7 +1393,7 @@ static int tune_all(stag_lattice lat, int prec, std::vector<stag_tune_result> &r
                                          : dslash_args(lat, prec, STAG_EVEN, w.t, w.Ap);
                 a.p = w.p;
                 a.regs = regs;
-                if (regs == REGS_PAIR && !pair16_used(prec, EPI_NONE, a))
+                if (regs == REGS_PAIR && !pair16_used(prec, EPI_NONE, a, 64))
                     continue;  // the pair form exists for the compressed 16-bit stencil only
                 const int epi = kind == 0 ? EPI_NONE : EPI_M_PART;
                 double us = 0;

@@ -93,7 +93,7 @@ extern "C" int stag_lattice_create(stag_lattice *out, const int dims[4], const d
             return cleanup(fail(STAG_ERR_CUDA, "cudaStreamCreate: %s", cudaGetErrorString(e)));
         lat->own_stream = true;
     }
-    const int nblk = (int)((Vh + 63) / 64) + 1;
+    const size_t nblk = dslash_max_blocks(Vh) + 1;
     if ((e = cudaMalloc(&lat->partial, sizeof(double) * nblk)) != cudaSuccess ||
         (e = cudaMalloc(&lat->sc, sizeof(CgScalars))) != cudaSuccess ||
         (e = cudaMemset(lat->sc, 0, sizeof(CgScalars))) != cudaSuccess ||
@@ -649,6 +649,7 @@ static int dslash_impl(stag_lattice lat, stag_field out, const stag_field in, in
     STAG_TRY(check_pair(lat, out, in, out_par, who));
     DEVICE_SCOPE(lat->device);
     DslashArgs a = dslash_args(lat, out->prec, out_par, in->data, out->data);
+    a.keep = 0;
     CUDA_TRY(launch_dslash(out->prec, EPI_NONE, a, lat->dslash_block[out->prec], lat->stream));
     return STAG_OK;
 }

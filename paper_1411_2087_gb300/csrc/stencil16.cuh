@@ -173,9 +173,9 @@ STAG_D float ld_vec16(const short2 *__restrict__ v, int j, cplx<float> w[3]) {
 }
 
 // rows 0, 1 of link idx of one kind (12-real 16-bit layout)
-STAG_D void ld_link16(const char *kb, int S, int idx, cplx<float> L[6]) {
-    const int4 a = ld_stream((const int4 *)kb + idx);
-    const int2 b = ld_stream((const int2 *)(kb + (size_t)16 * S) + idx);
+template <int LD> STAG_D void ld_link16(const char *kb, int S, int idx, l2pol pol, cplx<float> L[6]) {
+    const int4 a = ld_link<LD>((const int4 *)kb + idx, pol);
+    const int2 b = ld_link<LD>((const int2 *)(kb + (size_t)16 * S) + idx, pol);
     L[0] = cplx<float>{q_lo(a.x), q_hi(a.x)};
     L[1] = cplx<float>{q_lo(a.y), q_hi(a.y)};
     L[2] = cplx<float>{q_lo(a.z), q_hi(a.z)};
@@ -185,9 +185,9 @@ STAG_D void ld_link16(const char *kb, int S, int idx, cplx<float> L[6]) {
 }
 
 // the nine entries of link idx of one full kind
-STAG_D void ld_link16_full(const char *kb, int S, int idx, cplx<float> L[9]) {
+template <int LD> STAG_D void ld_link16_full(const char *kb, int S, int idx, l2pol pol, cplx<float> L[9]) {
     int w[9];
-    L16::load(kb, (size_t)S, idx, w);
+    L16::load<LD>(kb, (size_t)S, idx, pol, w);
 #pragma unroll
     for (int e = 0; e < 9; e++)
         L[e] = cplx<float>{q_lo(w[e]), q_hi(w[e])};
@@ -199,43 +199,17 @@ STAG_D cplx<float2> q2(int wa, int wb) {
     return cplx<float2>{make_float2(q_lo(wa), q_lo(wb)), make_float2(q_hi(wa), q_hi(wb))};
 }
 
-STAG_D float2 ld_vec16(const short2 *__restrict__ v, int ja, int jb, cplx<float2> w[3]) {
-    const int4 qa = ld_cell16(v, ja), qb = ld_cell16(v, jb);
-    w[0] = q2(qa.x, qb.x);
-    w[1] = q2(qa.y, qb.y);
-    w[2] = q2(qa.z, qb.z);
-    return make_float2(__int_as_float(qa.w), __int_as_float(qb.w));
-}
-
-STAG_D void ld_link16(const char *kb, int S, int ia, int ib, cplx<float2> L[6]) {
-    const int4 a = ld_stream((const int4 *)kb + ia), c = ld_stream((const int4 *)kb + ib);
-    const int2 b = ld_stream((const int2 *)(kb + (size_t)16 * S) + ia);
-    const int2 d = ld_stream((const int2 *)(kb + (size_t)16 * S) + ib);
-    const int wa[6] = {a.x, a.y, a.z, a.w, b.x, b.y}, wb[6] = {c.x, c.y, c.z, c.w, d.x, d.y};
-#pragma unroll
-    for (int e = 0; e < 6; e++)
-        L[e] = cplx<float2>{make_float2(q_lo(wa[e]), q_lo(wb[e])), make_float2(q_hi(wa[e]), q_hi(wb[e]))};
-}
-
-STAG_D void ld_link16_full(const char *kb, int S, int ia, int ib, cplx<float2> L[9]) {
-    int wa[9], wb[9];
-    L16::load(kb, (size_t)S, ia, wa);
-    L16::load(kb, (size_t)S, ib, wb);
-#pragma unroll
-    for (int e = 0; e < 9; e++)
-        L[e] = q2(wa[e], wb[e]);
-}
-
 // ---- the site loops -------------------------------------------------------
 
 // acc += D psi at checkerboard site c of parity par (one site)
-template <int CM, class A>
+template <int CM, int LD, class A>
 STAG_D void stencil16_site(const Geom &g, int par, int c, const void *__restrict__ Gout,
                            const void *__restrict__ Gin, const short2 *__restrict__ in, const A &a,
                            cplx<float> acc[3]) {
     const int S = g.stride;
     int x[4];
     cb_coords(g, c, par, x);
+    const LinkPolicy<LD> pol(a.keep);
 #pragma unroll
     for (int mu = 0; mu < 4; mu++) {
         int esum = 0;
@@ -257,11 +231,11 @@ STAG_D void stencil16_site(const Geom &g, int par, int c, const void *__restrict
                 if (c12) {
                     const int flip = (esum + (a.bc_neg[mu] ? hop_wraps(x[mu], s, g.L[mu]) : 0)) & 1;
                     cplx<float> L[6];
-                    ld_link16(ko, S, c, L);
+                    ld_link16<LD>(ko, S, c, pol.of(c), L);
                     hop_fwd16(acc, L, v, cf, vmul(cf, ls * (flip ? -a.inv_c[h] : a.inv_c[h])));
                 } else {
                     cplx<float> L[9];
-                    ld_link16_full(ko, S, c, L);
+                    ld_link16_full<LD>(ko, S, c, pol.of(c), L);
                     hop_fwd16_full(acc, L, v, cf);
                 }
             }
@@ -272,11 +246,11 @@ STAG_D void stencil16_site(const Geom &g, int par, int c, const void *__restrict
                 if (c12) {
                     const int flip = (esum + (a.bc_neg[mu] ? hop_wraps(x[mu], -s, g.L[mu]) : 0)) & 1;
                     cplx<float> L[6];
-                    ld_link16(ki, S, j, L);
+                    ld_link16<LD>(ki, S, j, pol.of(j), L);
                     hop_bwd16(acc, L, v, cf, ls * (flip ? -a.inv_c[h] : a.inv_c[h]));
                 } else {
                     cplx<float> L[9];
-                    ld_link16_full(ki, S, j, L);
+                    ld_link16_full<LD>(ki, S, j, pol.of(j), L);
                     hop_bwd16_full(acc, L, v, cf);
                 }
             }
@@ -318,16 +292,18 @@ STAG_D void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "mem
 template <int N> STAG_D void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
 
 // cells per slot: 5 when every link is 12-real, 7 when some are full
-template <int CM> __host__ __device__ constexpr int pair16_cells() { return CM == 3 ? 5 : 7; }
+__host__ __device__ constexpr int pair16_cells(int cm) { return cm == 3 ? 5 : 7; }
+template <int CM> __host__ __device__ constexpr int pair16_cells() { return pair16_cells(CM); }
 
 // ring depth: up to three hops in flight per thread while a block's ring
 // stays within 40 KB of shared memory (128-thread blocks: three hops, 30 KB;
 // 256: two), fewer beyond; 0: no pair form for this block size.  At 48^3x96
 // on 12-real links the 128-thread form took 368 us with three hops against
 // 373.5 us with two (four and more measured slower at 768 threads per SM).
-template <int BLOCK, int CM> __host__ __device__ constexpr int pair16_ring() {
-    return 40960 / (pair16_cells<CM>() * 16 * BLOCK) >= 3 ? 3 : 40960 / (pair16_cells<CM>() * 16 * BLOCK);
+__host__ __device__ constexpr int pair16_ring(int block, int cm) {
+    return 40960 / (pair16_cells(cm) * 16 * block) >= 3 ? 3 : 40960 / (pair16_cells(cm) * 16 * block);
 }
+template <int BLOCK, int CM> __host__ __device__ constexpr int pair16_ring() { return pair16_ring(BLOCK, CM); }
 
 // the indices of hop k = 4 mu + 2 h + dir (dir 1: backward) of the pair
 // (c, c + H): neighbour vectors at ja, jb, links at ia, ib of kind 4h + mu
