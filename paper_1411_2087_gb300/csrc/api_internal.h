@@ -134,7 +134,8 @@ struct stag_lattice_s {
     double *staging = nullptr;             // canonical [Vh][3] complex128 for host import/export
     float link_scale[2] = {0.f, 0.f};      // 16-bit links: field max / 32767 (one-link, three-link)
     float *xs = nullptr;                   // F32 correction x_sloppy of the mixed solver
-    unsigned *absmax = nullptr;            // scratch for the 16-bit link scales
+    unsigned *absmax = nullptr;            // scratch of the field checks
+    LinkScan *scan = nullptr;              // scratch of a gauge upload (two fields)
     struct MixedGraph {
         cudaGraphExec_t exec = nullptr;
         cudaGraph_t graph = nullptr;
@@ -202,11 +203,17 @@ static inline const void *links_of(const stag_lattice lat, int prec, int parity)
     return base + (size_t)parity * 8 * 9 * lat->geom.stride * prec_link_elem_bytes(prec);
 }
 
-static inline void free_cg(CgWork &w) {
+static inline void drop_cg_graph(CgWork &w) {
     if (w.exec)
         cudaGraphExecDestroy(w.exec);
     if (w.graph)
         cudaGraphDestroy(w.graph);
+    w.exec = nullptr;
+    w.graph = nullptr;
+}
+
+static inline void free_cg(CgWork &w) {
+    drop_cg_graph(w);
     void *bufs[] = {w.r, w.p, w.Ap, w.t, w.bw, w.xw};
     for (void *b : bufs)
         if (b)
@@ -319,21 +326,29 @@ static inline int m_block(const stag_lattice lat, int prec) {
     return lat->dslash_block[prec] > 0 ? lat->dslash_block[prec] : dslash_default_block(prec);
 }
 
-// lattices up to this many sites per parity sum <p, Ap> in the M Dslash's
-// last block (one launch less per iteration, which is what counts when the
-// launches are short); larger ones write block partials and sum them in a
-// one-block kernel, which lets the Dslash blocks retire without a ticket
+// On lattices up to this many sites per parity the launches are short and
+// counting them is what matters: plain CG leaves its sums to the next kernel
+// (launch_cg_small_vectors), the other solvers sum <p, Ap> in the M Dslash's
+// last block.  Larger ones write block partials and sum them in a one-block
+// kernel, which lets the Dslash blocks retire without a ticket.
 constexpr int kSmallVh = 65536;
 
-// Ap = m^2 p - D_eo t with <p, Ap>, alpha and the breakdown test in sc
-// (skip_if_done: everything returns at once after the solve)
-static inline cudaError_t enqueue_m_pap(stag_lattice lat, int prec, const void *t, void *Ap, const void *p,
-                                        bool skip_if_done, cudaStream_t s, const int *gate = nullptr) {
+// the M Dslash Ap = m^2 p - D_eo t of an iteration (skip_if_done: it returns
+// at once after the solve)
+static inline DslashArgs m_part_args(stag_lattice lat, int prec, const void *t, void *Ap, const void *p,
+                                     bool skip_if_done) {
     DslashArgs a = dslash_args(lat, prec, STAG_EVEN, t, Ap);
     a.p = p;
     a.skip_if_done = skip_if_done;
-    a.gate = gate;
     a.regs = lat->mdslash_block[prec] > 0 ? lat->mdslash_regs[prec] : lat->dslash_regs[prec];
+    return a;
+}
+
+// Ap = m^2 p - D_eo t with <p, Ap>, alpha and the breakdown test in sc
+static inline cudaError_t enqueue_m_pap(stag_lattice lat, int prec, const void *t, void *Ap, const void *p,
+                                        bool skip_if_done, cudaStream_t s, const int *gate = nullptr) {
+    DslashArgs a = m_part_args(lat, prec, t, Ap, p, skip_if_done);
+    a.gate = gate;
     const int block = m_block(lat, prec);
     if (lat->geom.Vh <= kSmallVh)
         return launch_dslash(prec, EPI_M_PAP, a, block, s);

@@ -67,6 +67,11 @@ struct CgScalars {
     // mixed multi-shift: this iteration's Dslash pair in the high precision
     // (hi_op) or the low one (lo_op = !hi_op), the gates of the two paths
     int ms_hi_op, ms_lo_op;
+    // plain CG on small lattices (cg_small_update_kernel): what the update
+    // kernel hands to the direction kernel, which writes rr, iter, status
+    double up_rr;    // |r_k|^2
+    int up_iter;     // k
+    int up_status;
 };
 
 // multi-shift CG

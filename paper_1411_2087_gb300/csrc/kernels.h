@@ -30,6 +30,10 @@ cudaError_t launch_cg_update(int prec, const Geom &g, void *x, void *r, const vo
                              const void *Ap, double *partial, CgScalars *sc, cudaStream_t s);
 cudaError_t launch_cg_p_update(int prec, const Geom &g, const void *r, void *p,
                                const CgScalars *sc, cudaStream_t s);
+// x, r and p of one iteration of plain CG on a small lattice, with alpha from
+// the M Dslash's npap partials at `partial` (room for Vh / 128 more behind)
+cudaError_t launch_cg_small_vectors(int prec, const Geom &g, void *x, void *r, void *p, const void *Ap,
+                                    double *partial, int npap, CgScalars *sc, cudaStream_t s);
 // <p, M p> from the n block partials of a Dslash with EPI_M_PART, summed in
 // block order; then alpha = |r|^2 / <p, M p> and the breakdown test (as the
 // EPI_M_PAP epilogue).  Returns at once when skip_if_done and the solve has
@@ -43,24 +47,32 @@ cudaError_t launch_import(int prec, const Geom &g, const double *canon, void *fi
 cudaError_t launch_export(int prec, const Geom &g, const void *field, double *canon, cudaStream_t s);
 
 // fold c1/c3, Kogut-Susskind phases and boundary signs into the canonical
-// fat/long links (device, complex128 [4][V][3][3]) and lay them out per parity
-// (inv_scale: 16-bit links only, 32767 / largest |entry| of the folded
-// one-link and three-link fields; ignored otherwise)
-cudaError_t launch_fold_links(int prec, const Geom &g, const double bc[4], double c1, double c3,
-                              const double *fat, const double *lng, void *links,
-                              const float inv_scale[2], cudaStream_t s);
+// fat/long links (device, complex128 [4][V][3][3]) and write every copy with
+// a buffer in `out`: full kinds by precision, and the copies (FP32, 16-bit)
+// whose kinds of the groups in `mask` are 12-real (see C12 in fields.cuh)
+// (inv_scale: 16-bit links, 32767 / largest |entry| of the folded one-link
+// and three-link fields)
+struct FoldOut {
+    void *full[4];
+    void *c12[4];
+    int mask;
+};
+cudaError_t launch_fold_links(const Geom &g, const double bc[4], double c1, double c3, const double *fat,
+                              const double *lng, const FoldOut &out, const float inv_scale[2], cudaStream_t s);
 
-// fold into the 12-real layout (FP32 or 16-bit; see C12 in fields.cuh)
-cudaError_t launch_fold_links_c12(int prec, const Geom &g, const double bc[4], double c1, double c3,
-                                  const double *fat, const double *lng, void *links, const float inv_scale[2],
-                                  int mask, cudaStream_t s);
-// largest deviation from SU(3) over nlinks canonical 3x3 complex128
-// matrices, as float bits in *out (device)
-cudaError_t launch_su3_deviation(const double *U, long long nlinks, unsigned *out, cudaStream_t s);
-
-// largest |re| / |im| over n doubles, as float bits in *out (device); a
-// NaN, an infinity or a value beyond the FP32 range gives +infinity
-cudaError_t launch_absmax(const double *a, long long n, unsigned *out, cudaStream_t s);
+// one pass over one or two fields of nlinks canonical 3x3 complex128
+// matrices (device; f1 may be NULL), into out[0..1] (device)
+struct LinkScan {
+    unsigned long long maxbits;  // largest |re| or |im|, the double's bits
+    unsigned dev;                // largest deviation from SU(3) (with su3), the float's bits
+    unsigned pad;
+};
+cudaError_t launch_scan_links(const double *f0, const double *f1, long long nlinks, bool su3, LinkScan *out,
+                              cudaStream_t s);
+// of a scan copied to the host: the largest |entry| (infinite if the field
+// holds a NaN, an infinity or a value beyond the FP32 range), the deviation
+float scan_absmax(const LinkScan &s);
+float scan_su3_deviation(const LinkScan &s);
 
 // *flag = 1 if a finite entry of n doubles lies beyond the FP32 range (device)
 cudaError_t launch_finite_overflow(const double *a, long long n, unsigned *flag, cudaStream_t s);

@@ -135,16 +135,16 @@ extern "C" int stag_net_create(stag_lattice lat, const double *fat, int ptr_kind
         }
     }
     // the 16-bit copy's scale: the largest |re| or |im| of the field
-    unsigned *amax_d = (unsigned *)(n->scal + 3);
-    e = launch_absmax(fat_d, (long long)(4 * V * 18), amax_d, s);
-    float amax = 0.f;
-    if (e == cudaSuccess) {
-        unsigned bits = 0;
-        e = cudaMemcpyAsync(&bits, amax_d, sizeof bits, cudaMemcpyDeviceToHost, s);
-        if (e == cudaSuccess)
-            e = cudaStreamSynchronize(s);
-        memcpy(&amax, &bits, sizeof amax);
-    }
+    // (and whether they are special unitary, below)
+    LinkScan *scan_d = (LinkScan *)n->scal;
+    static_assert(sizeof(LinkScan) <= 4 * sizeof(double), "scan scratch");
+    LinkScan scan = {};
+    e = launch_scan_links(fat_d, nullptr, (long long)(4 * V), true, scan_d, s);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(&scan, scan_d, sizeof scan, cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess)
+        e = cudaStreamSynchronize(s);
+    const float amax = scan_absmax(scan);
     if (e == cudaSuccess && !(amax < INFINITY)) {
         if (owned)
             cudaFree(fat_d);
@@ -161,22 +161,12 @@ extern "C" int stag_net_create(stag_lattice lat, const double *fat, int ptr_kind
     // special unitary fat links (within 1e-6): the solver's 16-bit net links
     // keep rows 0 and 1 only and the kernels rebuild row 2 (two thirds of
     // the link bytes of the net's two stencil passes)
-    if (e == cudaSuccess)
-        e = launch_su3_deviation(fat_d, (long long)(4 * V), amax_d, s);
-    if (e == cudaSuccess) {
-        unsigned bits = 0;
-        e = cudaMemcpyAsync(&bits, amax_d, sizeof bits, cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess && scan_su3_deviation(scan) <= 1e-6f) {
+        e = cudaMalloc(&n->NL12, net_links12_bytes(lat->geom));
         if (e == cudaSuccess)
-            e = cudaStreamSynchronize(s);
-        float dev = 1.f;
-        memcpy(&dev, &bits, sizeof dev);
-        if (e == cudaSuccess && dev <= 1e-6f) {
-            e = cudaMalloc(&n->NL12, net_links12_bytes(lat->geom));
-            if (e == cudaSuccess)
-                e = cudaMemsetAsync(n->NL12, 0, net_links12_bytes(lat->geom), s);
-            if (e == cudaSuccess)
-                e = launch_net_links12(lat->geom, lat->bc, fat_d, n->NL12, amax > 0.f ? kQ16 / amax : 0.f, s);
-        }
+            e = cudaMemsetAsync(n->NL12, 0, net_links12_bytes(lat->geom), s);
+        if (e == cudaSuccess)
+            e = launch_net_links12(lat->geom, lat->bc, fat_d, n->NL12, amax > 0.f ? kQ16 / amax : 0.f, s);
     }
     cudaError_t e2 = cudaStreamSynchronize(s);
     if (owned)

@@ -93,7 +93,7 @@ extern "C" int stag_lattice_create(stag_lattice *out, const int dims[4], const d
             return cleanup(fail(STAG_ERR_CUDA, "cudaStreamCreate: %s", cudaGetErrorString(e)));
         lat->own_stream = true;
     }
-    const size_t nblk = dslash_max_blocks(Vh) + 1;
+    const size_t nblk = dslash_max_blocks(Vh) + (size_t)(Vh + 127) / 128 + 1;
     if ((e = cudaMalloc(&lat->partial, sizeof(double) * nblk)) != cudaSuccess ||
         (e = cudaMalloc(&lat->sc, sizeof(CgScalars))) != cudaSuccess ||
         (e = cudaMemset(lat->sc, 0, sizeof(CgScalars))) != cudaSuccess ||
@@ -162,6 +162,8 @@ extern "C" int stag_lattice_destroy(stag_lattice lat) {
         cudaFree(lat->ms_blo);
     if (lat->absmax)
         cudaFree(lat->absmax);
+    if (lat->scan)
+        cudaFree(lat->scan);
     for (int h = 0; h < 4; h++)
         for (int l = 0; l < 4; l++) {
             if (lat->mixed[h][l].exec)
@@ -209,6 +211,26 @@ extern "C" int stag_lattice_set_cg_launch(stag_lattice lat, int mode, int chunk)
 // --------------------------------------------------------------------------
 // gauge upload
 // --------------------------------------------------------------------------
+
+// free the link copies that an upload of precisions prec_mask with
+// compression mask cmask does not write (0, 0: all), and the solver
+// workspaces of the precisions it leaves out
+static void drop_links(stag_lattice lat, unsigned prec_mask, int cmask) {
+    for (int p = 0; p < 4; p++) {
+        const bool want = (prec_mask >> p) & 1u;
+        if (!want)
+            free_cg(lat->cg[p]);
+        if (lat->links[p] && !want) {
+            cudaFree(lat->links[p]);
+            lat->links[p] = nullptr;
+        }
+        if (lat->links_c12[p] && (!want || lat->c12_mask[p] != cmask)) {
+            cudaFree(lat->links_c12[p]);
+            lat->links_c12[p] = nullptr;
+            lat->c12_mask[p] = 0;
+        }
+    }
+}
 
 // device copy of a canonical gauge field: returns a device pointer, allocating
 // a temporary when the source is on the host
@@ -289,118 +311,92 @@ extern "C" int stag_gauge_upload(stag_lattice lat, const double *fat, const doub
         release();
         return st;
     }
-    // drop old copies and solver graphs; until the new copies exist the
-    // lattice has no gauge field
+    // until the new copies exist the lattice has no gauge field; the solvers'
+    // graphs hold the old link scales and coefficients
     cudaStreamSynchronize(lat->stream);
     lat->has_gauge = false;
-    for (int p = 0; p < 4; p++) {
-        free_cg(lat->cg[p]);
-        if (lat->links[p]) {
-            cudaFree(lat->links[p]);
-            lat->links[p] = nullptr;
-        }
-        if (lat->links_c12[p]) {
-            cudaFree(lat->links_c12[p]);
-            lat->links_c12[p] = nullptr;
-        }
-        lat->c12_mask[p] = 0;
-    }
+    for (int p = 0; p < 4; p++)
+        drop_cg_graph(lat->cg[p]);
     drop_mixed_graphs(lat);
-    if (compress) {
-        // the 12-real form rebuilds row 3 from rows 1 and 2: only valid for
-        // links in SU(3) (the paper's Sec. 4 notes smeared links are not)
-        unsigned *dev_bits = nullptr;
-        cudaError_t e = cudaMalloc(&dev_bits, 2 * sizeof(unsigned));
-        if (e == cudaSuccess)
-            e = launch_su3_deviation(fat_d, 4LL * lat->V, dev_bits, lat->stream);
-        if (e == cudaSuccess)
-            e = launch_su3_deviation(lng_d, 4LL * lat->V, dev_bits + 1, lat->stream);
-        unsigned bits[2] = {0u, 0u};
-        if (e == cudaSuccess)
-            e = cudaMemcpyAsync(bits, dev_bits, sizeof bits, cudaMemcpyDeviceToHost, lat->stream);
-        if (e == cudaSuccess)
-            e = cudaStreamSynchronize(lat->stream);
-        if (dev_bits)
-            cudaFree(dev_bits);
-        if (e != cudaSuccess) {
-            release();
-            return fail(STAG_ERR_CUDA, "SU(3) check: %s", cudaGetErrorString(e));
-        }
-        float dev[2];
-        memcpy(dev, bits, sizeof dev);
-        if (((cmask & 1) && !(dev[0] <= 1e-6f)) || !(dev[1] <= 1e-6f)) {
-            release();
-            return fail(STAG_ERR_ARG, "stag_gauge_upload: links deviate from SU(3) by %.2e (fat) / %.2e (long); "
-                        "12-real compression needs special unitary links%s", dev[0], dev[1],
-                        (cmask & 1) ? " (STAG_COMPRESS12_LONG compresses the long links only)" : "");
-        }
-    }
-    lat->has_gauge = false;
+    auto refuse = [&](int code) {  // no copy survives a refused upload
+        release();
+        drop_links(lat, 0, 0);
+        return code;
+    };
+    // one pass over both fields: the largest |entry| of each rejects
+    // non-finite links and is the scale of the 16-bit copy (one per field,
+    // after folding); the 12-real form rebuilds row 3 from rows 1 and 2, only
+    // valid for links in SU(3) (the paper's Sec. 4 notes smeared links are not)
     float inv_scale[2] = {0.f, 0.f};
     {
-        // largest |entry| of each field: rejects non-finite links, and is the
-        // scale of the 16-bit copy (one per field, after folding)
-        cudaError_t e = lat->absmax ? cudaSuccess : cudaMalloc(&lat->absmax, 2 * sizeof(unsigned));
-        const long long n = 4LL * lat->V * 18;
+        cudaError_t e = lat->scan ? cudaSuccess : cudaMalloc(&lat->scan, 2 * sizeof(LinkScan));
+        LinkScan scan[2] = {};
         if (e == cudaSuccess)
-            e = launch_absmax(fat_d, n, lat->absmax, lat->stream);
+            e = launch_scan_links(fat_d, lng_d, 4LL * lat->V, compress, lat->scan, lat->stream);
         if (e == cudaSuccess)
-            e = launch_absmax(lng_d, n, lat->absmax + 1, lat->stream);
-        unsigned bits[2] = {0u, 0u};
-        if (e == cudaSuccess)
-            e = cudaMemcpyAsync(bits, lat->absmax, sizeof bits, cudaMemcpyDeviceToHost, lat->stream);
+            e = cudaMemcpyAsync(scan, lat->scan, sizeof scan, cudaMemcpyDeviceToHost, lat->stream);
         if (e == cudaSuccess)
             e = cudaStreamSynchronize(lat->stream);
-        if (e != cudaSuccess) {
-            release();
-            return fail(STAG_ERR_CUDA, "16-bit link scales: %s", cudaGetErrorString(e));
-        }
+        if (e != cudaSuccess)
+            return refuse(fail(STAG_ERR_CUDA, "gauge scan: %s", cudaGetErrorString(e)));
         const double cf[2] = {std::fabs(c1), std::fabs(c3)};
         for (int h = 0; h < 2; h++) {
-            float m;
-            memcpy(&m, &bits[h], sizeof m);
-            if (!std::isfinite(m)) {
-                release();
-                return fail(STAG_ERR_ARG, "stag_gauge_upload: the %s links hold NaN, infinite or out-of-range "
-                            "entries", h ? "long" : "fat");
-            }
+            const float m = scan_absmax(scan[h]);
+            if (!std::isfinite(m))
+                return refuse(fail(STAG_ERR_ARG, "stag_gauge_upload: the %s links hold NaN, infinite or "
+                                   "out-of-range entries", h ? "long" : "fat"));
             if ((prec_mask >> STAG_F16) & 1u) {
                 const double mx = (double)m * cf[h];
                 lat->link_scale[h] = mx > 0 ? (float)(mx / 32767.0) : 0.f;
                 inv_scale[h] = mx > 0 ? (float)(32767.0 / mx) : 0.f;
             }
         }
+        const float dev[2] = {scan_su3_deviation(scan[0]), scan_su3_deviation(scan[1])};
+        if (compress && (((cmask & 1) && !(dev[0] <= 1e-6f)) || !(dev[1] <= 1e-6f)))
+            return refuse(fail(STAG_ERR_ARG, "stag_gauge_upload: links deviate from SU(3) by %.2e (fat) / %.2e "
+                               "(long); 12-real compression needs special unitary links%s", dev[0], dev[1],
+                               (cmask & 1) ? " (STAG_COMPRESS12_LONG compresses the long links only)" : ""));
     }
+    // the copies of the last upload keep their buffers where this one has
+    // the same (allocating 24^3x48 in DF64, FP32 and 16-bit anew took 1.5 ms)
+    drop_links(lat, prec_mask, cmask);
+    FoldOut out;
+    memset(&out, 0, sizeof out);
+    out.mask = cmask;
     for (int p = 0; p < 4; p++) {
         if (!((prec_mask >> p) & 1u))
             continue;
-        cudaError_t e = cudaMalloc(&lat->links[p], link_bytes(lat, p));
-        if (e == cudaSuccess)
-            e = cudaMemsetAsync(lat->links[p], 0, link_bytes(lat, p), lat->stream);
-        if (e == cudaSuccess)
-            e = launch_fold_links(p, lat->geom, lat->bc, c1, c3, fat_d, lng_d, lat->links[p], inv_scale,
-                                  lat->stream);
+        cudaError_t e = cudaSuccess;
+        // the padding sites of new buffers are zero; the fold writes the others
+        if (!lat->links[p]) {
+            e = cudaMalloc(&lat->links[p], link_bytes(lat, p));
+            if (e == cudaSuccess)
+                e = cudaMemsetAsync(lat->links[p], 0, link_bytes(lat, p), lat->stream);
+        }
+        out.full[p] = lat->links[p];
         if (e == cudaSuccess && compress && (p == STAG_F32 || p == STAG_F16)) {
-            const size_t cb = c12_link_bytes(p, (size_t)lat->geom.stride, cmask);
-            e = cudaMalloc(&lat->links_c12[p], cb);
-            if (e == cudaSuccess)
-                e = cudaMemsetAsync(lat->links_c12[p], 0, cb, lat->stream);
-            if (e == cudaSuccess)
-                e = launch_fold_links_c12(p, lat->geom, lat->bc, c1, c3, fat_d, lng_d, lat->links_c12[p],
-                                          inv_scale, cmask, lat->stream);
-            if (e == cudaSuccess)
-                lat->c12_mask[p] = cmask;
+            if (!lat->links_c12[p]) {
+                const size_t cb = c12_link_bytes(p, (size_t)lat->geom.stride, cmask);
+                e = cudaMalloc(&lat->links_c12[p], cb);
+                if (e == cudaSuccess)
+                    e = cudaMemsetAsync(lat->links_c12[p], 0, cb, lat->stream);
+            }
+            lat->c12_mask[p] = cmask;
+            out.c12[p] = lat->links_c12[p];
         }
-        if (e != cudaSuccess) {
-            release();
-            return fail(e == cudaErrorMemoryAllocation ? STAG_ERR_NOMEM : STAG_ERR_CUDA,
-                        "gauge fold (%s): %s", prec_name(p), cudaGetErrorString(e));
-        }
+        if (e != cudaSuccess)
+            return refuse(fail(e == cudaErrorMemoryAllocation ? STAG_ERR_NOMEM : STAG_ERR_CUDA,
+                               "gauge copy (%s): %s", prec_name(p), cudaGetErrorString(e)));
+    }
+    {
+        const cudaError_t e = launch_fold_links(lat->geom, lat->bc, c1, c3, fat_d, lng_d, out, inv_scale, lat->stream);
+        if (e != cudaSuccess)
+            return refuse(fail(STAG_ERR_CUDA, "gauge fold: %s", cudaGetErrorString(e)));
     }
     cudaError_t e = cudaStreamSynchronize(lat->stream);
-    release();
     if (e != cudaSuccess)
-        return fail(STAG_ERR_CUDA, "stag_gauge_upload: %s", cudaGetErrorString(e));
+        return refuse(fail(STAG_ERR_CUDA, "stag_gauge_upload: %s", cudaGetErrorString(e)));
+    release();
     lat->has_gauge = true;
     lat->c1 = c1;
     lat->c3 = c3;
@@ -708,6 +704,15 @@ cudaError_t enqueue_cg_body(stag_lattice lat, CgWork &w, cudaStream_t s, bool sk
     a1.skip_if_done = skip_if_done;
     if ((e = launch_dslash(prec, EPI_NONE, a1, lat->dslash_block[prec], s)) != cudaSuccess)
         return e;
+    if (lat->geom.Vh <= kSmallVh) {
+        // the vector kernels sum the partials of <p, Ap> themselves
+        DslashArgs a2 = m_part_args(lat, prec, w.t, w.Ap, w.p, skip_if_done);
+        const int block = m_block(lat, prec);
+        if ((e = launch_dslash(prec, EPI_M_PART, a2, block, s)) != cudaSuccess)
+            return e;
+        return launch_cg_small_vectors(prec, lat->geom, w.xw, w.r, w.p, w.Ap, lat->partial,
+                                       dslash_blocks(prec, EPI_M_PART, a2, block), lat->sc, s);
+    }
     // Ap = M p with one partial of <p, Ap> per block; a one-block kernel sums
     // them (cheaper at these grid sizes than a last-block ticket in the Dslash)
     if ((e = enqueue_m_pap(lat, prec, w.t, w.Ap, w.p, skip_if_done, s)) != cudaSuccess)
