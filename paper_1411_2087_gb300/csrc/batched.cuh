@@ -47,6 +47,7 @@ struct BatchArgs {
     int kmax;     // the largest group: selects the kernels' K
     int nblocks;  // total blocks of the grouped launch
     int dnblocks; // total blocks of a lane-mapped Dslash launch
+    int split;    // the lane-mapped Dslash in split form (32 (site, system) items per block)
     BatchGroup grp[BATCH_MAX_G];
     CgScalars *sys;    // one per system
     unsigned *tickets; // one per group
@@ -101,14 +102,10 @@ STAG_D bool group_sum(const T (&v)[K], int Kact, double *partial, int lblk, int 
     if (!last)
         return false;
     __threadfence();
-    const volatile double *vp = partial;
 #pragma unroll
     for (int k = 0; k < K; k++) {
         if (k < Kact) {
-            double acc = 0.0;
-            for (int i = threadIdx.x; i < nblk; i += BLOCK)
-                acc += vp[(size_t)i * K + k];
-            acc = block_sum<BLOCK>(acc, smem);
+            const double acc = block_sum<BLOCK>(partials_share<BLOCK>(partial + k, nblk, K), smem);
             if (threadIdx.x == 0)
                 res[k] = acc;
         }
@@ -119,6 +116,62 @@ STAG_D bool group_sum(const T (&v)[K], int Kact, double *partial, int lblk, int 
 #pragma unroll
     for (int k = 0; k < K; k++)
         tot[k] = k < Kact ? res[k] : 0.0;
+    __syncthreads();
+    return true;
+}
+
+// The same sums when each thread holds the value of one system: thread t <
+// ITEMS of block lblk that of system (lblk ITEMS + t) % Kact, and threads
+// t + ITEMS, t + 2 ITEMS further shares of the same (ROWS in all).  One pass
+// through shared memory, warp k sums system k's threads (in thread order,
+// then the warp tree).
+template <int BLOCK, int K, int ITEMS, int ROWS, class T>
+STAG_D bool group_sum_lanes(T v, int Kact, double *partial, int lblk, int nblk, unsigned *ticket,
+                            double *smem, double (&tot)[K]) {
+    static_assert(K <= BLOCK / 32, "a warp per system");
+    __shared__ bool last;
+    __shared__ double res[K];
+    __shared__ T all[BLOCK];
+    all[threadIdx.x] = v;
+    __syncthreads();
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (w < Kact) {
+        const int first = (w - (int)((lblk * (long long)ITEMS) % Kact) + Kact) % Kact;
+        T s = red_zero<T>();
+        for (int t = first + lane * Kact; t < ITEMS; t += 32 * Kact)
+#pragma unroll
+            for (int q = 0; q < ROWS; q++)
+                s = red_add(s, all[q * ITEMS + t]);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+            s = red_add(s, shfl_down(s, o));
+        if (lane == 0)
+            partial[(size_t)lblk * K + w] = red_to_double(s);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        const unsigned t = atomicAdd(ticket, 1u);
+        last = (t == (unsigned)nblk - 1);
+    }
+    __syncthreads();
+    if (!last)
+        return false;
+    __threadfence();
+#pragma unroll
+    for (int q = 0; q < K; q++) {
+        if (q < Kact) {
+            const double acc = block_sum<BLOCK>(partials_share<BLOCK>(partial + q, nblk, K), smem);
+            if (threadIdx.x == 0)
+                res[q] = acc;
+        }
+    }
+    if (threadIdx.x == 0)
+        *ticket = 0u;
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < K; q++)
+        tot[q] = q < Kact ? res[q] : 0.0;
     __syncthreads();
     return true;
 }

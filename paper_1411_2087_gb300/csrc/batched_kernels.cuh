@@ -2,6 +2,7 @@
 // instantiated per precision in batched_<prec>.cu.
 #pragma once
 #include "batched.cuh"
+#include "dslash_split.cuh"
 #include "kernels.h"
 
 namespace stag {
@@ -203,12 +204,12 @@ STAG_D red_t<typename Fmt<P>::R> batch_lane_epilogue(const BatchArgs &a, const B
 
 // the group's sums of a lane-mapped Dslash and what its last block makes of
 // them: alpha_k (EPI_M_PAP) or the true residual (EPI_RESID)
-template <int EPI, int BLOCK, int K, class T>
+template <int EPI, int BLOCK, int K, int ITEMS, int ROWS, class T>
 STAG_D void batch_lane_reduce(const BatchArgs &a, int gi, const BatchGroup &G, const int *act, int lblk,
-                              const T (&dot)[K], double *smem) {
+                              T dot, double *smem) {
     if (EPI == EPI_M_PAP || EPI == EPI_RESID) {
         double tot[K];
-        if (group_sum<BLOCK, K>(dot, G.K, G.partial, lblk, G.dnblocks, &a.tickets[gi], smem, tot) &&
+        if (group_sum_lanes<BLOCK, K, ITEMS, ROWS>(dot, G.K, G.partial, lblk, G.dnblocks, &a.tickets[gi], smem, tot) &&
             threadIdx.x == 0) {
             for (int kk = 0; kk < G.K; kk++) {
                 if (!act[kk])
@@ -237,8 +238,16 @@ STAG_D const void *batch_lane_input(const BatchGroup &G, int k, int src_x) {
 // Lane-mapped multi-RHS Dslash (double-float and FP64): thread t of the
 // group's range handles site t / GK for system t % GK (GK = systems in the
 // group), with the single-site stencil; epilogues as batch_dslash_kernel.
+// Bound by the FMA pipe in double-float (4 x 576 multiply-adds of 12 FP32
+// operations per site).  The hops of one direction are unrolled and the four
+// directions a loop: all sixteen unrolled are 110 KB of code, which the warps
+// of an SM, each elsewhere in it, fetch again and again.  An iteration of a
+// batched solve of four systems on 24^3x48 in double float: 1083 us unrolled
+// at 640 to 768 resident threads, 1036 at 1024; in steps of eight hops 985,
+// four 918 (at 896 threads; 924 at 768), two 917, one 959.  Two systems on
+// 12x16x20x24: 96, 98, 97, 98, 103, 105.
 template <int P, int EPI, int BLOCK, int K>
-__global__ void __launch_bounds__(BLOCK) batch_dslash_lanes_kernel(BatchArgs a, int out_par, int src_x) {
+__global__ void __launch_bounds__(BLOCK, P == P_DF64 ? 896 / BLOCK : 0) batch_dslash_lanes_kernel(const __grid_constant__ BatchArgs a, int out_par, int src_x) {
     using F = Fmt<P>;
     using R = typename F::R;
     using E = typename F::Elem;
@@ -252,24 +261,68 @@ __global__ void __launch_bounds__(BLOCK) batch_dslash_lanes_kernel(BatchArgs a, 
     const int k = t % G.K;
     const int c = t / G.K;
     const Geom &g = G.g;
-    red_t<R> dot[K];
-#pragma unroll
-    for (int kk = 0; kk < K; kk++)
-        dot[kk] = red_zero<red_t<R>>();
+    red_t<R> dot = red_zero<red_t<R>>();
     if (c < g.Vh && act[k]) {
-        DslashArgs da = {};
-        da.link_scale[0] = G.link_scale[0];
-        da.link_scale[1] = G.link_scale[1];
+        int x[4];
+        cb_coords(g, c, out_par, x);
         cplx<R> acc[3] = {czero<R>(), czero<R>(), czero<R>()};
-        dslash_site<P, 0, LD_STREAM>(g, out_par, c, G.links[out_par], G.links[1 - out_par],
-                              (const E *)batch_lane_input<EPI>(G, k, src_x), da, acc);
-        const red_t<R> dk = batch_lane_epilogue<P, EPI>(a, G, k, c, acc);
-#pragma unroll
-        for (int kk = 0; kk < K; kk++)
-            if (kk == k)
-                dot[kk] = dk;
+        const void *Gout = G.links[out_par], *Gin = G.links[1 - out_par];
+        const E *in = (const E *)batch_lane_input<EPI>(G, k, src_x);
+#pragma unroll 4
+        for (int hop = 0; hop < 16; hop++)
+            stencil_hop<P, 0, LD_STREAM>(g, Gout, Gin, in, 0, 0, c, x, hop >> 2, (hop >> 1) & 1, hop & 1, acc);
+        dot = batch_lane_epilogue<P, EPI>(a, G, k, c, acc);
     }
-    batch_lane_reduce<EPI, BLOCK, K>(a, gi, G, act, lblk, dot, smem);
+    batch_lane_reduce<EPI, BLOCK, K, BLOCK, 1>(a, gi, G, act, lblk, dot, smem);
+}
+
+// The lane-mapped Dslash in split form (dslash_split.cuh) for batches too
+// small to fill the chip with one thread per (site, system): 32 items per
+// block, the hops spread over its four warps.
+template <int P, int EPI, int K>
+__global__ void __launch_bounds__(128, 7) batch_dslash_split_kernel(const __grid_constant__ BatchArgs a, int out_par,
+                                                                    int src_x) {
+    using F = Fmt<P>;
+    using R = typename F::R;
+    using E = typename F::Elem;
+    constexpr int NG = 4, BLOCK = 32 * NG;
+    __shared__ double smem[32];
+    __shared__ int act[K];
+    __shared__ E part[NG][3][SPLIT_SITES];
+    const int gi = group_of_lanes(a, blockIdx.x);
+    const BatchGroup &G = a.grp[gi];
+    load_active<K>(a, G, act, EPI != EPI_RESID && !src_x);
+    const int lblk = blockIdx.x - G.dblock0, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int t = lblk * SPLIT_SITES + lane;
+    const int k = t % G.K;
+    const int c = t / G.K;
+    const Geom &g = G.g;
+    const bool on = c < g.Vh && act[k];
+    if (on) {
+        int x[4];
+        cb_coords(g, c, out_par, x);
+        cplx<R> acc[3] = {czero<R>(), czero<R>(), czero<R>()};
+        const E *in = (const E *)batch_lane_input<EPI>(G, k, src_x);
+#pragma unroll 1
+        for (int q = 0; q < 16 / NG; q++) {
+            const int hop = w * (16 / NG) + q;
+            stencil_hop<P, 0, LD_STREAM>(g, G.links[out_par], G.links[1 - out_par], in, 0, 0, c, x, hop >> 2,
+                                         (hop >> 1) & 1, hop & 1, acc);
+        }
+#pragma unroll
+        for (int r = 0; r < 3; r++)
+            part[w][r][lane] = F::pack(acc[r]);
+    }
+    __syncthreads();
+    red_t<R> dot = red_zero<red_t<R>>();
+    if (w < 3 && on) {
+        const cplx<R> o = split_sum<P, NG>(part, w, lane);
+        const R m2 = EPI == EPI_NONE ? rzero<R>() : scalar_as<R>(a.sys[G.sys0 + k].m2);
+        dot = split_epilogue<P, EPI>((E *)(EPI == EPI_NONE ? G.t[k] : G.Ap[k]),
+                                     (const E *)(EPI == EPI_RESID ? G.x[k] : G.p[k]), (const E *)G.b[k], m2,
+                                     w * g.stride + c, o);
+    }
+    batch_lane_reduce<EPI, BLOCK, K, SPLIT_SITES, 3>(a, gi, G, act, lblk, dot, smem);
 }
 
 // x = 0, r = b, p = b, |b|^2 per system
@@ -448,6 +501,15 @@ cudaError_t launch_batch_pbk(int what, const BatchArgs &a, cudaStream_t s) {
     const int grid = a.nblocks;
     if constexpr (P != P_F32) {
         const int dgrid = a.dnblocks;
+        if (a.split) {
+            switch (what) {
+            case BATCH_DSLASH_OE: batch_dslash_split_kernel<P, EPI_NONE, K><<<dgrid, 128, 0, s>>>(a, 1, 0); return cudaGetLastError();
+            case BATCH_DSLASH_X: batch_dslash_split_kernel<P, EPI_NONE, K><<<dgrid, 128, 0, s>>>(a, 1, 1); return cudaGetLastError();
+            case BATCH_M_PAP: batch_dslash_split_kernel<P, EPI_M_PAP, K><<<dgrid, 128, 0, s>>>(a, 0, 0); return cudaGetLastError();
+            case BATCH_RESID: batch_dslash_split_kernel<P, EPI_RESID, K><<<dgrid, 128, 0, s>>>(a, 0, 0); return cudaGetLastError();
+            default: break;
+            }
+        }
         switch (what) {
         case BATCH_DSLASH_OE: batch_dslash_lanes_kernel<P, EPI_NONE, BLOCK, K><<<dgrid, BLOCK, 0, s>>>(a, 1, 0); return cudaGetLastError();
         case BATCH_DSLASH_X: batch_dslash_lanes_kernel<P, EPI_NONE, BLOCK, K><<<dgrid, BLOCK, 0, s>>>(a, 1, 1); return cudaGetLastError();

@@ -366,10 +366,20 @@ __global__ void __launch_bounds__(BLOCK, (kCapThreads<P, CM> + BLOCK - 1) / BLOC
     dslash_body<P, EPI, BLOCK, CM>(a);
 }
 
+// The pair form is the default on 12-real links from here on: Dslash, M with
+// partials at 221184 sites 20.7, 22.8 us against 24.8, 26.9 one site per
+// thread, 1048576: 79, 85 against 93, 99, 48^3x96: 363, 385 against 430,
+// 450; equal at 128000, slower below (32768: 8.4, 9.7 against 6.8, 8.2).
+// On full and three-link-only links it gains nothing (1048576: 98, 85
+// against 92, 84).
+constexpr int PAIR16_MIN_SITES = 150000;
+
 // whether a launch of precision prec, epilogue epi and block size block
 // runs the pair form
 STAG_HD bool pair16_used(int prec, int epi, const DslashArgs &a, int block) {
-    return prec == P_F16 && a.regs == REGS_PAIR && pair16_ring(block, a.compressed) > 0 &&
+    const bool wanted = a.regs == REGS_PAIR ||
+                        (a.regs == REGS_DEFAULT && a.compressed == 3 && a.g.Vh >= PAIR16_MIN_SITES);
+    return prec == P_F16 && wanted && pair16_ring(block, a.compressed) > 0 &&
            (epi == EPI_NONE || epi == EPI_M_PART) &&
            a.c0 == 0 && (a.cn == 0 || a.cn == a.g.Vh) && a.cnb == 0 && pair16_applies(a.g);
 }

@@ -21,14 +21,15 @@ namespace stag {
 
 constexpr int SPLIT_SITES = 32;  // output sites per block, one per lane
 
-// acc += one hop of the stencil at site c (coordinates x): direction mu,
-// h = 0 one-link, 1 three-link, dir = 0 forward, 1 backward (warp-uniform)
-template <int P, int CM>
-STAG_D void split_hop(const DslashArgs &a, int c, const int x[4], int mu, int h, int dir,
-                      cplx<typename Fmt<P>::R> acc[3]) {
+// acc += one hop of the stencil at site c (coordinates x) of the parity of
+// Gout: direction mu, h = 0 one-link, 1 three-link, dir = 0 forward, 1
+// backward, all three known at run time only (warp-uniform).  q carries the
+// 12-real links' constants (DslashArgs; not read on full links).
+template <int P, int CM, int LD, class Q>
+STAG_D void stencil_hop(const Geom &g, const void *__restrict__ Gout, const void *__restrict__ Gin,
+                        const typename Fmt<P>::Elem *__restrict__ in, const Q &q, int keep, int c, const int x[4],
+                        int mu, int h, int dir, cplx<typename Fmt<P>::R> acc[3]) {
     using R = typename Fmt<P>::R;
-    using E = typename Fmt<P>::Elem;
-    const Geom &g = a.g;
     const int S = g.stride;
     const int xm = mu == 0 ? x[0] : mu == 1 ? x[1] : mu == 2 ? x[2] : x[3];
     const int s = h ? 3 : 1, hop = dir ? -s : s, L = g.L[mu];
@@ -41,16 +42,18 @@ STAG_D void split_hop(const DslashArgs &a, int c, const int x[4], int mu, int h,
     }
     const int j = mu == 0 ? c + (((x[0] & 1) + y - xm) >> 1) : c + (y - xm) * g.plane[mu];
     float inv_s = 0.f;
-    if ((CM >> h) & 1) {
-        const int esum = (mu > 0 ? x[0] : 0) + (mu > 1 ? x[1] : 0) + (mu > 2 ? x[2] : 0);
-        const int flip = (esum + (a.bc_neg[mu] ? wraps : 0)) & 1;
-        inv_s = flip ? -a.inv_c[h] : a.inv_c[h];
+    if constexpr (CM != 0) {
+        if ((CM >> h) & 1) {
+            const int esum = (mu > 0 ? x[0] : 0) + (mu > 1 ? x[1] : 0) + (mu > 2 ? x[2] : 0);
+            const int flip = (esum + (q.bc_neg[mu] ? wraps : 0)) & 1;
+            inv_s = flip ? -q.inv_c[h] : q.inv_c[h];
+        }
     }
     cplx<R> v[3], U[9];
-    const l2pol pol = LinkPolicy<LD_KEEP>(a.keep).of(dir ? j : c);
-    load_vec<P>((const E *)a.in, S, j, v);
+    const l2pol pol = LinkPolicy<LD>(keep).of(dir ? j : c);
+    load_vec<P>(in, S, j, v);
     if (dir) {
-        load_link<P, CM, LD_KEEP>(a.links_in, 4 * h + mu, S, j, a.link_scale[h], inv_s, pol, U);
+        load_link<P, CM, LD>(Gin, 4 * h + mu, S, j, 0.f, inv_s, pol, U);
 #pragma unroll
         for (int b = 0; b < 3; b++)
             v[b] = cneg(v[b]);
@@ -60,7 +63,7 @@ STAG_D void split_hop(const DslashArgs &a, int c, const int x[4], int mu, int h,
             for (int b = 0; b < 3; b++)
                 cmac_conj(acc[r], U[3 * b + r], v[b]);
     } else {
-        load_link<P, CM, LD_KEEP>(a.links_out, 4 * h + mu, S, c, a.link_scale[h], inv_s, pol, U);
+        load_link<P, CM, LD>(Gout, 4 * h + mu, S, c, 0.f, inv_s, pol, U);
 #pragma unroll
         for (int r = 0; r < 3; r++)
 #pragma unroll
@@ -76,6 +79,56 @@ STAG_D void acc_add(df &a, df b) {  // lo left unnormalised, as df_mac leaves it
     two_sum(a.hi, b.hi, s, e);
     a.hi = s;
     a.lo = __fadd_rn(a.lo, __fadd_rn(e, b.lo));
+}
+
+// the epilogue of one component o of D psi, at element `at` of its plane:
+// store it (EPI_NONE), or m^2 p - o, or b minus that (residuals; EPI_RESID
+// stores nothing); returns the component's share of the sum
+template <int P, int EPI>
+STAG_D red_t<typename Fmt<P>::R> split_epilogue(typename Fmt<P>::Elem *out, const typename Fmt<P>::Elem *pp,
+                                                const typename Fmt<P>::Elem *bp, typename Fmt<P>::R m2, int at,
+                                                cplx<typename Fmt<P>::R> o) {
+    using F = Fmt<P>;
+    using R = typename F::R;
+    if (EPI == EPI_NONE) {
+        o.re = rnorm<R>(o.re);
+        o.im = rnorm<R>(o.im);
+        __stcs(out + at, F::pack(o));
+        return red_zero<red_t<R>>();
+    }
+    const cplx<R> p = F::unpack(ld_keep(pp + at));
+    o = cneg(o);
+    mac(o.re, m2, p.re);
+    mac(o.im, m2, p.im);
+    o.re = rnorm<R>(o.re);
+    o.im = rnorm<R>(o.im);
+    const bool resid = EPI == EPI_RESID || EPI == EPI_RESID_STORE;
+    if (resid) {
+        const cplx<R> b = F::unpack(ld_keep(bp + at));
+        o.re = rsub(b.re, o.re);
+        o.im = rsub(b.im, o.im);
+    }
+    if (EPI != EPI_RESID)
+        __stcs(out + at, F::pack(o));
+    R d = rzero<R>();
+    mac(d, resid ? o.re : p.re, o.re);
+    mac(d, resid ? o.im : p.im, o.im);
+    return to_red(d);
+}
+
+// component w (colour) at lane `lane` of the block's NG partial sums, added
+// in the warps' order
+template <int P, int NG>
+STAG_D cplx<typename Fmt<P>::R> split_sum(const typename Fmt<P>::Elem (&part)[NG][3][SPLIT_SITES], int w, int lane) {
+    using F = Fmt<P>;
+    cplx<typename F::R> o = F::unpack(part[0][w][lane]);
+#pragma unroll
+    for (int q = 1; q < NG; q++) {
+        const cplx<typename F::R> u = F::unpack(part[q][w][lane]);
+        acc_add(o.re, u.re);
+        acc_add(o.im, u.im);
+    }
+    return o;
 }
 
 // NG warps per block; warp w takes the hops w 16/NG .. of the block's 32
@@ -107,7 +160,8 @@ __global__ void __launch_bounds__(32 * NG, 896 / (32 * NG)) dslash_split_kernel(
 #pragma unroll 1
         for (int q = 0; q < 16 / NG; q++) {
             const int hop = w * (16 / NG) + q;
-            split_hop<P, CM>(a, c, x, hop >> 2, (hop >> 1) & 1, hop & 1, acc);
+            stencil_hop<P, CM, LD_KEEP>(a.g, a.links_out, a.links_in, (const E *)a.in, a, a.keep, c, x, hop >> 2,
+                                        (hop >> 1) & 1, hop & 1, acc);
         }
 #pragma unroll
         for (int k = 0; k < 3; k++)
@@ -116,39 +170,9 @@ __global__ void __launch_bounds__(32 * NG, 896 / (32 * NG)) dslash_split_kernel(
     __syncthreads();
     red_t<R> dot = red_zero<red_t<R>>();
     if (w < 3 && in_range) {
-        cplx<R> o = F::unpack(part[0][w][lane]);
-#pragma unroll
-        for (int q = 1; q < NG; q++) {
-            const cplx<R> u = F::unpack(part[q][w][lane]);
-            acc_add(o.re, u.re);
-            acc_add(o.im, u.im);
-        }
-        const int S = a.g.stride;
-        if (EPI == EPI_NONE) {
-            o.re = rnorm<R>(o.re);
-            o.im = rnorm<R>(o.im);
-            __stcs((E *)a.out + w * S + c, F::pack(o));
-        } else {
-            const R m2 = scalar_as<R>(a.m2_in_args ? a.m2 : a.sc->m2);
-            const cplx<R> p = F::unpack(ld_keep((const E *)a.p + w * S + c));
-            o = cneg(o);
-            mac(o.re, m2, p.re);
-            mac(o.im, m2, p.im);
-            o.re = rnorm<R>(o.re);
-            o.im = rnorm<R>(o.im);
-            if (EPI == EPI_RESID || EPI == EPI_RESID_STORE) {
-                const cplx<R> b = F::unpack(ld_keep((const E *)a.b + w * S + c));
-                o.re = rsub(b.re, o.re);
-                o.im = rsub(b.im, o.im);
-            }
-            if (EPI != EPI_RESID)
-                __stcs((E *)a.out + w * S + c, F::pack(o));
-            R d = rzero<R>();
-            const bool resid = EPI == EPI_RESID || EPI == EPI_RESID_STORE;
-            mac(d, resid ? o.re : p.re, o.re);
-            mac(d, resid ? o.im : p.im, o.im);
-            dot = to_red(d);
-        }
+        const cplx<R> o = split_sum<P, NG>(part, w, lane);
+        const R m2 = EPI == EPI_NONE ? rzero<R>() : scalar_as<R>(a.m2_in_args ? a.m2 : a.sc->m2);
+        dot = split_epilogue<P, EPI>((E *)a.out, (const E *)a.p, (const E *)a.b, m2, w * a.g.stride + c, o);
     }
     dslash_reduce<EPI, BLOCK>(a, dot, smem);
 }

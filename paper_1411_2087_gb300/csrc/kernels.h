@@ -31,7 +31,7 @@ cudaError_t launch_cg_update(int prec, const Geom &g, void *x, void *r, const vo
 cudaError_t launch_cg_p_update(int prec, const Geom &g, const void *r, void *p,
                                const CgScalars *sc, cudaStream_t s);
 // x, r and p of one iteration of plain CG on a small lattice, with alpha from
-// the M Dslash's npap partials at `partial` (room for Vh / 128 more behind)
+// the M Dslash's npap partials at `partial` (room for Vh / 256 more behind)
 cudaError_t launch_cg_small_vectors(int prec, const Geom &g, void *x, void *r, void *p, const void *Ap,
                                     double *partial, int npap, CgScalars *sc, cudaStream_t s);
 // <p, M p> from the n block partials of a Dslash with EPI_M_PART, summed in
@@ -115,6 +115,9 @@ struct BatchArgs;
 cudaError_t launch_batch(int prec, int what, const BatchArgs &a, int block, cudaStream_t s);
 int batch_max_k(int prec);
 int batch_min_k(int prec);
+// batches of at most this many (site, system) items run the lane-mapped
+// Dslash in split form
+long long batch_split_items(int prec);
 
 // record the calling thread's last error message (read back by
 // stag_last_error_message) and return `code`

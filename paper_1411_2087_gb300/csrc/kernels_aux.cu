@@ -144,27 +144,20 @@ constexpr int FINISH_BLOCK = 1024;
 __global__ void __launch_bounds__(FINISH_BLOCK)
 pap_finish_kernel(const double *__restrict__ partial, int n, CgScalars *sc, int skip_if_done, const int *gate) {
     __shared__ double smem[32];
-    if (skip_if_done && sc->status != CG_RUNNING)
+    // the scalars are read together with the partials, not before them
+    const double rr = sc->rr;
+    const int status = sc->status;
+    const int open = gate ? *gate : 1;
+    const double share = partials_share<FINISH_BLOCK>(partial, n);
+    if ((skip_if_done && status != CG_RUNNING) || open == 0)
         return;
-    if (gate && *gate == 0)
-        return;
-    // four independent sums per thread over a fixed assignment, then the block tree
-    double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
-    int i = threadIdx.x;
-    for (; i + 3 * FINISH_BLOCK < n; i += 4 * FINISH_BLOCK) {
-        a0 += partial[i];
-        a1 += partial[i + FINISH_BLOCK];
-        a2 += partial[i + 2 * FINISH_BLOCK];
-        a3 += partial[i + 3 * FINISH_BLOCK];
-    }
-    for (; i < n; i += FINISH_BLOCK)
-        a0 += partial[i];
-    const double total = block_sum<FINISH_BLOCK>((a0 + a1) + (a2 + a3), smem);
+    const double total = block_sum<FINISH_BLOCK>(share, smem);
     if (threadIdx.x == 0) {
         sc->pAp = total;
-        if (sc->status == CG_RUNNING && !(total > 0.0 && total < INFINITY))
+        const bool ok = total > 0.0 && total < INFINITY;
+        if (status == CG_RUNNING && !ok)
             sc->status = CG_BREAKDOWN;
-        sc->alpha = make_dpair(sc->status == CG_RUNNING ? sc->rr / total : 0.0);
+        sc->alpha = make_dpair(status == CG_RUNNING && ok ? rr / total : 0.0);
     }
 }
 
@@ -188,15 +181,7 @@ cudaError_t launch_pap_finish(const double *partial, int n, CgScalars *sc, bool 
 // sum of n partials, valid in every thread
 template <int BLOCK> STAG_D double sum_partials(const double *__restrict__ v, int n, double *smem) {
     __shared__ double all;
-    double a = 0.0, b = 0.0;
-    int i = threadIdx.x;
-    for (; i + BLOCK < n; i += 2 * BLOCK) {
-        a += __ldcg(v + i);
-        b += __ldcg(v + i + BLOCK);
-    }
-    if (i < n)
-        a += __ldcg(v + i);
-    const double t = block_sum<BLOCK>(a + b, smem);
+    const double t = block_sum<BLOCK>(partials_share<BLOCK>(v, n), smem);
     if (threadIdx.x == 0)
         all = t;
     __syncthreads();
@@ -361,7 +346,7 @@ cudaError_t launch_cg_p_update(int prec, const Geom &g, const void *r, void *p,
     return cudaGetLastError();
 }
 
-constexpr int SMALL_BLOCK = 128;
+constexpr int SMALL_BLOCK = 256;
 static int small_grid(const Geom &g) { return (g.Vh + SMALL_BLOCK - 1) / SMALL_BLOCK; }
 
 cudaError_t launch_cg_small_vectors(int prec, const Geom &g, void *x, void *r, void *p, const void *Ap,

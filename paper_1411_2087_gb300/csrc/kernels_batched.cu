@@ -25,6 +25,12 @@ STAG_BATCH_EXTERN(P_F64, 256, 4)
 int batch_max_k(int prec) { return prec == P_F32 ? 8 : 4; }
 int batch_min_k(int prec) { return prec == P_F32 ? 4 : 2; }
 
+// An iteration in split form against one thread per (site, system): double
+// float 4096 items 35 / 50 us, 27648: 51 / 60, 55296: 87.5 / 83.5, 65536: 80.5
+// / 83, 98304: 114 / 119, 131072: 148 / 134; FP64 4096: 44 / 82, 41472: 132 /
+// 154, 98304: 254 / 278, 131072: 326 / 323.
+long long batch_split_items(int prec) { return prec == P_F64 ? 100000 : prec == P_DF64 ? 70000 : 0; }
+
 cudaError_t launch_batch(int prec, int what, const BatchArgs &a, int block, cudaStream_t s) {
     if (block != 128 && block != 256)
         return cudaErrorInvalidValue;

@@ -985,27 +985,18 @@ constexpr int FCG_FINISH = 1024;
 __global__ void __launch_bounds__(FCG_FINISH)
 fcg_finish_kernel(const double *__restrict__ partial, int n, CgScalars *sc, int first) {
     __shared__ double smem[32];
-    if (sc->status != CG_RUNNING)
+    // the scalars are read together with the partials, not before them
+    const int status = sc->status, reliable = sc->reliable;
+    const double rr = sc->rr, alpha = sc->alpha.d;
+    const double a = partials_share<FCG_FINISH>(partial, n), b = partials_share<FCG_FINISH>(partial + n, n);
+    if (status != CG_RUNNING)
         return;
-    // two independent sums per value and thread over a fixed assignment
-    double a0 = 0.0, a1 = 0.0, b0 = 0.0, b1 = 0.0;
-    int i = threadIdx.x;
-    for (; i + FCG_FINISH < n; i += 2 * FCG_FINISH) {
-        a0 += partial[i];
-        a1 += partial[i + FCG_FINISH];
-        b0 += partial[n + i];
-        b1 += partial[n + i + FCG_FINISH];
-    }
-    if (i < n) {
-        a0 += partial[i];
-        b0 += partial[n + i];
-    }
-    const double zr = block_sum<FCG_FINISH>(a0 + a1, smem);
-    const double zap = block_sum<FCG_FINISH>(b0 + b1, smem);
+    const double zr = block_sum<FCG_FINISH>(a, smem);
+    const double zap = block_sum<FCG_FINISH>(b, smem);
     if (threadIdx.x == 0) {
         double beta = 0.0;
         if (!first)
-            beta = sc->reliable ? zr / sc->rr : -sc->alpha.d * zap / sc->rr;
+            beta = reliable ? zr / rr : -alpha * zap / rr;
         sc->beta = make_dpair(beta);
         sc->rr = zr;
         if (!(zr > 0.0 && zr < INFINITY)) {

@@ -61,6 +61,30 @@ template <int BLOCK, class T> STAG_D double block_sum(T v, double *smem) {
     return r;
 }
 
+// This thread's share of the sum of n partials of stride `step` that other
+// blocks wrote: a fixed assignment to BLOCK threads, eight loads in flight
+// (one after the other, the last block of a 4096-block reduction waited 16
+// L2 latencies).  A warp past n skips its adds: an FP64 add costs its
+// scheduler 64 cycles also when it adds nothing.
+template <int BLOCK> STAG_D double partials_share(const double *__restrict__ v, int n, int step = 1) {
+    if (n <= BLOCK)
+        return (int)threadIdx.x < n ? __ldcg(v + (size_t)threadIdx.x * step) : 0.0;
+    double a = 0.0;
+    for (int base = threadIdx.x & ~31; base < n; base += 8 * BLOCK) {
+        double t[8];
+#pragma unroll
+        for (int u = 0; u < 8; u++) {
+            const int i = base + u * BLOCK + (threadIdx.x & 31);
+            t[u] = i < n ? __ldcg(v + (size_t)i * step) : 0.0;
+        }
+#pragma unroll
+        for (int u = 0; u < 8; u++)
+            if (base + u * BLOCK < n)
+                a += t[u];
+    }
+    return a;
+}
+
 // Grid-wide sum.  Every thread of every block must call it.  Returns true in
 // all threads of the one block that finishes last; there `total` holds the
 // grid sum (in every thread).  `ticket` must be zero on entry and is reset to
@@ -79,11 +103,7 @@ STAG_D bool grid_sum(T v, double *partial, unsigned *ticket, double *smem, doubl
     if (!last)
         return false;
     __threadfence();
-    double acc = 0.0;
-    const volatile double *vp = partial;
-    for (unsigned i = threadIdx.x; i < gridDim.x; i += BLOCK)
-        acc += vp[i];
-    acc = block_sum<BLOCK>(acc, smem);
+    const double acc = block_sum<BLOCK>(partials_share<BLOCK>(partial, (int)gridDim.x), smem);
     if (threadIdx.x == 0) {
         smem[0] = acc;
         *ticket = 0u;
@@ -113,14 +133,8 @@ STAG_D bool grid_sum2(T v0, T v1, double *partial, unsigned *ticket, double *sme
     if (!last)
         return false;
     __threadfence();
-    const volatile double *vp = partial;
-    double a0 = 0.0, a1 = 0.0;
-    for (unsigned i = threadIdx.x; i < gridDim.x; i += BLOCK) {
-        a0 += vp[2 * i];
-        a1 += vp[2 * i + 1];
-    }
-    a0 = block_sum<BLOCK>(a0, smem);
-    a1 = block_sum<BLOCK>(a1, smem);
+    const double a0 = block_sum<BLOCK>(partials_share<BLOCK>(partial, (int)gridDim.x, 2), smem);
+    const double a1 = block_sum<BLOCK>(partials_share<BLOCK>(partial + 1, (int)gridDim.x, 2), smem);
     __shared__ double res[2];
     if (threadIdx.x == 0) {
         res[0] = a0;

@@ -2,6 +2,7 @@
 // updates, multi-shift, batched multi-right-hand-side CG, and the block-size
 // autotuner.  Documentation in include/stag.h.
 #include "api_internal.h"
+#include "dslash_split.cuh"
 
 #include <algorithm>
 #include <map>
@@ -867,10 +868,15 @@ static int plan_batch(BatchPlan &P, int n, stag_lattice *lats, void *const *x, c
         P.a.kmax = std::max(P.a.kmax, P.a.grp[gi].K);
     // lane-mapped Dslash (double-float, FP64): one thread per (site, system)
     int dblocks = 0;
+    long long items = 0;
+    for (int gi = 0; gi < G; gi++)
+        items += (long long)P.a.grp[gi].g.Vh * P.a.grp[gi].K;
+    P.a.split = prec != STAG_F32 && items <= batch_split_items(prec);
+    const int per = P.a.split ? SPLIT_SITES : P.block;
     for (int gi = 0; gi < G; gi++) {
         BatchGroup &gr = P.a.grp[gi];
         gr.dblock0 = dblocks;
-        gr.dnblocks = (int)(((long long)gr.g.Vh * gr.K + P.block - 1) / P.block);
+        gr.dnblocks = (int)(((long long)gr.g.Vh * gr.K + per - 1) / per);
         dblocks += gr.dnblocks;
         partial_total += (size_t)std::max(gr.nblocks, gr.dnblocks) * BATCH_KMAX;
     }
