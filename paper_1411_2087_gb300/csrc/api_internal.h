@@ -21,6 +21,7 @@
 #include "batched.cuh"
 #include "dslash.cuh"
 #include "kernels.h"
+#include "small_sums.cuh"
 
 using namespace stag;
 
@@ -327,10 +328,9 @@ static inline int m_block(const stag_lattice lat, int prec) {
 }
 
 // On lattices up to this many sites per parity the launches are short and
-// counting them is what matters: plain CG leaves its sums to the next kernel
-// (launch_cg_small_vectors), the other solvers sum <p, Ap> in the M Dslash's
-// last block.  Larger ones write block partials and sum them in a one-block
-// kernel, which lets the Dslash blocks retire without a ticket.
+// counting them is what matters: the solvers leave <p, Ap> to the next kernel
+// (small_sums.cuh).  Larger ones sum the M Dslash's partials in a one-block
+// kernel.
 constexpr int kSmallVh = 65536;
 
 // the M Dslash Ap = m^2 p - D_eo t of an iteration (skip_if_done: it returns
@@ -344,19 +344,28 @@ static inline DslashArgs m_part_args(stag_lattice lat, int prec, const void *t, 
     return a;
 }
 
-// Ap = m^2 p - D_eo t with <p, Ap>, alpha and the breakdown test in sc
+// Ap = m^2 p - D_eo t with the partials of <p, Ap> in *pap for the next
+// kernel, or (larger lattices) with alpha and the breakdown test in sc
 static inline cudaError_t enqueue_m_pap(stag_lattice lat, int prec, const void *t, void *Ap, const void *p,
-                                        bool skip_if_done, cudaStream_t s, const int *gate = nullptr) {
+                                        bool skip_if_done, cudaStream_t s, PapPartials *pap,
+                                        const int *gate = nullptr) {
     DslashArgs a = m_part_args(lat, prec, t, Ap, p, skip_if_done);
     a.gate = gate;
     const int block = m_block(lat, prec);
-    if (lat->geom.Vh <= kSmallVh)
-        return launch_dslash(prec, EPI_M_PAP, a, block, s);
     cudaError_t e = launch_dslash(prec, EPI_M_PART, a, block, s);
     if (e != cudaSuccess)
         return e;
-    return launch_pap_finish(lat->partial, dslash_blocks(prec, EPI_M_PART, a, block), lat->sc, skip_if_done, s, gate);
+    *pap = PapPartials();
+    const int n = dslash_blocks(prec, EPI_M_PART, a, block);
+    if (lat->geom.Vh > kSmallVh)
+        return launch_pap_finish(lat->partial, n, lat->sc, skip_if_done, s, gate);
+    pap->v = lat->partial;
+    pap->n = n;
+    return cudaSuccess;
 }
+
+// where a kernel that reads those partials puts its own
+static inline double *next_partial(stag_lattice lat) { return lat->partial + dslash_max_blocks(lat->Vh); }
 
 // Source normalisation (stag_api.cu): when the exponent k of b's largest
 // entry is far from 0 (double-float and FP32 fields), `scaled` is a copy

@@ -30,10 +30,11 @@ cudaError_t launch_cg_update(int prec, const Geom &g, void *x, void *r, const vo
                              const void *Ap, double *partial, CgScalars *sc, cudaStream_t s);
 cudaError_t launch_cg_p_update(int prec, const Geom &g, const void *r, void *p,
                                const CgScalars *sc, cudaStream_t s);
-// x, r and p of one iteration of plain CG on a small lattice, with alpha from
-// the M Dslash's npap partials at `partial` (room for Vh / 256 more behind)
+// x, r and p of one iteration of plain CG on a small lattice (rr_part: room
+// for Vh / 256 + 1 partials)
+struct PapPartials;
 cudaError_t launch_cg_small_vectors(int prec, const Geom &g, void *x, void *r, void *p, const void *Ap,
-                                    double *partial, int npap, CgScalars *sc, cudaStream_t s);
+                                    const PapPartials &pap, double *rr_part, CgScalars *sc, cudaStream_t s);
 // <p, M p> from the n block partials of a Dslash with EPI_M_PART, summed in
 // block order; then alpha = |r|^2 / <p, M p> and the breakdown test (as the
 // EPI_M_PAP epilogue).  Returns at once when skip_if_done and the solve has
@@ -90,7 +91,7 @@ cudaError_t launch_long_links(const Geom &g, const double *fat, double *lng, cud
 cudaError_t launch_mixed_init(int hi, int lo, const Geom &g, void *x, void *r, const void *b, float *xs,
                               void *rs, void *p, double *partial, CgScalars *sc, cudaStream_t s);
 cudaError_t launch_mixed_update(int lo, const Geom &g, float *xs, void *rs, const void *p, const void *Ap,
-                                double *partial, CgScalars *sc, cudaStream_t s);
+                                const PapPartials &pap, double *partial, CgScalars *sc, cudaStream_t s);
 cudaError_t launch_mixed_accum(int hi, const Geom &g, void *x, float *xs, const CgScalars *sc,
                                cudaStream_t s);
 cudaError_t launch_mixed_restart(int hi, int lo, const Geom &g, const void *r, void *rs, CgScalars *sc,
@@ -100,8 +101,9 @@ cudaError_t launch_mixed_restart(int hi, int lo, const Geom &g, const void *r, v
 // lo >= 0: mixed precision (vectors in prec, the Dslash pair in lo = FP32)
 cudaError_t launch_ms_init(int prec, const Geom &g, const MsArgs &a, double *partial, CgScalars *sc,
                            ShiftState *st, cudaStream_t s, int lo = -1);
-cudaError_t launch_ms_update(int prec, const Geom &g, const MsArgs &a, const void *Ap, double *partial,
-                             CgScalars *sc, ShiftState *st, cudaStream_t s, int lo = -1);
+// pap[0]: of the Dslash pair in prec, pap[1]: in lo
+cudaError_t launch_ms_update(int prec, const Geom &g, const MsArgs &a, const void *Ap, const PapPartials pap[2],
+                             double *partial, CgScalars *sc, ShiftState *st, cudaStream_t s, int lo = -1);
 cudaError_t launch_ms_p(int prec, const Geom &g, const MsArgs &a, const CgScalars *sc,
                         const ShiftState *st, cudaStream_t s, int lo = -1);
 // after a reliable update of the base residual (gated on sc->reliable)

@@ -1,6 +1,7 @@
 // CG vector kernels and field import/export.
 #include "dslash.cuh"
 #include "kernels.h"
+#include "small_sums.cuh"
 
 #include <cfloat>
 
@@ -168,36 +169,22 @@ cudaError_t launch_pap_finish(const double *partial, int n, CgScalars *sc, bool 
 }
 
 // --------------------------------------------------------------------------
-// The vector kernels of plain CG on small lattices.  There every launch lasts
-// a few microseconds, and a reduction that ends in its own kernel costs as
-// much again: partial, fence, ticket, and the last block's loads one after
-// the other (at 8^4 the M Dslash took 8.5 us with the ticket and takes 4.6
-// without, the update 6.9 and now 4.4).  Here a kernel leaves its block
-// partials and each block of the next kernel sums them for itself, in the
-// same order, so all blocks get the same scalars.  No kernel reads a scalar
-// that it writes: the update kernel reads rr, iter, status and writes alpha,
-// pAp, up_*; the direction kernel reads up_* and writes the others.
+// The vector kernels of plain CG on small lattices: <p, Ap> and |r|^2 are
+// both summed by the kernel after the one that leaves their partials
+// (small_sums.cuh; the update at 8^4 took 6.9 us with a ticket, now 4.4).  No
+// kernel reads a scalar that it writes: the update kernel reads rr, iter,
+// status and writes alpha, pAp, up_*; the direction kernel reads up_* and
+// writes the others.
 // --------------------------------------------------------------------------
-// sum of n partials, valid in every thread
-template <int BLOCK> STAG_D double sum_partials(const double *__restrict__ v, int n, double *smem) {
-    __shared__ double all;
-    const double t = block_sum<BLOCK>(partials_share<BLOCK>(v, n), smem);
-    if (threadIdx.x == 0)
-        all = t;
-    __syncthreads();
-    return all;
-}
-
 // x += alpha p, r -= alpha Ap with alpha = rr / <p, Ap> from the M Dslash's
 // npap partials; one partial of |r|^2 per block
 template <int P, int BLOCK>
 __global__ void __launch_bounds__(BLOCK)
 cg_small_update_kernel(Geom g, typename Fmt<P>::Elem *x, typename Fmt<P>::Elem *r, const typename Fmt<P>::Elem *p,
-                       const typename Fmt<P>::Elem *Ap, const double *pap, int npap, double *rr_part, CgScalars *sc) {
+                       const typename Fmt<P>::Elem *Ap, PapPartials pap, double *rr_part, CgScalars *sc) {
     using R = typename Fmt<P>::R;
     __shared__ double smem[32];
     __shared__ dpair salpha;
-    __shared__ int sstatus;
     const int c = blockIdx.x * BLOCK + threadIdx.x;
     cplx<R> xv[3], rv[3], pv[3], av[3];
     if (c < g.Vh) {  // in flight while the partials are summed
@@ -206,20 +193,7 @@ cg_small_update_kernel(Geom g, typename Fmt<P>::Elem *x, typename Fmt<P>::Elem *
         load_vec<P>(p, g.stride, c, pv);
         load_vec<P>(Ap, g.stride, c, av);
     }
-    int status = sc->status;
-    if (status == CG_RUNNING) {
-        const double total = sum_partials<BLOCK>(pap, npap, smem);
-        if (threadIdx.x == 0) {
-            sstatus = total > 0.0 && total < INFINITY ? CG_RUNNING : CG_BREAKDOWN;
-            salpha = make_dpair(sstatus == CG_RUNNING ? sc->rr / total : 0.0);
-            if (blockIdx.x == 0) {
-                sc->pAp = total;
-                sc->alpha = salpha;
-            }
-        }
-        __syncthreads();
-        status = sstatus;
-    }
+    const int status = iteration_alpha<BLOCK>(pap, sc, smem, salpha);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         sc->up_rr = sc->rr;
         sc->up_iter = sc->iter;
@@ -350,13 +324,12 @@ constexpr int SMALL_BLOCK = 256;
 static int small_grid(const Geom &g) { return (g.Vh + SMALL_BLOCK - 1) / SMALL_BLOCK; }
 
 cudaError_t launch_cg_small_vectors(int prec, const Geom &g, void *x, void *r, void *p, const void *Ap,
-                                    double *partial, int npap, CgScalars *sc, cudaStream_t s) {
-    double *rr_part = partial + npap;
+                                    const PapPartials &pap, double *rr_part, CgScalars *sc, cudaStream_t s) {
     const int grid = small_grid(g);
     STAG_PREC_SWITCH(prec, {
         using E = typename Fmt<P>::Elem;
         cg_small_update_kernel<P, SMALL_BLOCK><<<grid, SMALL_BLOCK, 0, s>>>(g, (E *)x, (E *)r, (const E *)p,
-                                                                           (const E *)Ap, partial, npap, rr_part, sc);
+                                                                           (const E *)Ap, pap, rr_part, sc);
         cg_small_p_kernel<P, SMALL_BLOCK><<<grid, SMALL_BLOCK, 0, s>>>(g, (const E *)r, (E *)p, rr_part, grid, sc);
     });
     return cudaGetLastError();

@@ -4,6 +4,7 @@
 // kernels_netpath.cu.
 #include "learned.cuh"
 #include "kernels.h"
+#include "small_sums.cuh"
 
 namespace stag {
 
@@ -65,15 +66,16 @@ __global__ void solver_to_pair_kernel(Geom sg, const typename Fmt<P>::Elem *f, c
 template <int P, int BLOCK>
 __global__ void __launch_bounds__(BLOCK)
 fcg_update_kernel(Geom g, typename Fmt<P>::Elem *x, typename Fmt<P>::Elem *r,
-                  const typename Fmt<P>::Elem *p, const typename Fmt<P>::Elem *Ap, double *partial,
-                  CgScalars *sc) {
+                  const typename Fmt<P>::Elem *p, const typename Fmt<P>::Elem *Ap, PapPartials pap,
+                  double *partial, CgScalars *sc) {
     using R = typename Fmt<P>::R;
     __shared__ double smem[32];
-    const bool run = sc->status == CG_RUNNING;
+    __shared__ dpair salpha;
+    const int status = iteration_alpha<BLOCK>(pap, sc, smem, salpha);
     const int c = blockIdx.x * BLOCK + threadIdx.x;
     red_t<R> dot = red_zero<red_t<R>>();
-    if (run && c < g.Vh) {
-        const R alpha = scalar_as<R>(sc->alpha);
+    if (status == CG_RUNNING && c < g.Vh) {
+        const R alpha = scalar_as<R>(salpha);
         const R malpha = -alpha;
         cplx<R> xv[3], rv[3], pv[3], av[3];
         load_vec<P>(x, g.stride, c, xv);
@@ -97,7 +99,8 @@ fcg_update_kernel(Geom g, typename Fmt<P>::Elem *x, typename Fmt<P>::Elem *r,
     }
     double total;
     if (grid_sum<BLOCK>(dot, partial, &sc->ticket, smem, total) && threadIdx.x == 0) {
-        if (sc->status == CG_RUNNING) {
+        sc->status = status;
+        if (status == CG_RUNNING) {
             sc->fcg_rr = total;
             sc->iter += 1;
             if (!(total < INFINITY))
@@ -141,11 +144,11 @@ cudaError_t launch_solver_to_pair(int prec, const Geom &sg, const void *f, const
 constexpr int FB = 256;
 
 cudaError_t launch_fcg_update(int prec, const Geom &g, void *x, void *r, const void *p, const void *Ap,
-                              double *partial, CgScalars *sc, cudaStream_t s) {
+                              const PapPartials &pap, double *partial, CgScalars *sc, cudaStream_t s) {
     NP_SWITCH(prec, {
         using E = typename Fmt<P>::Elem;
         fcg_update_kernel<P, FB><<<(g.Vh + FB - 1) / FB, FB, 0, s>>>(g, (E *)x, (E *)r, (const E *)p,
-                                                                     (const E *)Ap, partial, sc);
+                                                                     (const E *)Ap, pap, partial, sc);
     });
     return cudaGetLastError();
 }

@@ -24,6 +24,7 @@
 // rr = <r_s, z>; mixed_update and mixed_restart then leave both alone.
 #include "dslash.cuh"
 #include "kernels.h"
+#include "small_sums.cuh"
 
 namespace stag {
 
@@ -93,20 +94,23 @@ mixed_init_kernel(Geom g, typename Fmt<PH>::Elem *x, typename Fmt<PH>::Elem *r,
 template <int PL>
 __global__ void __launch_bounds__(MB)
 mixed_update_kernel(Geom g, float2 *xs, typename Fmt<PL>::Elem *rs, const typename Fmt<PL>::Elem *p,
-                    const typename Fmt<PL>::Elem *Ap, double *partial, CgScalars *sc) {
+                    const typename Fmt<PL>::Elem *Ap, PapPartials pap, double *partial, CgScalars *sc) {
     using RL = typename Fmt<PL>::R;
     __shared__ double smem[32];
+    __shared__ dpair salpha;
     const int c = blockIdx.x * MB + threadIdx.x;
-    const bool run = sc->status == CG_RUNNING;
-    red_t<RL> dot = red_zero<red_t<RL>>();
-    if (run && c < g.Vh) {
-        const float alpha = scalar_as<float>(sc->alpha);
-        cplx<float> xv[3];
-        cplx<RL> rv[3], pv[3], av[3];
+    cplx<float> xv[3];
+    cplx<RL> rv[3], pv[3], av[3];
+    if (c < g.Vh) {  // in flight while alpha is found
         load_vec<P_F32>(xs, g.stride, c, xv);
         load_vec<PL>(rs, g.stride, c, rv);
         load_vec<PL>(p, g.stride, c, pv);
         load_vec<PL>(Ap, g.stride, c, av);
+    }
+    const int status = iteration_alpha<MB>(pap, sc, smem, salpha);
+    red_t<RL> dot = red_zero<red_t<RL>>();
+    if (status == CG_RUNNING && c < g.Vh) {
+        const float alpha = scalar_as<float>(salpha);
 #pragma unroll
         for (int k = 0; k < 3; k++) {
             xv[k].re = fmaf(alpha, (float)pv[k].re, xv[k].re);
@@ -121,7 +125,8 @@ mixed_update_kernel(Geom g, float2 *xs, typename Fmt<PL>::Elem *rs, const typena
     double total;
     if (grid_sum<MB>(dot, partial, &sc->ticket, smem, total) && threadIdx.x == 0) {
         sc->reliable = 0;
-        if (sc->status == CG_RUNNING) {
+        sc->status = status;
+        if (status == CG_RUNNING) {
             sc->iter += 1;
             const double rn = sqrt(total);
             if (!(total < INFINITY)) {
@@ -237,11 +242,11 @@ cudaError_t launch_mixed_init(int hi, int lo, const Geom &g, void *x, void *r, c
 }
 
 cudaError_t launch_mixed_update(int lo, const Geom &g, float *xs, void *rs, const void *p, const void *Ap,
-                                double *partial, CgScalars *sc, cudaStream_t s) {
+                                const PapPartials &pap, double *partial, CgScalars *sc, cudaStream_t s) {
     LO_SWITCH(lo, {
         using EL = typename Fmt<PL>::Elem;
         mixed_update_kernel<PL><<<grid_of(g), MB, 0, s>>>(g, (float2 *)xs, (EL *)rs, (const EL *)p,
-                                                          (const EL *)Ap, partial, sc);
+                                                          (const EL *)Ap, pap, partial, sc);
     });
     return cudaGetLastError();
 }

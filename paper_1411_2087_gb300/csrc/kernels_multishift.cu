@@ -35,6 +35,7 @@
 // the exact operator (sc->ms_hi_op / ms_lo_op gate the two paths).
 #include "dslash.cuh"
 #include "kernels.h"
+#include "small_sums.cuh"
 
 namespace stag {
 
@@ -118,11 +119,11 @@ ms_init_kernel(Geom g, MsArgs a, double *partial, CgScalars *sc, ShiftState *st)
 
 // zeta_{k+1}, alpha^s for every shift from the scalars of the base CG; every
 // block computes them (one lane per shift) into shared memory
-STAG_D void ms_shift_scalars(const MsArgs &a, const CgScalars *sc, const ShiftState *st,
+STAG_D void ms_shift_scalars(const MsArgs &a, double al, const CgScalars *sc, const ShiftState *st,
                              double *zeta_next, double *alpha_s) {
     const int s = threadIdx.x;
     if (s < a.n) {
-        const double al = sc->alpha.d, alp = sc->alpha_prev, bep = sc->beta_prev;
+        const double alp = sc->alpha_prev, bep = sc->beta_prev;
         const double z = st[s].zeta, zp = st[s].zeta_prev;
         const double den = al * bep * (zp - z) + zp * alp * (1.0 + a.delta[s] * al);
         const double zn = z * zp * alp / den;
@@ -135,7 +136,8 @@ STAG_D void ms_shift_scalars(const MsArgs &a, const CgScalars *sc, const ShiftSt
 // updates x_s += alpha^s p_s run in ms_p_kernel, which reads p_s anyway)
 template <int P, int PA>
 __global__ void __launch_bounds__(MSB)
-ms_update_kernel(Geom g, MsArgs a, const void *Ap, double *partial, CgScalars *sc, ShiftState *st) {
+ms_update_kernel(Geom g, MsArgs a, const void *Ap, PapPartials pap0, PapPartials pap1, double *partial,
+                 CgScalars *sc, ShiftState *st) {
     using F = Fmt<P>;
     using R = typename F::R;
     using E = typename F::Elem;
@@ -143,24 +145,26 @@ ms_update_kernel(Geom g, MsArgs a, const void *Ap, double *partial, CgScalars *s
     __shared__ double smem[32];
     __shared__ double zeta_next[MS_MAX], alpha_s[MS_MAX];
     __shared__ int active[MS_MAX];
+    __shared__ dpair salpha;
     // the previous iteration's solution updates are done (ms_p_kernel has
     // finished); written before this block's ticket, so before the last
     // block below advances the iteration count
     if (blockIdx.x == 0 && threadIdx.x == 0)
         sc->ms_xdone = sc->iter;
-    const bool run = sc->status == CG_RUNNING;
     // which path computed M p this iteration (read before any block's ticket,
     // so before the last block below sets it for the next iteration)
     const bool hi_path = PA == P || sc->ms_hi_op;
+    const int status = iteration_alpha<MSB>(hi_path ? pap0 : pap1, sc, smem, salpha);
+    const bool run = status == CG_RUNNING;
     if (run)
-        ms_shift_scalars(a, sc, st, zeta_next, alpha_s);
+        ms_shift_scalars(a, salpha.d, sc, st, zeta_next, alpha_s);
     if (threadIdx.x < MS_MAX)
         active[threadIdx.x] = threadIdx.x < a.n ? st[threadIdx.x].active : 0;
     __syncthreads();
     const int c = blockIdx.x * MSB + threadIdx.x;
     red_t<R> dot = red_zero<red_t<R>>();
     if (run && c < g.Vh) {
-        const R alpha = scalar_as<R>(sc->alpha);
+        const R alpha = scalar_as<R>(salpha);
         cplx<R> rv[3], av[3];
         load_vec<P>((const E *)a.r, g.stride, c, rv);
         if (hi_path) {
@@ -184,7 +188,8 @@ ms_update_kernel(Geom g, MsArgs a, const void *Ap, double *partial, CgScalars *s
     }
     double total;
     if (grid_sum<MSB>(dot, partial, &sc->ticket, smem, total) && threadIdx.x == 0) {
-        if (sc->status == CG_RUNNING) {
+        sc->status = status;
+        if (status == CG_RUNNING) {
             const double beta = total / sc->rr;
             sc->beta = make_dpair(beta);
             sc->iter += 1;
@@ -208,7 +213,7 @@ ms_update_kernel(Geom g, MsArgs a, const void *Ap, double *partial, CgScalars *s
                 else
                     any = true;
             }
-            sc->alpha_prev = sc->alpha.d;
+            sc->alpha_prev = salpha.d;
             sc->beta_prev = beta;
             sc->rr = total;
             const double rn = sqrt(total);
@@ -395,18 +400,18 @@ cudaError_t launch_ms_init(int prec, const Geom &g, const MsArgs &a, double *par
     return cudaGetLastError();
 }
 
-cudaError_t launch_ms_update(int prec, const Geom &g, const MsArgs &a, const void *Ap, double *partial,
-                             CgScalars *sc, ShiftState *st, cudaStream_t s, int lo) {
+cudaError_t launch_ms_update(int prec, const Geom &g, const MsArgs &a, const void *Ap, const PapPartials pap[2],
+                             double *partial, CgScalars *sc, ShiftState *st, cudaStream_t s, int lo) {
     if (lo == P_F32 && (prec == P_F64 || prec == P_DF64)) {
         if (prec == P_F64)
-            ms_update_kernel<P_F64, P_F32><<<grid_of(g), MSB, 0, s>>>(g, a, Ap, partial, sc, st);
+            ms_update_kernel<P_F64, P_F32><<<grid_of(g), MSB, 0, s>>>(g, a, Ap, pap[0], pap[1], partial, sc, st);
         else
-            ms_update_kernel<P_DF64, P_F32><<<grid_of(g), MSB, 0, s>>>(g, a, Ap, partial, sc, st);
+            ms_update_kernel<P_DF64, P_F32><<<grid_of(g), MSB, 0, s>>>(g, a, Ap, pap[0], pap[1], partial, sc, st);
         return cudaGetLastError();
     }
     if (lo >= 0)
         return cudaErrorInvalidValue;
-    MS_PREC_SWITCH(prec, ms_update_kernel<P, P><<<grid_of(g), MSB, 0, s>>>(g, a, Ap, partial, sc, st));
+    MS_PREC_SWITCH(prec, ms_update_kernel<P, P><<<grid_of(g), MSB, 0, s>>>(g, a, Ap, pap[0], pap[1], partial, sc, st));
     return cudaGetLastError();
 }
 

@@ -687,9 +687,10 @@ static int fcg_run(stag_net n, int prec, bool use_net, double mass, double tol2b
             DslashArgs b1 = dslash_args(lat, prec, STAG_ODD, w.p, w.t);
             b1.skip_if_done = 1;
             CUDA_TRY(launch_dslash(prec, EPI_NONE, b1, lat->dslash_block[prec], s));
-            CUDA_TRY(enqueue_m_pap(lat, prec, w.t, w.Ap, w.p, true, s));
+            PapPartials pap;
+            CUDA_TRY(enqueue_m_pap(lat, prec, w.t, w.Ap, w.p, true, s, &pap));
             // x += alpha p, r -= alpha Ap, |r|^2 and the stopping test
-            CUDA_TRY(launch_fcg_update(prec, g, w.xw, w.r, w.p, w.Ap, lat->partial, lat->sc, s));
+            CUDA_TRY(launch_fcg_update(prec, g, w.xw, w.r, w.p, w.Ap, pap, next_partial(lat), lat->sc, s));
             // z = N(r), beta = -alpha <z, Ap> / <z_old, r_old>, p = z + beta p
             CUDA_TRY(precondition(n, prec, use_net, w.r, n->z[prec], w.Ap, 0, gate, s));
             CUDA_TRY(launch_cg_p_update(prec, g, n->z[prec], w.p, lat->sc, s));

@@ -65,7 +65,8 @@ cudaError_t launch_adam(int n, double *w, const double *grad, double *m, double 
                         cudaStream_t s);
 cudaError_t launch_solver_to_pair(int prec, const Geom &sg, const void *f, const void *sub, float2 *pair,
                                   cudaStream_t s);
+struct PapPartials;
 cudaError_t launch_fcg_update(int prec, const Geom &g, void *x, void *r, const void *p, const void *Ap,
-                              double *partial, CgScalars *sc, cudaStream_t s);
+                              const PapPartials &pap, double *partial, CgScalars *sc, cudaStream_t s);
 
 }  // namespace stag

@@ -53,9 +53,10 @@ static cudaError_t enqueue_mixed_body(stag_lattice lat, int hi, int lo, bool hos
     a1.skip_if_done = host_mode;
     if ((e = launch_dslash(lo, EPI_NONE, a1, lat->dslash_block[lo], s)) != cudaSuccess)
         return e;
-    if ((e = enqueue_m_pap(lat, lo, L.t, L.Ap, L.p, host_mode, s)) != cudaSuccess)
+    PapPartials pap;
+    if ((e = enqueue_m_pap(lat, lo, L.t, L.Ap, L.p, host_mode, s, &pap)) != cudaSuccess)
         return e;
-    if ((e = launch_mixed_update(lo, g, lat->xs, L.r, L.p, L.Ap, lat->partial, lat->sc, s)) != cudaSuccess)
+    if ((e = launch_mixed_update(lo, g, lat->xs, L.r, L.p, L.Ap, pap, next_partial(lat), lat->sc, s)) != cudaSuccess)
         return e;
     if (!side) {
         if ((e = enqueue_reliable_update(lat, hi, lo, s)) != cudaSuccess)
@@ -365,7 +366,7 @@ static const int *scalar_flag(stag_lattice lat, size_t off) { return (const int 
 // the Dslash pair M p_base of one iteration in precision op, with the
 // <p, M p> partials and alpha; gate: run only while *gate != 0
 static cudaError_t enqueue_ms_op(stag_lattice lat, int op, const void *pb, bool host_mode, const int *gate,
-                                 cudaStream_t s) {
+                                 PapPartials *pap, cudaStream_t s) {
     CgWork &w = lat->cg[op];
     DslashArgs a1 = dslash_args(lat, op, STAG_ODD, pb, w.t);
     a1.skip_if_done = host_mode;
@@ -373,26 +374,27 @@ static cudaError_t enqueue_ms_op(stag_lattice lat, int op, const void *pb, bool 
     cudaError_t e = launch_dslash(op, EPI_NONE, a1, lat->dslash_block[op], s);
     if (e != cudaSuccess)
         return e;
-    return enqueue_m_pap(lat, op, w.t, w.Ap, pb, host_mode, s, gate);
+    return enqueue_m_pap(lat, op, w.t, w.Ap, pb, host_mode, s, pap, gate);
 }
 
 static cudaError_t enqueue_ms_body(stag_lattice lat, int prec, const MsArgs &a, bool host_mode, int lo = -1,
                                    cudaStream_t side = nullptr) {
     cudaStream_t s = lat->stream;
     cudaError_t e;
+    PapPartials pap[2];
     if (lo < 0) {
-        if ((e = enqueue_ms_op(lat, prec, a.p[a.base], host_mode, nullptr, s)) != cudaSuccess)
+        if ((e = enqueue_ms_op(lat, prec, a.p[a.base], host_mode, nullptr, &pap[0], s)) != cudaSuccess)
             return e;
     } else {
         // the exact operator while |r| is large, the FP32 one afterwards
         if ((e = enqueue_ms_op(lat, prec, a.p[a.base], host_mode, scalar_flag(lat, offsetof(CgScalars, ms_hi_op)),
-                               s)) != cudaSuccess ||
-            (e = enqueue_ms_op(lat, lo, a.p_lo, host_mode, scalar_flag(lat, offsetof(CgScalars, ms_lo_op)), s)) !=
-                cudaSuccess)
+                               &pap[0], s)) != cudaSuccess ||
+            (e = enqueue_ms_op(lat, lo, a.p_lo, host_mode, scalar_flag(lat, offsetof(CgScalars, ms_lo_op)), &pap[1],
+                               s)) != cudaSuccess)
             return e;
     }
     const void *Ap = lat->cg[lo >= 0 ? lo : prec].Ap;
-    if ((e = launch_ms_update(prec, lat->geom, a, Ap, lat->partial, lat->sc, lat->ms_state, s, lo)) !=
+    if ((e = launch_ms_update(prec, lat->geom, a, Ap, pap, next_partial(lat), lat->sc, lat->ms_state, s, lo)) !=
         cudaSuccess)
         return e;
     if ((e = launch_ms_p(prec, lat->geom, a, lat->sc, lat->ms_state, s, lo)) != cudaSuccess)

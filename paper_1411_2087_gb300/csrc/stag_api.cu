@@ -704,19 +704,12 @@ cudaError_t enqueue_cg_body(stag_lattice lat, CgWork &w, cudaStream_t s, bool sk
     a1.skip_if_done = skip_if_done;
     if ((e = launch_dslash(prec, EPI_NONE, a1, lat->dslash_block[prec], s)) != cudaSuccess)
         return e;
-    if (lat->geom.Vh <= kSmallVh) {
-        // the vector kernels sum the partials of <p, Ap> themselves
-        DslashArgs a2 = m_part_args(lat, prec, w.t, w.Ap, w.p, skip_if_done);
-        const int block = m_block(lat, prec);
-        if ((e = launch_dslash(prec, EPI_M_PART, a2, block, s)) != cudaSuccess)
-            return e;
-        return launch_cg_small_vectors(prec, lat->geom, w.xw, w.r, w.p, w.Ap, lat->partial,
-                                       dslash_blocks(prec, EPI_M_PART, a2, block), lat->sc, s);
-    }
-    // Ap = M p with one partial of <p, Ap> per block; a one-block kernel sums
-    // them (cheaper at these grid sizes than a last-block ticket in the Dslash)
-    if ((e = enqueue_m_pap(lat, prec, w.t, w.Ap, w.p, skip_if_done, s)) != cudaSuccess)
+    // Ap = M p with one partial of <p, Ap> per block
+    PapPartials pap;
+    if ((e = enqueue_m_pap(lat, prec, w.t, w.Ap, w.p, skip_if_done, s, &pap)) != cudaSuccess)
         return e;
+    if (pap.n > 0)
+        return launch_cg_small_vectors(prec, lat->geom, w.xw, w.r, w.p, w.Ap, pap, next_partial(lat), lat->sc, s);
     if ((e = launch_cg_update(prec, lat->geom, w.xw, w.r, w.p, w.Ap, lat->partial, lat->sc, s)) !=
         cudaSuccess)
         return e;
