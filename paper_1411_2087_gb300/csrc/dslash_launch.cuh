@@ -35,9 +35,12 @@ static void launch_one(int grid, const DslashArgs &a, cudaStream_t s) {
 // the split form with NG warps per block
 template <int P, int NG, int CM>
 static cudaError_t launch_split_g(int epi, const DslashArgs &a, cudaStream_t s) {
-    const int grid = dslash_blocks(P, epi, a, 0), block = 32 * NG;
-    if (grid == 0)
+    const dim3 grid(dslash_blocks(P, epi, a, 0), a.nbatch > 1 ? a.nbatch : 1);
+    const int block = 32 * NG;
+    if (grid.x == 0)
         return cudaSuccess;
+    if (grid.y > 1 && epi != EPI_NONE && epi != EPI_M)
+        return cudaErrorInvalidValue;
     switch (epi) {
     case EPI_NONE: dslash_split_kernel<P, EPI_NONE, NG, CM><<<grid, block, 0, s>>>(a); break;
     case EPI_M: dslash_split_kernel<P, EPI_M, NG, CM><<<grid, block, 0, s>>>(a); break;
@@ -74,6 +77,8 @@ static cudaError_t launch_p_b_c(int epi, const DslashArgs &a, cudaStream_t s) {
     const int grid = dslash_blocks(P, epi, a, BLOCK);
     if (grid == 0)
         return cudaSuccess;
+    if (a.nbatch > 1)  // the split form only
+        return cudaErrorInvalidValue;
     switch (epi) {
     case EPI_NONE: launch_one<P, EPI_NONE, BLOCK, CM>(grid, a, s); break;
     case EPI_M: launch_one<P, EPI_M, BLOCK, CM>(grid, a, s); break;

@@ -153,6 +153,7 @@ __global__ void __launch_bounds__(32 * NG, 896 / (32 * NG)) dslash_split_kernel(
     const int n2 = a.cn ? a.cnb : 0;
     const int c = i < n1 ? a.c0 + i : a.c0b + (i - n1);
     const bool in_range = i < n1 + n2;
+    const size_t vec = blockIdx.y * a.vec_step;  // this block's vector of a batch
     if (in_range) {
         int x[4];
         cb_coords(a.g, c, a.out_par, x);
@@ -160,8 +161,8 @@ __global__ void __launch_bounds__(32 * NG, 896 / (32 * NG)) dslash_split_kernel(
 #pragma unroll 1
         for (int q = 0; q < 16 / NG; q++) {
             const int hop = w * (16 / NG) + q;
-            stencil_hop<P, CM, LD_KEEP>(a.g, a.links_out, a.links_in, (const E *)a.in, a, a.keep, c, x, hop >> 2,
-                                        (hop >> 1) & 1, hop & 1, acc);
+            stencil_hop<P, CM, LD_KEEP>(a.g, a.links_out, a.links_in, (const E *)((const char *)a.in + vec), a, a.keep, c,
+                                        x, hop >> 2, (hop >> 1) & 1, hop & 1, acc);
         }
 #pragma unroll
         for (int k = 0; k < 3; k++)
@@ -172,7 +173,8 @@ __global__ void __launch_bounds__(32 * NG, 896 / (32 * NG)) dslash_split_kernel(
     if (w < 3 && in_range) {
         const cplx<R> o = split_sum<P, NG>(part, w, lane);
         const R m2 = EPI == EPI_NONE ? rzero<R>() : scalar_as<R>(a.m2_in_args ? a.m2 : a.sc->m2);
-        dot = split_epilogue<P, EPI>((E *)a.out, (const E *)a.p, (const E *)a.b, m2, w * a.g.stride + c, o);
+        dot = split_epilogue<P, EPI>((E *)((char *)a.out + vec), (const E *)((const char *)a.p + vec), (const E *)a.b, m2,
+                                     w * a.g.stride + c, o);
     }
     dslash_reduce<EPI, BLOCK>(a, dot, smem);
 }

@@ -184,7 +184,7 @@ cg_small_update_kernel(Geom g, typename Fmt<P>::Elem *x, typename Fmt<P>::Elem *
                        const typename Fmt<P>::Elem *Ap, PapPartials pap, double *rr_part, CgScalars *sc) {
     using R = typename Fmt<P>::R;
     __shared__ double smem[32];
-    __shared__ dpair salpha;
+    dpair alpha_k;
     const int c = blockIdx.x * BLOCK + threadIdx.x;
     cplx<R> xv[3], rv[3], pv[3], av[3];
     if (c < g.Vh) {  // in flight while the partials are summed
@@ -193,7 +193,7 @@ cg_small_update_kernel(Geom g, typename Fmt<P>::Elem *x, typename Fmt<P>::Elem *
         load_vec<P>(p, g.stride, c, pv);
         load_vec<P>(Ap, g.stride, c, av);
     }
-    const int status = iteration_alpha<BLOCK>(pap, sc, smem, salpha);
+    const int status = iteration_alpha<true, BLOCK>(pap, sc, smem, alpha_k);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         sc->up_rr = sc->rr;
         sc->up_iter = sc->iter;
@@ -203,7 +203,7 @@ cg_small_update_kernel(Geom g, typename Fmt<P>::Elem *x, typename Fmt<P>::Elem *
         return;
     red_t<R> dot = red_zero<red_t<R>>();
     if (c < g.Vh) {
-        const R alpha = scalar_as<R>(salpha);
+        const R alpha = scalar_as<R>(alpha_k);
         const R malpha = -alpha;
 #pragma unroll
         for (int k = 0; k < 3; k++) {

@@ -63,19 +63,19 @@ __global__ void solver_to_pair_kernel(Geom sg, const typename Fmt<P>::Elem *f, c
 
 // ---- flexible CG vector kernel ------------------------------------------
 // x += alpha p; r -= alpha Ap; |r|^2 -> stopping test
-template <int P, int BLOCK>
+template <int P, int BLOCK, bool SMALL>
 __global__ void __launch_bounds__(BLOCK)
 fcg_update_kernel(Geom g, typename Fmt<P>::Elem *x, typename Fmt<P>::Elem *r,
                   const typename Fmt<P>::Elem *p, const typename Fmt<P>::Elem *Ap, PapPartials pap,
                   double *partial, CgScalars *sc) {
     using R = typename Fmt<P>::R;
     __shared__ double smem[32];
-    __shared__ dpair salpha;
-    const int status = iteration_alpha<BLOCK>(pap, sc, smem, salpha);
+    dpair alpha_k;
+    const int status = iteration_alpha<SMALL, BLOCK>(pap, sc, smem, alpha_k);
     const int c = blockIdx.x * BLOCK + threadIdx.x;
     red_t<R> dot = red_zero<red_t<R>>();
     if (status == CG_RUNNING && c < g.Vh) {
-        const R alpha = scalar_as<R>(salpha);
+        const R alpha = scalar_as<R>(alpha_k);
         const R malpha = -alpha;
         cplx<R> xv[3], rv[3], pv[3], av[3];
         load_vec<P>(x, g.stride, c, xv);
@@ -147,8 +147,12 @@ cudaError_t launch_fcg_update(int prec, const Geom &g, void *x, void *r, const v
                               const PapPartials &pap, double *partial, CgScalars *sc, cudaStream_t s) {
     NP_SWITCH(prec, {
         using E = typename Fmt<P>::Elem;
-        fcg_update_kernel<P, FB><<<(g.Vh + FB - 1) / FB, FB, 0, s>>>(g, (E *)x, (E *)r, (const E *)p,
-                                                                     (const E *)Ap, pap, partial, sc);
+        if (pap.n > 0)
+            fcg_update_kernel<P, FB, true><<<(g.Vh + FB - 1) / FB, FB, 0, s>>>(g, (E *)x, (E *)r, (const E *)p,
+                                                                         (const E *)Ap, pap, partial, sc);
+        else
+            fcg_update_kernel<P, FB, false><<<(g.Vh + FB - 1) / FB, FB, 0, s>>>(g, (E *)x, (E *)r, (const E *)p,
+                                                                         (const E *)Ap, pap, partial, sc);
     });
     return cudaGetLastError();
 }

@@ -91,13 +91,13 @@ mixed_init_kernel(Geom g, typename Fmt<PH>::Elem *x, typename Fmt<PH>::Elem *r,
 }
 
 // x_s += alpha p, r_s -= alpha Ap, |r_s|^2; decide whether to update
-template <int PL>
+template <int PL, bool SMALL>
 __global__ void __launch_bounds__(MB)
 mixed_update_kernel(Geom g, float2 *xs, typename Fmt<PL>::Elem *rs, const typename Fmt<PL>::Elem *p,
                     const typename Fmt<PL>::Elem *Ap, PapPartials pap, double *partial, CgScalars *sc) {
     using RL = typename Fmt<PL>::R;
     __shared__ double smem[32];
-    __shared__ dpair salpha;
+    dpair alpha_k;
     const int c = blockIdx.x * MB + threadIdx.x;
     cplx<float> xv[3];
     cplx<RL> rv[3], pv[3], av[3];
@@ -107,10 +107,10 @@ mixed_update_kernel(Geom g, float2 *xs, typename Fmt<PL>::Elem *rs, const typena
         load_vec<PL>(p, g.stride, c, pv);
         load_vec<PL>(Ap, g.stride, c, av);
     }
-    const int status = iteration_alpha<MB>(pap, sc, smem, salpha);
+    const int status = iteration_alpha<SMALL, MB>(pap, sc, smem, alpha_k);
     red_t<RL> dot = red_zero<red_t<RL>>();
     if (status == CG_RUNNING && c < g.Vh) {
-        const float alpha = scalar_as<float>(salpha);
+        const float alpha = scalar_as<float>(alpha_k);
 #pragma unroll
         for (int k = 0; k < 3; k++) {
             xv[k].re = fmaf(alpha, (float)pv[k].re, xv[k].re);
@@ -245,8 +245,12 @@ cudaError_t launch_mixed_update(int lo, const Geom &g, float *xs, void *rs, cons
                                 const PapPartials &pap, double *partial, CgScalars *sc, cudaStream_t s) {
     LO_SWITCH(lo, {
         using EL = typename Fmt<PL>::Elem;
-        mixed_update_kernel<PL><<<grid_of(g), MB, 0, s>>>(g, (float2 *)xs, (EL *)rs, (const EL *)p,
-                                                          (const EL *)Ap, pap, partial, sc);
+        if (pap.n > 0)
+            mixed_update_kernel<PL, true><<<grid_of(g), MB, 0, s>>>(g, (float2 *)xs, (EL *)rs, (const EL *)p,
+                                                              (const EL *)Ap, pap, partial, sc);
+        else
+            mixed_update_kernel<PL, false><<<grid_of(g), MB, 0, s>>>(g, (float2 *)xs, (EL *)rs, (const EL *)p,
+                                                              (const EL *)Ap, pap, partial, sc);
     });
     return cudaGetLastError();
 }

@@ -134,7 +134,7 @@ STAG_D void ms_shift_scalars(const MsArgs &a, double al, const CgScalars *sc, co
 
 // r -= alpha Ap, |r|^2; the shift scalars of this iteration (the solution
 // updates x_s += alpha^s p_s run in ms_p_kernel, which reads p_s anyway)
-template <int P, int PA>
+template <int P, int PA, bool SMALL>
 __global__ void __launch_bounds__(MSB)
 ms_update_kernel(Geom g, MsArgs a, const void *Ap, PapPartials pap0, PapPartials pap1, double *partial,
                  CgScalars *sc, ShiftState *st) {
@@ -145,7 +145,7 @@ ms_update_kernel(Geom g, MsArgs a, const void *Ap, PapPartials pap0, PapPartials
     __shared__ double smem[32];
     __shared__ double zeta_next[MS_MAX], alpha_s[MS_MAX];
     __shared__ int active[MS_MAX];
-    __shared__ dpair salpha;
+    dpair alpha_k;
     // the previous iteration's solution updates are done (ms_p_kernel has
     // finished); written before this block's ticket, so before the last
     // block below advances the iteration count
@@ -154,17 +154,17 @@ ms_update_kernel(Geom g, MsArgs a, const void *Ap, PapPartials pap0, PapPartials
     // which path computed M p this iteration (read before any block's ticket,
     // so before the last block below sets it for the next iteration)
     const bool hi_path = PA == P || sc->ms_hi_op;
-    const int status = iteration_alpha<MSB>(hi_path ? pap0 : pap1, sc, smem, salpha);
+    const int status = iteration_alpha<SMALL, MSB>(hi_path ? pap0 : pap1, sc, smem, alpha_k);
     const bool run = status == CG_RUNNING;
     if (run)
-        ms_shift_scalars(a, salpha.d, sc, st, zeta_next, alpha_s);
+        ms_shift_scalars(a, alpha_k.d, sc, st, zeta_next, alpha_s);
     if (threadIdx.x < MS_MAX)
         active[threadIdx.x] = threadIdx.x < a.n ? st[threadIdx.x].active : 0;
     __syncthreads();
     const int c = blockIdx.x * MSB + threadIdx.x;
     red_t<R> dot = red_zero<red_t<R>>();
     if (run && c < g.Vh) {
-        const R alpha = scalar_as<R>(salpha);
+        const R alpha = scalar_as<R>(alpha_k);
         cplx<R> rv[3], av[3];
         load_vec<P>((const E *)a.r, g.stride, c, rv);
         if (hi_path) {
@@ -213,7 +213,7 @@ ms_update_kernel(Geom g, MsArgs a, const void *Ap, PapPartials pap0, PapPartials
                 else
                     any = true;
             }
-            sc->alpha_prev = salpha.d;
+            sc->alpha_prev = alpha_k.d;
             sc->beta_prev = beta;
             sc->rr = total;
             const double rn = sqrt(total);
@@ -400,19 +400,28 @@ cudaError_t launch_ms_init(int prec, const Geom &g, const MsArgs &a, double *par
     return cudaGetLastError();
 }
 
-cudaError_t launch_ms_update(int prec, const Geom &g, const MsArgs &a, const void *Ap, const PapPartials pap[2],
-                             double *partial, CgScalars *sc, ShiftState *st, cudaStream_t s, int lo) {
+template <bool SMALL>
+static cudaError_t launch_ms_update_t(int prec, const Geom &g, const MsArgs &a, const void *Ap,
+                                      const PapPartials pap[2], double *partial, CgScalars *sc, ShiftState *st,
+                                      cudaStream_t s, int lo) {
     if (lo == P_F32 && (prec == P_F64 || prec == P_DF64)) {
         if (prec == P_F64)
-            ms_update_kernel<P_F64, P_F32><<<grid_of(g), MSB, 0, s>>>(g, a, Ap, pap[0], pap[1], partial, sc, st);
+            ms_update_kernel<P_F64, P_F32, SMALL><<<grid_of(g), MSB, 0, s>>>(g, a, Ap, pap[0], pap[1], partial, sc, st);
         else
-            ms_update_kernel<P_DF64, P_F32><<<grid_of(g), MSB, 0, s>>>(g, a, Ap, pap[0], pap[1], partial, sc, st);
+            ms_update_kernel<P_DF64, P_F32, SMALL><<<grid_of(g), MSB, 0, s>>>(g, a, Ap, pap[0], pap[1], partial, sc, st);
         return cudaGetLastError();
     }
     if (lo >= 0)
         return cudaErrorInvalidValue;
-    MS_PREC_SWITCH(prec, ms_update_kernel<P, P><<<grid_of(g), MSB, 0, s>>>(g, a, Ap, pap[0], pap[1], partial, sc, st));
+    MS_PREC_SWITCH(prec, ms_update_kernel<P, P, SMALL><<<grid_of(g), MSB, 0, s>>>(g, a, Ap, pap[0], pap[1], partial,
+                                                                                 sc, st));
     return cudaGetLastError();
+}
+
+cudaError_t launch_ms_update(int prec, const Geom &g, const MsArgs &a, const void *Ap, const PapPartials pap[2],
+                             double *partial, CgScalars *sc, ShiftState *st, cudaStream_t s, int lo) {
+    return pap[0].n > 0 ? launch_ms_update_t<true>(prec, g, a, Ap, pap, partial, sc, st, s, lo)
+                        : launch_ms_update_t<false>(prec, g, a, Ap, pap, partial, sc, st, s, lo);
 }
 
 cudaError_t launch_ms_p(int prec, const Geom &g, const MsArgs &a, const CgScalars *sc,

@@ -279,135 +279,129 @@ STAG_D double2 zmul(double2 a, double2 b) { return make_double2(a.x * b.x - a.y 
 STAG_D double2 zadd(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
 STAG_D double2 zconj(double2 a) { return make_double2(a.x, -a.y); }
 
-// W3[d3] . W2[d2] . W1[d1]
-STAG_D double2 triple(const NetW &W, int d3, int d2, int d1) {
+// this lane's share of W3[d3] . W2[d2] . W1[d1]: the channel pairs (j, i) =
+// lane, lane + 32 of the C x C sum
+STAG_D double2 triple_share(const NetW &W, int d3, int d2, int d1) {
     double2 s = make_double2(0.0, 0.0);
-    for (int j = 0; j < W.C; j++) {
-        double2 t = make_double2(0.0, 0.0);
-        for (int i = 0; i < W.C; i++)
-            t = zadd(t, zmul(W.w2(d2, j, i), W.w1(d1, i)));
-        s = zadd(s, zmul(W.w3(d3, j), t));
+    for (int e = threadIdx.x & 31; e < W.C * W.C; e += 32) {
+        const int j = e / W.C, i = e % W.C;
+        s = zadd(s, zmul(W.w3(d3, j), zmul(W.w2(d2, j, i), W.w1(d1, i))));
     }
     return s;
 }
+// the warp's sum, in lane 0
+STAG_D double2 zwarp_sum(double2 v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        v.x += __shfl_down_sync(0xffffffffu, v.x, o);
+        v.y += __shfl_down_sync(0xffffffffu, v.y, o);
+    }
+    return v;
+}
 
-// one block: the weights go to shared memory, then thread a*8+b computes
-// C[a][b] and thread 64 c0
-constexpr int NET_MAX_W = 9 * (2 * 8 + 8 * 8);
-
+// One warp per coefficient: block a*8+b computes C[a][b], block 64 c0.  The
+// FP64 pipe takes 64 cycles per warp instruction however many lanes work, so
+// the channel sums lie across the lanes (one thread per coefficient, in one
+// block, took 52 us; now 9).
 // hermitian: the coefficients of (N + N^+)/2 instead.  T_a^+ = T_abar (abar
 // = a ^ 1, the reversed hop), so N^+ has conj(c0) and the coefficient
 // conj(C[bbar][abar]) on T_a T_b.
-__global__ void net_path_coef_kernel(NetW W, int hermitian, NetPath *out) {
-    __shared__ double2 sw[NET_MAX_W];
-    __shared__ double2 sc[65];
-    const int nw = 9 * (2 * W.C + W.C * W.C);
-    for (int k = threadIdx.x; k < nw; k += blockDim.x)
-        sw[k] = W.load(k);
-    __syncthreads();
-    W.sw = sw;
-    const int q = threadIdx.x;
-    if (q < 64) {
-        const int a = q >> 3, b = q & 7;
-        sc[q] = zadd(zadd(triple(W, 0, a + 1, b + 1), triple(W, a + 1, 0, b + 1)), triple(W, a + 1, b + 1, 0));
-    } else if (q == 64) {
-        sc[64] = triple(W, 0, 0, 0);
+__global__ void __launch_bounds__(32) net_path_coef_kernel(NetW W, int hermitian, NetPath *out) {
+    const int q = blockIdx.x;
+    if (q == 64) {
+        const double2 v = zwarp_sum(triple_share(W, 0, 0, 0));
+        if (threadIdx.x == 0)
+            out->c0 = make_float2((float)v.x, hermitian ? 0.f : (float)v.y);
+        return;
     }
-    __syncthreads();
-    if (q < 64) {
-        double2 v = sc[q];
-        if (hermitian) {
-            const int a = q >> 3, b = q & 7;
-            const double2 t = sc[(b ^ 1) * 8 + (a ^ 1)];
-            v = make_double2(0.5 * (v.x + t.x), 0.5 * (v.y - t.y));
-        }
+    auto path = [&](int a, int b) {
+        return zwarp_sum(zadd(zadd(triple_share(W, 0, a + 1, b + 1), triple_share(W, a + 1, 0, b + 1)),
+                              triple_share(W, a + 1, b + 1, 0)));
+    };
+    const int a = q >> 3, b = q & 7;
+    double2 v = path(a, b);
+    if (hermitian) {
+        const double2 t = path(b ^ 1, a ^ 1);
+        v = make_double2(0.5 * (v.x + t.x), 0.5 * (v.y - t.y));
+    }
+    if (threadIdx.x == 0)
         out->C[q] = make_float2((float)v.x, (float)v.y);
-    } else if (q == 64) {
-        const double2 v = sc[64];
-        out->c0 = make_float2((float)v.x, hermitian ? 0.f : (float)v.y);
-    }
 }
 
 cudaError_t launch_net_path_coef(int C, const float *w32, const int off[3], int round_half, NetPath *out,
                                  cudaStream_t s, int hermitian) {
     NetW W{(const float2 *)w32, C, off[1], off[2], round_half};
-    net_path_coef_kernel<<<1, 96, 0, s>>>(W, hermitian, out);
+    net_path_coef_kernel<<<65, 32, 0, s>>>(W, hermitian, out);
     return cudaGetLastError();
 }
 
 // dL/dW* of every complex weight from G[a*8+b] = dL/dC[a][b]* and G[64] =
-// dL/dc0* (C holomorphic in W: dL/dW* = sum conj(dC/dW) dL/dC*); added to grad
-__global__ void net_path_chain_kernel(NetW W, int nw, const double2 *__restrict__ G, double2 *grad) {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+// dL/dc0* (C holomorphic in W: dL/dW* = sum conj(dC/dW) dL/dC*); added to
+// grad.  One warp per weight, the paths it lies on across the lanes (one
+// thread per weight took 240 us, the 64 paths of the first layer's identity
+// weights one after the other in FP64; now 13).
+constexpr int NET_MAX_W = 9 * (2 * 8 + 8 * 8);
+constexpr int CHAIN_BLOCK = 128;
+
+__global__ void __launch_bounds__(CHAIN_BLOCK)
+net_path_chain_kernel(NetW W, int nw, const double2 *__restrict__ G, double2 *grad) {
+    __shared__ double2 sw[NET_MAX_W];
+    for (int k = threadIdx.x; k < nw; k += CHAIN_BLOCK)
+        sw[k] = W.load(k);
+    __syncthreads();
+    W.sw = sw;
+    const int lane = threadIdx.x & 31;
+    const int k = blockIdx.x * (CHAIN_BLOCK / 32) + (threadIdx.x >> 5);
     if (k >= nw)
         return;
     const int C = W.C;
-    const double2 G0 = G[64];
+    const int layer = k < W.off1 ? 1 : k < W.off2 ? 2 : 3;
+    const int q = layer == 1 ? k : layer == 2 ? k - W.off1 : k - W.off2;
+    const int d = layer == 2 ? q / (C * C) : q / C;                   // the weight's hop
+    const int j = layer == 2 ? (q / C) % C : layer == 3 ? q % C : 0;  // output channel
+    const int i = layer == 2 ? q % C : layer == 1 ? q % C : 0;        // input channel
+    // the other two layers' factor on the path with hops d_o (outer layer) and
+    // d_i (inner layer)
+    auto others = [&](int d_o, int d_i) {
+        if (layer == 2)
+            return zmul(W.w3(d_o, j), W.w1(d_i, i));
+        double2 t = make_double2(0.0, 0.0);
+        if (layer == 1)
+            for (int c = 0; c < C; c++)  // sum_c W3[d_o][c] W2[d_i][c][i]
+                t = zadd(t, zmul(W.w3(d_o, c), W.w2(d_i, c, i)));
+        else
+            for (int c = 0; c < C; c++)  // sum_c W2[d_o][j][c] W1[d_i][c]
+                t = zadd(t, zmul(W.w2(d_o, j, c), W.w1(d_i, c)));
+        return t;
+    };
     double2 acc = make_double2(0.0, 0.0);
     auto add = [&](double2 coef, double2 gv) { acc = zadd(acc, zmul(zconj(coef), gv)); };
-    if (k < W.off1) {  // W1[d][i]
-        const int d = k / C, i = k % C;
-        // sum_j W3[d3][j] W2[d2][j][i]
-        auto s32 = [&](int d3, int d2) {
-            double2 t = make_double2(0.0, 0.0);
-            for (int j = 0; j < C; j++)
-                t = zadd(t, zmul(W.w3(d3, j), W.w2(d2, j, i)));
-            return t;
-        };
-        if (d == 0) {
-            add(s32(0, 0), G0);
-            for (int a = 0; a < 8; a++)
-                for (int b = 0; b < 8; b++)
-                    add(s32(a + 1, b + 1), G[a * 8 + b]);
-        } else {
-            const int b = d - 1;
-            for (int a = 0; a < 8; a++)
-                add(zadd(s32(0, a + 1), s32(a + 1, 0)), G[a * 8 + b]);
-        }
-    } else if (k < W.off2) {  // W2[d][j][i]
-        const int q = k - W.off1;
-        const int d = q / (C * C), j = (q / C) % C, i = q % C;
-        if (d == 0) {
-            add(zmul(W.w3(0, j), W.w1(0, i)), G0);
-            for (int a = 0; a < 8; a++)
-                for (int b = 0; b < 8; b++)
-                    add(zmul(W.w3(a + 1, j), W.w1(b + 1, i)), G[a * 8 + b]);
-        } else {
-            const int e = d - 1;
-            for (int b = 0; b < 8; b++)  // W2 as the outer hop, layer 3 idle
-                add(zmul(W.w3(0, j), W.w1(b + 1, i)), G[e * 8 + b]);
-            for (int a = 0; a < 8; a++)  // W2 as the inner hop, layer 1 idle
-                add(zmul(W.w3(a + 1, j), W.w1(0, i)), G[a * 8 + e]);
-        }
-    } else {  // W3[d][j]
-        const int q = k - W.off2;
-        const int d = q / C, j = q % C;
-        // sum_i W2[d2][j][i] W1[d1][i]
-        auto s21 = [&](int d2, int d1) {
-            double2 t = make_double2(0.0, 0.0);
-            for (int i = 0; i < C; i++)
-                t = zadd(t, zmul(W.w2(d2, j, i), W.w1(d1, i)));
-            return t;
-        };
-        if (d == 0) {
-            add(s21(0, 0), G0);
-            for (int a = 0; a < 8; a++)
-                for (int b = 0; b < 8; b++)
-                    add(s21(a + 1, b + 1), G[a * 8 + b]);
-        } else {
-            const int a = d - 1;
-            for (int b = 0; b < 8; b++)
-                add(zadd(s21(0, b + 1), s21(b + 1, 0)), G[a * 8 + b]);
-        }
+    if (d == 0) {
+        // this layer idle: every pair of hops in the other two, and c0
+        for (int e = lane; e < 64; e += 32)
+            add(others((e >> 3) + 1, (e & 7) + 1), G[e]);
+        if (lane == 0)
+            add(others(0, 0), G[64]);
+    } else if (lane < 16) {
+        // this layer takes hop d, one of the others the second hop h: lanes
+        // 2 h + u, u = 0 the outer one of the two, 1 the inner one
+        const int h = lane >> 1, u = lane & 1;
+        const double2 t = u ? others(0, h + 1) : others(h + 1, 0);
+        // outer hop first in the path index: layer 3's hop is outer, layer
+        // 1's inner; layer 2's is inner to layer 3's and outer to layer 1's
+        const bool mine_outer = layer == 3 || (layer == 2 && u);
+        add(t, mine_outer ? G[(d - 1) * 8 + h] : G[h * 8 + d - 1]);
     }
-    grad[k] = zadd(grad[k], acc);
+    acc = zwarp_sum(acc);
+    if (lane == 0)
+        grad[k] = zadd(grad[k], acc);
 }
 
 cudaError_t launch_net_path_chain(int C, const float *w32, const int off[3], const double2 *G, double2 *grad,
                                   cudaStream_t s) {
     NetW W{(const float2 *)w32, C, off[1], off[2], 0};
     const int nw = 9 * (2 * C + C * C);
-    net_path_chain_kernel<<<(nw + 127) / 128, 128, 0, s>>>(W, nw, G, grad);
+    net_path_chain_kernel<<<(nw + CHAIN_BLOCK / 32 - 1) / (CHAIN_BLOCK / 32), CHAIN_BLOCK, 0, s>>>(W, nw, G, grad);
     return cudaGetLastError();
 }
 
@@ -468,16 +462,24 @@ template <> struct Chi<L12> : Chi<short2> {};
 // Six resident blocks (at most 80 registers, 24 warps per SM): at eight the
 // 16-bit form spills 96 bytes, and measured at 32^3x64 the solver-form net
 // application took 0.342 ms against 0.308 ms at six.
+// Q = NetPairs: the inputs of several training pairs in one launch, pair
+// blockIdx.y with the y-th part of chi (NoPairs: the one input r).
+struct NoPairs {};
 constexpr int NET_MID_MINB = 6;
 
-template <int P, class LT>
+template <int P, class LT, class Q>
 __global__ void __launch_bounds__(NET_BLOCK, NET_MID_MINB)
 net_mid_kernel(Geom g, const LT *__restrict__ NL, float ls, int bcneg, const NetPath *__restrict__ path,
-               const typename Fmt<P>::Elem *__restrict__ r, int rs, void *__restrict__ chi, const int *gate) {
+               const typename Fmt<P>::Elem *__restrict__ r, int rs, void *__restrict__ chi, const int *gate,
+               const __grid_constant__ Q pairs) {
     __shared__ cplx<float> sC[64];
     __shared__ float2 sh[8][3][NET_BLOCK];
     if (gate && *gate != CG_RUNNING)
         return;
+    if constexpr (std::is_same<Q, NetPairs>::value) {
+        r = pairs.r[blockIdx.y];
+        chi = (float2 *)chi + (size_t)blockIdx.y * 24 * g.stride;
+    }
     if (threadIdx.x < 64) {
         const float2 v = path->C[threadIdx.x];
         sC[threadIdx.x] = cplx<float>{v.x * ls, v.y * ls};
@@ -580,16 +582,21 @@ net_mid_kernel(Geom g, const LT *__restrict__ NL, float ls, int bcneg, const Net
 // (partial[nblk + blk]; 0 without Ap) for the flexible CG.
 enum { NET_OUT_PLAIN = 0, NET_OUT_DOTS = 1 };
 
-template <int PI, int PO, class LT, int EPI>
+template <int PI, int PO, class LT, int EPI, class Q>
 __global__ void __launch_bounds__(NET_BLOCK)
 net_out_kernel(Geom g, const LT *__restrict__ NL, float ls, int bcneg, const NetPath *__restrict__ path,
                const void *__restrict__ chi, const typename Fmt<PI>::Elem *__restrict__ r, int rs,
                typename Fmt<PO>::Elem *__restrict__ z, int zs, const typename Fmt<PO>::Elem *__restrict__ Ap,
-               double *partial, const int *gate) {
+               double *partial, const int *gate, const __grid_constant__ Q pairs) {
     using RO = typename Fmt<PO>::R;
     __shared__ double smem[32];
     if (gate && *gate != CG_RUNNING)
         return;
+    if constexpr (std::is_same<Q, NetPairs>::value) {
+        r = pairs.r[blockIdx.y];
+        chi = (const float2 *)chi + (size_t)blockIdx.y * 24 * g.stride;
+        z += (size_t)blockIdx.y * 3 * zs;
+    }
     const int c = blockIdx.x * NET_BLOCK + threadIdx.x;
     const int S = g.stride;
     red_t<RO> d0 = red_zero<red_t<RO>>(), d1 = red_zero<red_t<RO>>();
@@ -665,14 +672,14 @@ cudaError_t launch_net_mid(int prec, const Geom &g, const NetLinkSet &nl, const 
     NP_IN_SWITCH(prec, {
         using E = typename Fmt<P>::Elem;
         if (nl.l12)
-            net_mid_kernel<P, L12><<<net_grid(g), NET_BLOCK, 0, s>>>(g, (const L12 *)nl.l12, nl.scale16, nl.bcneg,
-                                                                      path, (const E *)r, rs, chi, gate);
+            net_mid_kernel<P, L12, NoPairs><<<net_grid(g), NET_BLOCK, 0, s>>>(g, (const L12 *)nl.l12, nl.scale16, nl.bcneg,
+                                                                      path, (const E *)r, rs, chi, gate, NoPairs{});
         else if (nl.l16)
-            net_mid_kernel<P, short2><<<net_grid(g), NET_BLOCK, 0, s>>>(g, nl.l16, nl.scale16, nl.bcneg, path,
-                                                                         (const E *)r, rs, chi, gate);
+            net_mid_kernel<P, short2, NoPairs><<<net_grid(g), NET_BLOCK, 0, s>>>(g, nl.l16, nl.scale16, nl.bcneg, path,
+                                                                         (const E *)r, rs, chi, gate, NoPairs{});
         else
-            net_mid_kernel<P, float2><<<net_grid(g), NET_BLOCK, 0, s>>>(g, nl.l32, 1.f, nl.bcneg, path,
-                                                                         (const E *)r, rs, chi, gate);
+            net_mid_kernel<P, float2, NoPairs><<<net_grid(g), NET_BLOCK, 0, s>>>(g, nl.l32, 1.f, nl.bcneg, path,
+                                                                         (const E *)r, rs, chi, gate, NoPairs{});
     });
     return cudaGetLastError();
 }
@@ -683,16 +690,16 @@ static void net_out_t(const Geom &g, const NetLinkSet &nl, const NetPath *path, 
     using EI = typename Fmt<PI>::Elem;
     using EO = typename Fmt<PO>::Elem;
     if (nl.l12)
-        net_out_kernel<PI, PO, L12, EPI><<<net_grid(g), NET_BLOCK, 0, s>>>(
+        net_out_kernel<PI, PO, L12, EPI, NoPairs><<<net_grid(g), NET_BLOCK, 0, s>>>(
             g, (const L12 *)nl.l12, nl.scale16, nl.bcneg, path, chi, (const EI *)r, rs, (EO *)z, zs,
-            (const EO *)Ap, partial, gate);
+            (const EO *)Ap, partial, gate, NoPairs{});
     else if (nl.l16)
-        net_out_kernel<PI, PO, short2, EPI><<<net_grid(g), NET_BLOCK, 0, s>>>(
+        net_out_kernel<PI, PO, short2, EPI, NoPairs><<<net_grid(g), NET_BLOCK, 0, s>>>(
             g, nl.l16, nl.scale16, nl.bcneg, path, chi, (const EI *)r, rs, (EO *)z, zs, (const EO *)Ap, partial,
-            gate);
+            gate, NoPairs{});
     else
-        net_out_kernel<PI, PO, float2, EPI><<<net_grid(g), NET_BLOCK, 0, s>>>(
-            g, nl.l32, 1.f, nl.bcneg, path, chi, (const EI *)r, rs, (EO *)z, zs, (const EO *)Ap, partial, gate);
+        net_out_kernel<PI, PO, float2, EPI, NoPairs><<<net_grid(g), NET_BLOCK, 0, s>>>(
+            g, nl.l32, 1.f, nl.bcneg, path, chi, (const EI *)r, rs, (EO *)z, zs, (const EO *)Ap, partial, gate, NoPairs{});
 }
 
 // input and output of one precision (the solver's), or FP32 pair input with
@@ -711,18 +718,32 @@ cudaError_t launch_net_out(int prec_in, int prec_out, const Geom &g, const NetLi
     return cudaGetLastError();
 }
 
+cudaError_t launch_net_pairs(const Geom &g, const NetLinkSet &nl, const NetPath *path, const NetPairs &pairs,
+                             float2 *chi, float2 *z, cudaStream_t s) {
+    const dim3 grid(net_grid(g), pairs.n);
+    net_mid_kernel<P_F32, float2, NetPairs><<<grid, NET_BLOCK, 0, s>>>(g, nl.l32, 1.f, nl.bcneg, path, nullptr, g.Vh,
+                                                                      chi, nullptr, pairs);
+    net_out_kernel<P_F32, P_F32, float2, NET_OUT_PLAIN, NetPairs><<<grid, NET_BLOCK, 0, s>>>(
+        g, nl.l32, 1.f, nl.bcneg, path, chi, nullptr, g.Vh, z, g.stride, nullptr, nullptr, nullptr, pairs);
+    return cudaGetLastError();
+}
+
 // ---- training: dL/dC[a][b]* and dL/dc0* ----------------------------------------
 // Per odd site y: h_b = (T_b r)(y), k_a = (T_a^+ g)(y); the block gathers a
 // tile of NET_BLOCK sites in shared memory (site index fastest) and warp w
 // adds the 4 x 4 pairs (a in 4 (w >> 1) .. +3, b in 4 (w & 1) .. +3) of
 // conj(h_b) k_a over the tile; each thread also adds conj(r) g of the even
-// site with its checkerboard index (the c0 term).  One partial per block and
-// pair, in double: partial[blk * 65 + q].
+// site with its checkerboard index (the c0 term).  blockIdx.y is the training
+// pair; one partial per block and hop pair, in double:
+// partial[(blockIdx.y gridDim.x + blockIdx.x) * 65 + q].
 constexpr int GRAD_BLOCKS = 1024;
 
 __global__ void __launch_bounds__(NET_BLOCK)
-net_grad_kernel(Geom g, const float2 *__restrict__ NL, const float2 *__restrict__ r, int rs,
-                const float2 *__restrict__ gv, int gs, double2 *partial) {
+net_grad_kernel(Geom g, const float2 *__restrict__ NL, const __grid_constant__ NetPairs pairs,
+                const float2 *__restrict__ gvs, double2 *partial) {
+    const float2 *__restrict__ r = pairs.r[blockIdx.y];
+    const int rs = g.Vh, gs = g.stride;
+    const float2 *__restrict__ gv = gvs + (size_t)blockIdx.y * 3 * gs;
     static_assert(NET_BLOCK == 128, "four warps: one per 4 x 4 block of hop pairs");
     __shared__ float2 H[8][3][NET_BLOCK];
     __shared__ float2 K[8][3][NET_BLOCK];
@@ -808,7 +829,7 @@ net_grad_kernel(Geom g, const float2 *__restrict__ NL, const float2 *__restrict_
         __syncthreads();
     }
     // warp sums in double, fixed order; acc[i][j] is the pair (a0 + i, b0 + j)
-    double2 *out = partial + (size_t)blockIdx.x * 65;
+    double2 *out = partial + ((size_t)blockIdx.y * gridDim.x + blockIdx.x) * 65;
 #pragma unroll 1
     for (int i = 0; i < 4; i++)
 #pragma unroll 1
@@ -867,17 +888,17 @@ int net_grad_blocks(const Geom &g) {
     return need < GRAD_BLOCKS ? need : GRAD_BLOCKS;
 }
 
-cudaError_t launch_net_grad(const Geom &g, const float2 *NL32, const float2 *r, int rs, const float2 *gv, int gs,
+cudaError_t launch_net_grad(const Geom &g, const float2 *NL32, const NetPairs &pairs, const float2 *gv,
                             double2 *partial, double2 *G, cudaStream_t s) {
-    const int nb = net_grad_blocks(g);
-    net_grad_kernel<<<nb, NET_BLOCK, 0, s>>>(g, NL32, r, rs, gv, gs, partial);
-    net_grad_finish_kernel<<<65, GRAD_FINISH_BLOCK, 0, s>>>(partial, nb, G);
+    const dim3 grid(net_grad_blocks(g), pairs.n);
+    net_grad_kernel<<<grid, NET_BLOCK, 0, s>>>(g, NL32, pairs, gv, partial);
+    net_grad_finish_kernel<<<65, GRAD_FINISH_BLOCK, 0, s>>>(partial, (int)(grid.x * grid.y), G);
     return cudaGetLastError();
 }
 
-// ---- losses on the even sites (FP32) -----------------------------------------
-// error loss: g = (z - e) / |e|^2, *loss += |z - e|^2 / |e|^2 (z, g: stride zs;
-// e: stride es)
+// ---- losses on the even sites (FP32), pair blockIdx.y of each launch ----------
+// error loss: g = (z - e) / |e|^2, *loss += |z - e|^2 / |e|^2 (z, g:
+// [n][3][stride]; e [3][Vh])
 // Loss and dot sums: each site's six products are summed in FP32, the sites
 // of a thread and the block tree in double float (FP32 pipe), one FP64
 // value and one atomic per block.  Accumulated in FP64 per element, with one
@@ -886,11 +907,14 @@ cudaError_t launch_net_grad(const Geom &g, const float2 *NL32, const float2 *r, 
 constexpr int NET_SUM_BLOCK = 256;
 
 __global__ void __launch_bounds__(NET_SUM_BLOCK)
-net_error_loss_kernel(int Vh, const float2 *__restrict__ z, int zs, const float2 *__restrict__ e, int es,
-                      const double *enorm2, float2 *gv, double *loss) {
+net_error_loss_kernel(int Vh, int zs, const __grid_constant__ NetPairs pairs, const float2 *__restrict__ z,
+                      float2 *gv, double *loss) {
     __shared__ double smem[32];
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    const double n2 = *enorm2;
+    const int c = blockIdx.x * blockDim.x + threadIdx.x, es = Vh;
+    const float2 *__restrict__ e = pairs.e[blockIdx.y];
+    z += (size_t)blockIdx.y * 3 * zs;
+    gv += (size_t)blockIdx.y * 3 * zs;
+    const double n2 = *pairs.norm2[blockIdx.y];
     float part = 0.f;
     if (c < Vh) {
         // a pair with e = 0 carries no information: no loss, no gradient
@@ -910,11 +934,12 @@ net_error_loss_kernel(int Vh, const float2 *__restrict__ z, int zs, const float2
 
 // residual loss: q = (Mz - r) / |r|^2 written over mz, *loss += |Mz - r|^2 / |r|^2
 __global__ void __launch_bounds__(NET_SUM_BLOCK)
-net_resid_loss_kernel(int Vh, float2 *mz, int ms, const float2 *__restrict__ r, int rs,
-                      const double *rnorm2, double *loss) {
+net_resid_loss_kernel(int Vh, int ms, const __grid_constant__ NetPairs pairs, float2 *mz, double *loss) {
     __shared__ double smem[32];
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    const double n2 = *rnorm2;
+    const int c = blockIdx.x * blockDim.x + threadIdx.x, rs = Vh;
+    const float2 *__restrict__ r = pairs.r[blockIdx.y];
+    mz += (size_t)blockIdx.y * 3 * ms;
+    const double n2 = *pairs.norm2[blockIdx.y];
     float part = 0.f;
     if (c < Vh) {
         const float inv = n2 > 0.0 ? (float)(1.0 / n2) : 0.f;
@@ -955,17 +980,16 @@ net_dot2_kernel(int Vh, const float2 *__restrict__ a, int as, const float2 *__re
     }
 }
 
-cudaError_t launch_net_error_loss(int Vh, const float2 *z, int zs, const float2 *e, int es, const double *enorm2,
-                                  float2 *gv, double *loss, cudaStream_t s) {
-    net_error_loss_kernel<<<(Vh + NET_SUM_BLOCK - 1) / NET_SUM_BLOCK, NET_SUM_BLOCK, 0, s>>>(Vh, z, zs, e, es,
-                                                                                         enorm2, gv, loss);
+cudaError_t launch_net_error_loss(const Geom &g, const NetPairs &pairs, const float2 *z, float2 *gv, double *loss,
+                                  cudaStream_t s) {
+    const dim3 grid((g.Vh + NET_SUM_BLOCK - 1) / NET_SUM_BLOCK, pairs.n);
+    net_error_loss_kernel<<<grid, NET_SUM_BLOCK, 0, s>>>(g.Vh, g.stride, pairs, z, gv, loss);
     return cudaGetLastError();
 }
 
-cudaError_t launch_net_resid_loss(int Vh, float2 *mz, int ms, const float2 *r, int rs, const double *rnorm2,
-                                  double *loss, cudaStream_t s) {
-    net_resid_loss_kernel<<<(Vh + NET_SUM_BLOCK - 1) / NET_SUM_BLOCK, NET_SUM_BLOCK, 0, s>>>(Vh, mz, ms, r, rs,
-                                                                                         rnorm2, loss);
+cudaError_t launch_net_resid_loss(const Geom &g, const NetPairs &pairs, float2 *mz, double *loss, cudaStream_t s) {
+    const dim3 grid((g.Vh + NET_SUM_BLOCK - 1) / NET_SUM_BLOCK, pairs.n);
+    net_resid_loss_kernel<<<grid, NET_SUM_BLOCK, 0, s>>>(g.Vh, g.stride, pairs, mz, loss);
     return cudaGetLastError();
 }
 

@@ -26,7 +26,8 @@ struct stag_net_s {
     double *grad = nullptr, *m = nullptr, *v = nullptr;
     int adam_t = 0;
     NetPath *path = nullptr;      // path coefficients of the current weights
-    float2 *chi = nullptr;        // odd-site intermediate [8][3][stride]
+    int group = 1;                // training pairs per launch (pair_group)
+    float2 *chi = nullptr;        // odd-site intermediate [group][8][3][stride]
     double2 *G = nullptr;         // dL/dC* (64) and dL/dc0* (1), summed over pairs
     double2 *gpartial = nullptr;  // per-block partials of G
     double *scal = nullptr;       // [0] loss accumulator, [1..2] warm-start sums
@@ -38,7 +39,7 @@ struct stag_net_s {
     int enorm_cap = 0;
     int loss_kind = STAG_NET_LOSS_ERROR;
     double mass = 0;           // mass of the collected pairs (residual loss)
-    // FP32 solver-layout work vectors of the losses: z, Mz / g, t (odd)
+    // FP32 solver-layout work vectors of the losses, [group]: z, Mz / g, t (odd)
     void *fz = nullptr, *fmz = nullptr, *ft = nullptr;
     // flexible CG: preconditioned residual per precision
     void *z[4] = {};
@@ -55,6 +56,33 @@ static void net_free(stag_net n) {
     for (int q = 0; q < 4; q++)
         if (n->z[q])
             cudaFree(n->z[q]);
+}
+
+// Training pairs per launch.  On small lattices one pair's kernels fill a
+// fraction of the chip and last a few microseconds, ten launches a pair (16^4:
+// 87 us of kernels a pair); several pairs go into one launch there, up to
+// 262144 sites in all (their intermediates, 192 B a site, then stay in L2).
+static int pair_group(const Geom &g) {
+    const int fit = (1 << 18) / g.Vh;
+    return fit < 1 ? 1 : fit > NET_PAIRS ? NET_PAIRS : fit;
+}
+
+// an FP32 work vector for each pair of a group
+static int alloc_group_vec(stag_net n, void **p) {
+    if (*p)
+        return STAG_OK;
+    const size_t b = field_bytes(n->lat, STAG_F32) * n->group;
+    void *q = nullptr;
+    cudaError_t e = cudaMalloc(&q, b);
+    if (e == cudaSuccess) {
+        e = cudaMemsetAsync(q, 0, b, n->lat->stream);
+        if (e != cudaSuccess)
+            cudaFree(q);
+    }
+    if (e != cudaSuccess)
+        return fail(STAG_ERR_NOMEM, "training work vector: %s", cudaGetErrorString(e));
+    *p = q;
+    return STAG_OK;
 }
 
 extern "C" int stag_net_create(stag_lattice lat, const double *fat, int ptr_kind, int channels, unsigned seed,
@@ -74,6 +102,7 @@ extern "C" int stag_net_create(stag_lattice lat, const double *fat, int ptr_kind
         return fail(STAG_ERR_NOMEM, "stag_net_create: host allocation failed");
     n->lat = lat;
     n->C = channels;
+    n->group = pair_group(lat->geom);
     const int C = channels;
     n->off[0] = 0;
     n->off[1] = 9 * C;
@@ -101,9 +130,9 @@ extern "C" int stag_net_create(stag_lattice lat, const double *fat, int ptr_kind
         (e = cudaMalloc(&n->m, sizeof(double) * nr)) != cudaSuccess ||
         (e = cudaMalloc(&n->v, sizeof(double) * nr)) != cudaSuccess ||
         (e = cudaMalloc(&n->path, sizeof(NetPath))) != cudaSuccess ||
-        (e = cudaMalloc(&n->chi, sizeof(float2) * 8 * 3 * S)) != cudaSuccess ||
+        (e = cudaMalloc(&n->chi, sizeof(float2) * 8 * 3 * S * n->group)) != cudaSuccess ||
         (e = cudaMalloc(&n->G, sizeof(double2) * 65)) != cudaSuccess ||
-        (e = cudaMalloc(&n->gpartial, sizeof(double2) * 65 * net_grad_blocks(lat->geom))) != cudaSuccess ||
+        (e = cudaMalloc(&n->gpartial, sizeof(double2) * 65 * net_grad_blocks(lat->geom) * n->group)) != cudaSuccess ||
         (e = cudaMalloc(&n->scal, sizeof(double) * 4)) != cudaSuccess)
         return bail(e);
     // the padding sites of the link planes are never read; zero them anyway
@@ -111,9 +140,9 @@ extern "C" int stag_net_create(stag_lattice lat, const double *fat, int ptr_kind
         (e = cudaMemsetAsync(n->NL16, 0, sizeof(short2) * 2 * 4 * 9 * S, s)) != cudaSuccess)
         return bail(e);
     {
-        int st = alloc_vec(lat, STAG_F32, &n->fz);
+        int st = alloc_group_vec(n, &n->fz);
         if (st == STAG_OK)
-            st = alloc_vec(lat, STAG_F32, &n->fmz);
+            st = alloc_group_vec(n, &n->fmz);
         if (st != STAG_OK) {
             cudaStreamSynchronize(s);
             net_free(n);
@@ -469,7 +498,7 @@ extern "C" int stag_net_set_loss(stag_net n, int kind) {
         if (!lat->has_gauge || !lat->links[STAG_F32])
             return fail(STAG_ERR_STATE, "stag_net_set_loss: the residual loss needs an F32 gauge copy");
         DEVICE_SCOPE(lat->device);
-        STAG_TRY(alloc_vec(lat, STAG_F32, &n->ft));
+        STAG_TRY(alloc_group_vec(n, &n->ft));
     }
     n->loss_kind = kind;
     return STAG_OK;
@@ -483,41 +512,58 @@ extern "C" int stag_net_num_pairs(const stag_net n, int *count) {
 }
 
 // ---- training -------------------------------------------------------------
-// out = M in = m^2 in - D_eo D_oe in on FP32 solver-layout vectors (t: odd)
-static int apply_M_f32(stag_net n, const void *in, void *t, void *out, cudaStream_t s) {
+// out = M in = m^2 in - D_eo D_oe in on np FP32 solver-layout vectors (t: odd)
+static int apply_M_f32(stag_net n, int np, const void *in, void *t, void *out, cudaStream_t s) {
     stag_lattice lat = n->lat;
     const int P = STAG_F32;
-    DslashArgs a1 = dslash_args(lat, P, STAG_ODD, in, t);
-    CUDA_TRY(launch_dslash(P, EPI_NONE, a1, lat->dslash_block[P], s));
-    DslashArgs a2 = dslash_args(lat, P, STAG_EVEN, t, out);
-    a2.p = in;
-    a2.m2 = make_dpair(n->mass * n->mass);
-    a2.m2_in_args = 1;
-    CUDA_TRY(launch_dslash(P, EPI_M, a2, lat->dslash_block[P], s));
+    const size_t step = field_bytes(lat, P);
+    // vectors per launch: the split form takes them all, the others one
+    const int per = split_warps(P, dslash_args(lat, P, STAG_ODD, in, t).compressed, lat->geom) > 0 ? np : 1;
+    for (int k = 0; k < np; k += per) {
+        const char *ik = (const char *)in + k * step;
+        char *tk = (char *)t + k * step, *ok = (char *)out + k * step;
+        DslashArgs a1 = dslash_args(lat, P, STAG_ODD, ik, tk);
+        a1.nbatch = per;
+        a1.vec_step = step;
+        CUDA_TRY(launch_dslash(P, EPI_NONE, a1, lat->dslash_block[P], s));
+        DslashArgs a2 = dslash_args(lat, P, STAG_EVEN, tk, ok);
+        a2.nbatch = per;
+        a2.vec_step = step;
+        a2.p = ik;
+        a2.m2 = make_dpair(n->mass * n->mass);
+        a2.m2_in_args = 1;
+        CUDA_TRY(launch_dslash(P, EPI_M, a2, lat->dslash_block[P], s));
+    }
     return STAG_OK;
 }
 
-// loss of pair p added to scal[0] and its dL/dC*, dL/dc0* to G; the path
-// coefficients must be current.  z = N(r) -> fz; then the output gradient g:
+// losses of the pairs idx[0..np) (np <= group) added to scal[0] and their
+// dL/dC*, dL/dc0* to G; the path coefficients must be current.  z = N(r) ->
+// fz; then the output gradient g:
 //   error loss:    g = (z - e) / |e|^2                  -> fmz
 //   residual loss: q = (M z - r) / |r|^2 -> fmz, g = M q -> fz (M Hermitian)
-static int pair_loss_grad(stag_net n, int p, cudaStream_t s) {
-    stag_lattice lat = n->lat;
-    const Geom &g = lat->geom;
-    const int S = g.stride, Vh = g.Vh;
-    CUDA_TRY(net_apply_path(n, STAG_F32, n->pr[p], Vh, n->fz, S, false, false, nullptr, nullptr, s));
+static int pairs_loss_grad(stag_net n, const int *idx, int np, cudaStream_t s) {
+    const Geom &g = n->lat->geom;
+    const bool resid = n->loss_kind == STAG_NET_LOSS_RESIDUAL;
+    NetPairs pairs = {};
+    pairs.n = np;
+    for (int k = 0; k < np; k++) {
+        pairs.r[k] = n->pr[idx[k]];
+        pairs.e[k] = n->pe[idx[k]];
+        pairs.norm2[k] = (resid ? n->rnorm2 : n->enorm2) + idx[k];
+    }
+    CUDA_TRY(launch_net_pairs(g, net_links(n, false), n->path, pairs, n->chi, (float2 *)n->fz, s));
     const float2 *gv;
-    if (n->loss_kind == STAG_NET_LOSS_RESIDUAL) {
-        STAG_TRY(apply_M_f32(n, n->fz, n->ft, n->fmz, s));
-        CUDA_TRY(launch_net_resid_loss(Vh, (float2 *)n->fmz, S, n->pr[p], Vh, n->rnorm2 + p, n->scal, s));
-        STAG_TRY(apply_M_f32(n, n->fmz, n->ft, n->fz, s));
+    if (resid) {
+        STAG_TRY(apply_M_f32(n, np, n->fz, n->ft, n->fmz, s));
+        CUDA_TRY(launch_net_resid_loss(g, pairs, (float2 *)n->fmz, n->scal, s));
+        STAG_TRY(apply_M_f32(n, np, n->fmz, n->ft, n->fz, s));
         gv = (const float2 *)n->fz;
     } else {
-        CUDA_TRY(launch_net_error_loss(Vh, (const float2 *)n->fz, S, n->pe[p], Vh, n->enorm2 + p, (float2 *)n->fmz,
-                                       n->scal, s));
+        CUDA_TRY(launch_net_error_loss(g, pairs, (const float2 *)n->fz, (float2 *)n->fmz, n->scal, s));
         gv = (const float2 *)n->fmz;
     }
-    CUDA_TRY(launch_net_grad(g, n->NL32, n->pr[p], Vh, gv, S, n->gpartial, n->G, s));
+    CUDA_TRY(launch_net_grad(g, n->NL32, pairs, gv, n->gpartial, n->G, s));
     return STAG_OK;
 }
 
@@ -528,8 +574,8 @@ static int loss_grad_range(stag_net n, const int *idx, int count, double *loss) 
     CUDA_TRY(cudaMemsetAsync(n->G, 0, sizeof(double2) * 65, s));
     CUDA_TRY(cudaMemsetAsync(n->scal, 0, sizeof(double), s));
     CUDA_TRY(net_coefficients(n, 0, s));
-    for (int k = 0; k < count; k++)
-        STAG_TRY(pair_loss_grad(n, idx[k], s));
+    for (int k = 0; k < count; k += n->group)
+        STAG_TRY(pairs_loss_grad(n, idx + k, std::min(n->group, count - k), s));
     CUDA_TRY(launch_net_path_chain(n->C, n->w32, n->off, n->G, (double2 *)n->grad, s));
     if (loss) {
         CUDA_TRY(cudaMemcpyAsync(loss, n->scal, sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -568,7 +614,7 @@ static int residual_warm_start(stag_net n) {
     CUDA_TRY(net_coefficients(n, 0, s));
     for (size_t p = 0; p < n->pr.size(); p++) {
         CUDA_TRY(net_apply_path(n, STAG_F32, n->pr[p], Vh, n->fz, S, false, false, nullptr, nullptr, s));
-        STAG_TRY(apply_M_f32(n, n->fz, n->ft, n->fmz, s));
+        STAG_TRY(apply_M_f32(n, 1, n->fz, n->ft, n->fmz, s));
         CUDA_TRY(launch_net_dot2(Vh, (const float2 *)n->fmz, S, n->pr[p], Vh, n->scal + 1, s));
     }
     double h[2];

@@ -23,6 +23,15 @@ struct NetLinkSet {
     int bcneg = 0;              // bit mu: the boundary sign of direction mu is -1
 };
 
+// up to NET_PAIRS training pairs in one launch (blockIdx.y): their inputs,
+// and for the losses the targets' norms
+constexpr int NET_PAIRS = 8;
+struct NetPairs {
+    int n;
+    const float2 *r[NET_PAIRS], *e[NET_PAIRS];
+    const double *norm2[NET_PAIRS];
+};
+
 cudaError_t launch_net_links_cb(const Geom &g, const double bc[4], const double *fat, float2 *NL32, short2 *NL16,
                                 float inv_scale16, cudaStream_t s);
 // rows 0 and 1 of the net links in 16-bit: per (parity, mu) an int4 plane
@@ -47,13 +56,17 @@ cudaError_t launch_net_out(int prec_in, int prec_out, const Geom &g, const NetLi
                            double *partial, const int *gate, cudaStream_t s);
 int net_grid(const Geom &g);
 int net_grad_blocks(const Geom &g);
-// G[0..63] += dL/dC*, G[64] += dL/dc0* for input r and output gradient g (FP32)
-cudaError_t launch_net_grad(const Geom &g, const float2 *NL32, const float2 *r, int rs, const float2 *gv, int gs,
+// the same two passes on the FP32 inputs of training pairs (links FP32): chi
+// [n][8][3][stride], z [n][3][stride]
+cudaError_t launch_net_pairs(const Geom &g, const NetLinkSet &nl, const NetPath *path, const NetPairs &pairs,
+                             float2 *chi, float2 *z, cudaStream_t s);
+// G[0..63] += dL/dC*, G[64] += dL/dc0* for the pairs' inputs r and output
+// gradients gv [n][3][stride] (FP32); partial: 65 n net_grad_blocks double2
+cudaError_t launch_net_grad(const Geom &g, const float2 *NL32, const NetPairs &pairs, const float2 *gv,
                             double2 *partial, double2 *G, cudaStream_t s);
-cudaError_t launch_net_error_loss(int Vh, const float2 *z, int zs, const float2 *e, int es, const double *enorm2,
-                                  float2 *gv, double *loss, cudaStream_t s);
-cudaError_t launch_net_resid_loss(int Vh, float2 *mz, int ms, const float2 *r, int rs, const double *rnorm2,
-                                  double *loss, cudaStream_t s);
+cudaError_t launch_net_error_loss(const Geom &g, const NetPairs &pairs, const float2 *z, float2 *gv, double *loss,
+                                  cudaStream_t s);
+cudaError_t launch_net_resid_loss(const Geom &g, const NetPairs &pairs, float2 *mz, double *loss, cudaStream_t s);
 cudaError_t launch_net_dot2(int Vh, const float2 *a, int as, const float2 *b, int bs, double *out, cudaStream_t s);
 cudaError_t launch_fcg_finish(const double *partial, int n, CgScalars *sc, int first, cudaStream_t s);
 cudaError_t launch_fcg_copy_dots(int prec, const Geom &g, const void *r, void *z, const void *Ap, double *partial,

@@ -28,21 +28,21 @@ template <int BLOCK> STAG_D double sum_partials(const double *__restrict__ v, in
     return all;
 }
 
-// alpha = rr / <p, Ap> of this iteration into salpha (shared memory) and the
-// solve's status with the breakdown test on <p, Ap> applied, in every thread;
-// block 0 also stores pAp and alpha, which no block of the kernel may read
-// from the scalars then (nor write rr or status before every block has
-// called this).  Ends with a barrier.
-template <int BLOCK>
-STAG_D int iteration_alpha(const PapPartials &pap, CgScalars *sc, double *smem, dpair &salpha) {
-    __shared__ int sstatus;
+// alpha = rr / <p, Ap> of this iteration and the solve's status with the
+// breakdown test on <p, Ap> applied, in every thread; block 0 also stores pAp
+// and alpha, which no block of the kernel may read from the scalars then (nor
+// write rr or status before every block has called this).  Without partials
+// (SMALL false: the kernels of larger lattices, which the sum's registers
+// would cost occupancy) both are the scalars' own.
+template <bool SMALL, int BLOCK>
+STAG_D int iteration_alpha(const PapPartials &pap, CgScalars *sc, double *smem, dpair &alpha) {
     const int status = sc->status;
-    if (pap.n == 0 || status != CG_RUNNING) {
-        if (threadIdx.x == 0)
-            salpha = sc->alpha;
-        __syncthreads();
+    if (!SMALL || status != CG_RUNNING) {
+        alpha = sc->alpha;
         return status;
     }
+    __shared__ dpair salpha;
+    __shared__ int sstatus;
     const double total = sum_partials<BLOCK>(pap.v, pap.n, smem);
     if (threadIdx.x == 0) {
         sstatus = total > 0.0 && total < INFINITY ? CG_RUNNING : CG_BREAKDOWN;
@@ -53,6 +53,7 @@ STAG_D int iteration_alpha(const PapPartials &pap, CgScalars *sc, double *smem, 
         }
     }
     __syncthreads();
+    alpha = salpha;
     return sstatus;
 }
 
