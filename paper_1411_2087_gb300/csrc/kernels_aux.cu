@@ -69,32 +69,32 @@ cg_update_kernel(Geom g, typename Fmt<P>::Elem *x, typename Fmt<P>::Elem *r,
     using F = Fmt<P>;
     using R = typename F::R;
     __shared__ double smem[32];
-    const int c = blockIdx.x * BLOCK + threadIdx.x;
     const bool run = sc->status == CG_RUNNING;
+    const R alpha = scalar_as<R>(sc->alpha);
+    const R malpha = -alpha;
     red_t<R> dot = red_zero<red_t<R>>();
-    if (run && c < g.Vh) {
-        const R alpha = scalar_as<R>(sc->alpha);
-        const R malpha = -alpha;
-        cplx<R> xv[3], rv[3], pv[3], av[3];
-        load_vec<P>(x, g.stride, c, xv);
-        load_vec<P>(r, g.stride, c, rv);
-        load_vec<P>(p, g.stride, c, pv);
-        load_vec<P>(Ap, g.stride, c, av);
+    if (run)
+        for (int c = blockIdx.x * BLOCK + threadIdx.x; c < g.Vh; c += gridDim.x * BLOCK) {
+            cplx<R> xv[3], rv[3], pv[3], av[3];
+            load_vec<P>(x, g.stride, c, xv);
+            load_vec<P>(r, g.stride, c, rv);
+            load_vec<P>(p, g.stride, c, pv);
+            load_vec<P>(Ap, g.stride, c, av);
 #pragma unroll
-        for (int k = 0; k < 3; k++) {
-            mac(xv[k].re, alpha, pv[k].re);
-            mac(xv[k].im, alpha, pv[k].im);
-            mac(rv[k].re, malpha, av[k].re);
-            mac(rv[k].im, malpha, av[k].im);
-            xv[k].re = rnorm<R>(xv[k].re);
-            xv[k].im = rnorm<R>(xv[k].im);
-            rv[k].re = rnorm<R>(rv[k].re);
-            rv[k].im = rnorm<R>(rv[k].im);
+            for (int k = 0; k < 3; k++) {
+                mac(xv[k].re, alpha, pv[k].re);
+                mac(xv[k].im, alpha, pv[k].im);
+                mac(rv[k].re, malpha, av[k].re);
+                mac(rv[k].im, malpha, av[k].im);
+                xv[k].re = rnorm<R>(xv[k].re);
+                xv[k].im = rnorm<R>(xv[k].im);
+                rv[k].re = rnorm<R>(rv[k].re);
+                rv[k].im = rnorm<R>(rv[k].im);
+            }
+            store_vec<P>(x, g.stride, c, xv);
+            store_vec<P>(r, g.stride, c, rv);
+            dot = red_add(dot, re_dot3<R>(rv, rv));
         }
-        store_vec<P>(x, g.stride, c, xv);
-        store_vec<P>(r, g.stride, c, rv);
-        dot = re_dot3<R>(rv, rv);
-    }
     double total;
     if (grid_sum<BLOCK>(dot, partial, &sc->ticket, smem, total) && threadIdx.x == 0) {
         if (sc->status == CG_RUNNING) {
@@ -305,7 +305,7 @@ cudaError_t launch_cg_update(int prec, const Geom &g, void *x, void *r, const vo
                              const void *Ap, double *partial, CgScalars *sc, cudaStream_t s) {
     STAG_PREC_SWITCH(prec, {
         using E = typename Fmt<P>::Elem;
-        cg_update_kernel<P, CG_BLOCK><<<cg_grid(g), CG_BLOCK, 0, s>>>(
+        cg_update_kernel<P, CG_BLOCK><<<sum_grid(g.Vh, CG_BLOCK), CG_BLOCK, 0, s>>>(
             g, (E *)x, (E *)r, (const E *)p, (const E *)Ap, partial, sc);
     });
     return cudaGetLastError();

@@ -98,30 +98,37 @@ mixed_update_kernel(Geom g, float2 *xs, typename Fmt<PL>::Elem *rs, const typena
     using RL = typename Fmt<PL>::R;
     __shared__ double smem[32];
     dpair alpha_k;
-    const int c = blockIdx.x * MB + threadIdx.x;
     cplx<float> xv[3];
     cplx<RL> rv[3], pv[3], av[3];
-    if (c < g.Vh) {  // in flight while alpha is found
+    auto load = [&](int c) {
         load_vec<P_F32>(xs, g.stride, c, xv);
         load_vec<PL>(rs, g.stride, c, rv);
         load_vec<PL>(p, g.stride, c, pv);
         load_vec<PL>(Ap, g.stride, c, av);
-    }
+    };
+    int c = blockIdx.x * MB + threadIdx.x;
+    if (SMALL && c < g.Vh)  // one site per thread, in flight while alpha is found
+        load(c);
     const int status = iteration_alpha<SMALL, MB>(pap, sc, smem, alpha_k);
+    const float alpha = scalar_as<float>(alpha_k);
     red_t<RL> dot = red_zero<red_t<RL>>();
-    if (status == CG_RUNNING && c < g.Vh) {
-        const float alpha = scalar_as<float>(alpha_k);
+    if (status == CG_RUNNING)
+        for (; c < g.Vh; c += gridDim.x * MB) {
+            if (!SMALL)
+                load(c);
 #pragma unroll
-        for (int k = 0; k < 3; k++) {
-            xv[k].re = fmaf(alpha, (float)pv[k].re, xv[k].re);
-            xv[k].im = fmaf(alpha, (float)pv[k].im, xv[k].im);
-            rv[k].re = fmaf(-alpha, av[k].re, rv[k].re);
-            rv[k].im = fmaf(-alpha, av[k].im, rv[k].im);
+            for (int k = 0; k < 3; k++) {
+                xv[k].re = fmaf(alpha, (float)pv[k].re, xv[k].re);
+                xv[k].im = fmaf(alpha, (float)pv[k].im, xv[k].im);
+                rv[k].re = fmaf(-alpha, av[k].re, rv[k].re);
+                rv[k].im = fmaf(-alpha, av[k].im, rv[k].im);
+            }
+            store_vec<P_F32>(xs, g.stride, c, xv);
+            store_vec<PL>(rs, g.stride, c, rv);
+            dot = red_add(dot, re_dot3<RL>(rv, rv));
+            if (SMALL)
+                break;
         }
-        store_vec<P_F32>(xs, g.stride, c, xv);
-        store_vec<PL>(rs, g.stride, c, rv);
-        dot = re_dot3<RL>(rv, rv);
-    }
     double total;
     if (grid_sum<MB>(dot, partial, &sc->ticket, smem, total) && threadIdx.x == 0) {
         sc->reliable = 0;
@@ -247,10 +254,10 @@ cudaError_t launch_mixed_update(int lo, const Geom &g, float *xs, void *rs, cons
         using EL = typename Fmt<PL>::Elem;
         if (pap.n > 0)
             mixed_update_kernel<PL, true><<<grid_of(g), MB, 0, s>>>(g, (float2 *)xs, (EL *)rs, (const EL *)p,
-                                                              (const EL *)Ap, pap, partial, sc);
+                                                                    (const EL *)Ap, pap, partial, sc);
         else
-            mixed_update_kernel<PL, false><<<grid_of(g), MB, 0, s>>>(g, (float2 *)xs, (EL *)rs, (const EL *)p,
-                                                              (const EL *)Ap, pap, partial, sc);
+            mixed_update_kernel<PL, false><<<sum_grid(g.Vh, MB), MB, 0, s>>>(g, (float2 *)xs, (EL *)rs, (const EL *)p,
+                                                                             (const EL *)Ap, pap, partial, sc);
     });
     return cudaGetLastError();
 }

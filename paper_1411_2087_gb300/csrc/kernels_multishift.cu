@@ -117,23 +117,12 @@ ms_init_kernel(Geom g, MsArgs a, double *partial, CgScalars *sc, ShiftState *st)
     }
 }
 
-// zeta_{k+1}, alpha^s for every shift from the scalars of the base CG; every
-// block computes them (one lane per shift) into shared memory
-STAG_D void ms_shift_scalars(const MsArgs &a, double al, const CgScalars *sc, const ShiftState *st,
-                             double *zeta_next, double *alpha_s) {
-    const int s = threadIdx.x;
-    if (s < a.n) {
-        const double alp = sc->alpha_prev, bep = sc->beta_prev;
-        const double z = st[s].zeta, zp = st[s].zeta_prev;
-        const double den = al * bep * (zp - z) + zp * alp * (1.0 + a.delta[s] * al);
-        const double zn = z * zp * alp / den;
-        zeta_next[s] = zn;
-        alpha_s[s] = al * zn / z;
-    }
-}
-
 // r -= alpha Ap, |r|^2; the shift scalars of this iteration (the solution
-// updates x_s += alpha^s p_s run in ms_p_kernel, which reads p_s anyway)
+// updates x_s += alpha^s p_s run in ms_p_kernel, which reads p_s anyway).  The
+// scalars are FP64, whose adds and divisions take tens of cycles each: only
+// the last block computes them, one lane per shift.  (Every block computing
+// them, and one thread walking the shifts at the end, made this kernel 31 us
+// at 24^3x48 with 12 shifts, of which the vectors need 7.)
 template <int P, int PA, bool SMALL>
 __global__ void __launch_bounds__(MSB)
 ms_update_kernel(Geom g, MsArgs a, const void *Ap, PapPartials pap0, PapPartials pap1, double *partial,
@@ -143,8 +132,6 @@ ms_update_kernel(Geom g, MsArgs a, const void *Ap, PapPartials pap0, PapPartials
     using E = typename F::Elem;
     using RA = typename Fmt<PA>::R;
     __shared__ double smem[32];
-    __shared__ double zeta_next[MS_MAX], alpha_s[MS_MAX];
-    __shared__ int active[MS_MAX];
     dpair alpha_k;
     // the previous iteration's solution updates are done (ms_p_kernel has
     // finished); written before this block's ticket, so before the last
@@ -156,11 +143,6 @@ ms_update_kernel(Geom g, MsArgs a, const void *Ap, PapPartials pap0, PapPartials
     const bool hi_path = PA == P || sc->ms_hi_op;
     const int status = iteration_alpha<SMALL, MSB>(hi_path ? pap0 : pap1, sc, smem, alpha_k);
     const bool run = status == CG_RUNNING;
-    if (run)
-        ms_shift_scalars(a, alpha_k.d, sc, st, zeta_next, alpha_s);
-    if (threadIdx.x < MS_MAX)
-        active[threadIdx.x] = threadIdx.x < a.n ? st[threadIdx.x].active : 0;
-    __syncthreads();
     const int c = blockIdx.x * MSB + threadIdx.x;
     red_t<R> dot = red_zero<red_t<R>>();
     if (run && c < g.Vh) {
@@ -187,58 +169,63 @@ ms_update_kernel(Geom g, MsArgs a, const void *Ap, PapPartials pap0, PapPartials
         dot = re_dot3<R>(rv, rv);
     }
     double total;
-    if (grid_sum<MSB>(dot, partial, &sc->ticket, smem, total) && threadIdx.x == 0) {
-        sc->status = status;
-        if (status == CG_RUNNING) {
-            const double beta = total / sc->rr;
-            sc->beta = make_dpair(beta);
-            sc->iter += 1;
-            bool any = false;
-            for (int s = 0; s < a.n; s++) {
-                if (!active[s])
-                    continue;
-                const double zn = zeta_next[s], z = st[s].zeta;
-                const double ratio = zn / z;
-                st[s].alpha_s = make_dpair(alpha_s[s]);
-                st[s].beta_s = make_dpair(beta * ratio * ratio);
-                st[s].zeta_next = make_dpair(zn);
-                st[s].zeta_prev = z;
-                st[s].zeta = zn;
-                st[s].iters = sc->iter;
-                // the shifted residual zeta r meets the tolerance: freeze
-                // after this iteration's x update (iters == iter marks it
-                // for ms_p_kernel; p_s is not needed again)
-                if (zn * zn * total <= sc->rr_stop)
-                    st[s].active = 0;
-                else
-                    any = true;
-            }
-            sc->alpha_prev = alpha_k.d;
-            sc->beta_prev = beta;
-            sc->rr = total;
-            const double rn = sqrt(total);
-            sc->reliable = 0;
-            if (!(total < INFINITY)) {
-                sc->status = CG_BREAKDOWN;
-            } else if (sc->delta > 0.0 && ((!hi_path && rn < sc->delta * sc->rmax) || !any ||
-                                           sc->iter >= sc->max_iter)) {
-                // mixed precision: the base residual is recomputed first, and
-                // the stop is decided on it (ms_restart_kernel); iterations on
-                // the exact operator need no update on the way
-                sc->reliable = 1;
-            } else if (!any) {
-                sc->status = CG_CONVERGED;
-            } else if (sc->iter >= sc->max_iter) {
-                sc->status = CG_MAXITER;
-            }
-            sc->rmax = fmax(sc->rmax, rn);
-            sc->ms_hi_op = total > a.theta2 * sc->bb ? 1 : 0;
-            sc->ms_lo_op = 1 - sc->ms_hi_op;
-        }
-        if (sc->has_rel_cond)
-            cudaGraphSetConditional(sc->rel_cond, sc->reliable ? 1u : 0u);
-        ms_set_condition(sc);
+    if (!grid_sum<MSB>(dot, partial, &sc->ticket, smem, total))
+        return;
+    const double beta = run ? total / sc->rr : 0.0;
+    const int iter = sc->iter + 1;
+    bool still = false;
+    const int s = threadIdx.x;
+    if (run && s < a.n && st[s].active) {
+        // zeta_{k+1} and alpha^s of this shift from the base CG's scalars
+        const double al = alpha_k.d, alp = sc->alpha_prev, bep = sc->beta_prev;
+        const double z = st[s].zeta, zp = st[s].zeta_prev;
+        const double den = al * bep * (zp - z) + zp * alp * (1.0 + a.delta[s] * al);
+        const double zn = z * zp * alp / den;
+        const double ratio = zn / z;
+        st[s].alpha_s = make_dpair(al * zn / z);
+        st[s].beta_s = make_dpair(beta * ratio * ratio);
+        st[s].zeta_next = make_dpair(zn);
+        st[s].zeta_prev = z;
+        st[s].zeta = zn;
+        st[s].iters = iter;
+        // the shifted residual zeta r meets the tolerance: freeze after this
+        // iteration's x update (iters == iter marks it for ms_p_kernel; p_s
+        // is not needed again)
+        still = !(zn * zn * total <= sc->rr_stop);
+        if (!still)
+            st[s].active = 0;
     }
+    const bool any = __syncthreads_or(still);  // and every lane has read the scalars
+    if (threadIdx.x != 0)
+        return;
+    sc->status = status;
+    if (run) {
+        sc->beta = make_dpair(beta);
+        sc->iter = iter;
+        sc->alpha_prev = alpha_k.d;
+        sc->beta_prev = beta;
+        sc->rr = total;
+        const double rn = sqrt(total);
+        sc->reliable = 0;
+        if (!(total < INFINITY)) {
+            sc->status = CG_BREAKDOWN;
+        } else if (sc->delta > 0.0 && ((!hi_path && rn < sc->delta * sc->rmax) || !any || iter >= sc->max_iter)) {
+            // mixed precision: the base residual is recomputed first, and
+            // the stop is decided on it (ms_restart_kernel); iterations on
+            // the exact operator need no update on the way
+            sc->reliable = 1;
+        } else if (!any) {
+            sc->status = CG_CONVERGED;
+        } else if (iter >= sc->max_iter) {
+            sc->status = CG_MAXITER;
+        }
+        sc->rmax = fmax(sc->rmax, rn);
+        sc->ms_hi_op = total > a.theta2 * sc->bb ? 1 : 0;
+        sc->ms_lo_op = 1 - sc->ms_hi_op;
+    }
+    if (sc->has_rel_cond)
+        cudaGraphSetConditional(sc->rel_cond, sc->reliable ? 1u : 0u);
+    ms_set_condition(sc);
 }
 
 // after a reliable update (r = b - (M + sigma_0) x_0 recomputed, |r|^2 in

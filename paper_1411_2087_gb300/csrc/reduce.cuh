@@ -62,23 +62,23 @@ template <int BLOCK, class T> STAG_D double block_sum(T v, double *smem) {
 }
 
 // This thread's share of the sum of n partials of stride `step` that other
-// blocks wrote: a fixed assignment to BLOCK threads, eight loads in flight
+// blocks wrote: a fixed assignment to BLOCK threads, U loads in flight
 // (one after the other, the last block of a 4096-block reduction waited 16
 // L2 latencies).  A warp past n skips its adds: an FP64 add costs its
 // scheduler 64 cycles also when it adds nothing.
-template <int BLOCK> STAG_D double partials_share(const double *__restrict__ v, int n, int step = 1) {
+template <int BLOCK, int U = 8> STAG_D double partials_share(const double *__restrict__ v, int n, int step = 1) {
     if (n <= BLOCK)
         return (int)threadIdx.x < n ? __ldcg(v + (size_t)threadIdx.x * step) : 0.0;
     double a = 0.0;
-    for (int base = threadIdx.x & ~31; base < n; base += 8 * BLOCK) {
-        double t[8];
+    for (int base = threadIdx.x & ~31; base < n; base += U * BLOCK) {
+        double t[U];
 #pragma unroll
-        for (int u = 0; u < 8; u++) {
+        for (int u = 0; u < U; u++) {
             const int i = base + u * BLOCK + (threadIdx.x & 31);
             t[u] = i < n ? __ldcg(v + (size_t)i * step) : 0.0;
         }
 #pragma unroll
-        for (int u = 0; u < 8; u++)
+        for (int u = 0; u < U; u++)
             if (base + u * BLOCK < n)
                 a += t[u];
     }
@@ -103,7 +103,7 @@ STAG_D bool grid_sum(T v, double *partial, unsigned *ticket, double *smem, doubl
     if (!last)
         return false;
     __threadfence();
-    const double acc = block_sum<BLOCK>(partials_share<BLOCK>(partial, (int)gridDim.x), smem);
+    const double acc = block_sum<BLOCK>(partials_share<BLOCK, 4>(partial, (int)gridDim.x), smem);
     if (threadIdx.x == 0) {
         smem[0] = acc;
         *ticket = 0u;
@@ -112,6 +112,17 @@ STAG_D bool grid_sum(T v, double *partial, unsigned *ticket, double *smem, doubl
     total = smem[0];
     __syncthreads();
     return true;
+}
+
+// Blocks of a vector kernel that ends in grid_sum: at most eight per SM, each
+// thread then takes several sites.  With one site per thread a block spends
+// as long on its fence and ticket as on its loads (16-bit update at 1048576
+// sites: 25 us, now 21; a mixed solve on 48^3x96 598 -> 583 ms).  Not where
+// some threads would take two sites and most one (331776 sites: 19.3 -> 20.4).
+constexpr int SUM_BLOCKS = 8 * 152;
+inline int sum_grid(int n, int block) {
+    const int need = (n + block - 1) / block;
+    return need <= 2 * SUM_BLOCKS ? need : SUM_BLOCKS;
 }
 
 // Grid-wide sum of two values per thread (same protocol as grid_sum;
