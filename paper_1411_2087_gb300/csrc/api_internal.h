@@ -330,8 +330,12 @@ static inline int m_block(const stag_lattice lat, int prec) {
 // On lattices up to this many sites per parity the launches are short and
 // counting them is what matters: the solvers leave <p, Ap> to the next kernel
 // (small_sums.cuh).  Larger ones sum the M Dslash's partials in a one-block
-// kernel.
-constexpr int kSmallVh = 65536;
+// kernel: there are too many for every block to add them in FP64 (an
+// iteration of plain CG, multi-shift CG in double float left to the next
+// kernel against summed by the one block: 80000 sites 84.8, 97.9 against
+// 86.0, 100.2 us, 96000: 99.2, 112.5 against 100.8, 113.0, 128000: 133, 145
+// against 126, 143).
+constexpr int kSmallVh = 100000;
 
 // the M Dslash Ap = m^2 p - D_eo t of an iteration (skip_if_done: it returns
 // at once after the solve)

@@ -132,7 +132,14 @@ template <> struct Fmt<P_F32> {
 // three components.
 constexpr float kQ16 = 32767.f;
 
-STAG_D short q16(float v) { return (short)__float2int_rn(fminf(fmaxf(v, -kQ16), kQ16)); }
+// the conversion saturates, and |v| <= 32767 up to rounding by the choice of
+// the scales (an explicit clamp took two more instructions per value: a
+// learned 16-bit solve at 32^3x64 163.9 -> 161.7 ms)
+STAG_D short q16(float v) {
+    short q;
+    asm("cvt.rni.s16.f32 %0, %1;" : "=h"(q) : "f"(v));
+    return q;
+}
 
 // the two int16 halves of a 32-bit word (a short2: x low, y high) as floats
 // (exact), and the word from two stored values

@@ -459,13 +459,13 @@ template <> struct Chi<L12> : Chi<short2> {};
 // links' scale (1 for FP32).  The eight transported vectors go to shared
 // memory first (each thread reads back only its own), so that the loads of
 // the transport phase and the mixing's 48 live values never meet.
-// Six resident blocks (at most 80 registers, 24 warps per SM): at eight the
-// 16-bit form spills 96 bytes, and measured at 32^3x64 the solver-form net
-// application took 0.342 ms against 0.308 ms at six.
+// Seven resident blocks (72 registers, 28 warps per SM): a learned mixed solve
+// at 32^3x64 takes 160.9 ms at six, 160.4 at seven, 163.0 at eight, where the
+// 16-bit form spills.
 // Q = NetPairs: the inputs of several training pairs in one launch, pair
 // blockIdx.y with the y-th part of chi (NoPairs: the one input r).
 struct NoPairs {};
-constexpr int NET_MID_MINB = 6;
+constexpr int NET_MID_MINB = 7;
 
 template <int P, class LT, class Q>
 __global__ void __launch_bounds__(NET_BLOCK, NET_MID_MINB)
@@ -580,10 +580,14 @@ net_mid_kernel(Geom g, const LT *__restrict__ NL, float ls, int bcneg, const Net
 // z(x) = c0 r(x) + sum_a (T_a chi_a)(x) on the even sites.  NET_OUT_DOTS
 // adds per-block partials of Re<z, r> (partial[blk]) and Re<z, Ap>
 // (partial[nblk + blk]; 0 without Ap) for the flexible CG.
+// Nine resident blocks (56 registers, latency-bound at eight: 66 us at
+// 32^3x64; a learned mixed solve 161.7 ms at eight, 160.9 at nine and ten,
+// 163.4 at twelve).
 enum { NET_OUT_PLAIN = 0, NET_OUT_DOTS = 1 };
+constexpr int NET_OUT_MINB = 9;
 
 template <int PI, int PO, class LT, int EPI, class Q>
-__global__ void __launch_bounds__(NET_BLOCK)
+__global__ void __launch_bounds__(NET_BLOCK, NET_OUT_MINB)
 net_out_kernel(Geom g, const LT *__restrict__ NL, float ls, int bcneg, const NetPath *__restrict__ path,
                const void *__restrict__ chi, const typename Fmt<PI>::Elem *__restrict__ r, int rs,
                typename Fmt<PO>::Elem *__restrict__ z, int zs, const typename Fmt<PO>::Elem *__restrict__ Ap,
