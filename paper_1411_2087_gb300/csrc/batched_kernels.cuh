@@ -269,8 +269,14 @@ __global__ void __launch_bounds__(BLOCK, P == P_DF64 ? 896 / BLOCK : 0) batch_ds
         const void *Gout = G.links[out_par], *Gin = G.links[1 - out_par];
         const E *in = (const E *)batch_lane_input<EPI>(G, k, src_x);
 #pragma unroll 4
-        for (int hop = 0; hop < 16; hop++)
+        for (int hop = 0; hop < 16; hop++) {
             stencil_hop<P, 0, LD_STREAM>(g, Gout, Gin, in, 0, 0, c, x, hop >> 2, (hop >> 1) & 1, hop & 1, acc);
+            if ((hop & 3) == 3) {
+#pragma unroll
+                for (int r = 0; r < 3; r++)
+                    cnorm(acc[r]);
+            }
+        }
         dot = batch_lane_epilogue<P, EPI>(a, G, k, c, acc);
     }
     batch_lane_reduce<EPI, BLOCK, K, BLOCK, 1>(a, gi, G, act, lblk, dot, smem);

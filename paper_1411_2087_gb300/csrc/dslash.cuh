@@ -185,6 +185,9 @@ STAG_D void dslash_site(const Geom &g, int par, int c, const void *__restrict__ 
                             cmac_conj(acc[r], L[3 * b + r], v[b]);
                 }
             }
+#pragma unroll
+            for (int r = 0; r < 3; r++)
+                cnorm(acc[r]);
         }
     }
 }
