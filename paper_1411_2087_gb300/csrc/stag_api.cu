@@ -360,6 +360,19 @@ extern "C" int stag_gauge_upload(stag_lattice lat, const double *fat, const doub
     // the copies of the last upload keep their buffers where this one has
     // the same (allocating 24^3x48 in DF64, FP32 and 16-bit anew took 1.5 ms)
     drop_links(lat, prec_mask, cmask);
+    // (the solver workspaces are kept too; they go when memory is short, the
+    // next solve makes them again)
+    auto alloc_copy = [&](void **p, size_t bytes) {
+        cudaError_t e = cudaMalloc(p, bytes);
+        if (e == cudaErrorMemoryAllocation) {
+            cudaGetLastError();
+            for (int q = 0; q < 4; q++)
+                free_cg(lat->cg[q]);
+            e = cudaMalloc(p, bytes);
+        }
+        // the padding sites of a new buffer are zero; the fold writes the others
+        return e == cudaSuccess ? cudaMemsetAsync(*p, 0, bytes, lat->stream) : e;
+    };
     FoldOut out;
     memset(&out, 0, sizeof out);
     out.mask = cmask;
@@ -367,20 +380,12 @@ extern "C" int stag_gauge_upload(stag_lattice lat, const double *fat, const doub
         if (!((prec_mask >> p) & 1u))
             continue;
         cudaError_t e = cudaSuccess;
-        // the padding sites of new buffers are zero; the fold writes the others
-        if (!lat->links[p]) {
-            e = cudaMalloc(&lat->links[p], link_bytes(lat, p));
-            if (e == cudaSuccess)
-                e = cudaMemsetAsync(lat->links[p], 0, link_bytes(lat, p), lat->stream);
-        }
+        if (!lat->links[p])
+            e = alloc_copy(&lat->links[p], link_bytes(lat, p));
         out.full[p] = lat->links[p];
         if (e == cudaSuccess && compress && (p == STAG_F32 || p == STAG_F16)) {
-            if (!lat->links_c12[p]) {
-                const size_t cb = c12_link_bytes(p, (size_t)lat->geom.stride, cmask);
-                e = cudaMalloc(&lat->links_c12[p], cb);
-                if (e == cudaSuccess)
-                    e = cudaMemsetAsync(lat->links_c12[p], 0, cb, lat->stream);
-            }
+            if (!lat->links_c12[p])
+                e = alloc_copy(&lat->links_c12[p], c12_link_bytes(p, (size_t)lat->geom.stride, cmask));
             lat->c12_mask[p] = cmask;
             out.c12[p] = lat->links_c12[p];
         }

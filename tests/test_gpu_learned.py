@@ -331,3 +331,25 @@ def test_learned_solver_edges():
         with pytest.raises(stag.StagError):
             stag.Net(lat, U, channels=3)
         net.close()
+
+
+@pytest.mark.parametrize("kind", ["error", "residual"])
+def test_gradient_of_several_launch_groups(kind):
+    """Eleven pairs (one launch group of eight and a rest of three) give the
+    sum of their single gradients and losses: the kernels are the same per
+    pair, so only the FP64 sums over pairs differ in order."""
+    dims, mass = (6, 4, 6, 10), 0.05
+    U = synth.su3_field(dims, 0.3, 91).numpy()
+    Vh = int(np.prod(dims)) // 2
+    with stag.Lattice(dims) as lat:
+        lat.upload_gauge(U, None, precisions=("df64", "f32"))
+        net = stag.Net(lat, U, 8, 5)
+        net.set_loss(kind)
+        b = lat.field(stag.EVEN, "df64", synth.gaussian_colour_field(Vh, 92).numpy())
+        assert net.collect_pairs(b, mass, 1e-10, 3, 11) == 11
+        loss, grads = net.loss_grad(0, 11)
+        parts = [net.loss_grad(k, 1) for k in range(11)]
+        assert abs(loss - sum(p[0] for p in parts)) <= 1e-10 * abs(loss)
+        for layer, g in enumerate(grads):
+            want = sum(p[1][layer] for p in parts)
+            assert np.abs(g - want).max() <= 1e-10 * max(np.abs(p[1][layer]).max() for p in parts)
