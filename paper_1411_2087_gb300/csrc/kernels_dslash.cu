@@ -22,7 +22,8 @@ int dslash_default_block(int prec) {
 //                 331776: 298 / 305, 1048576: 891 / 894, 3538944: 2930 / 2898
 //   FP64          2048: 34 / 60, 20736: 74 / 97, 32768: 94 / 97, 46080: 126 / 140,
 //                 96000: 229 / 221, 1048576: 2230 / 2128; single calls lose 4 % at 50000
-//   FP32 full     65536: 23 / 28, 80000: 29 / 30, 96000: 36 / 33
+//   FP32 full     65536: 23 / 28, 80000: 29 / 30, 96000: 36 / 33; a single
+//                 M at 65536, whose links nothing keeps in L2, 21.0 / 20.1
 //   FP32 12-real  20736: 12 / 14 (all), 12 / 16 (three-link); 32768: 16.5 / 15, 16.5 / 16.5
 // Eight warps per 32 sites on the smallest lattices (double float, 2048
 // sites: 24.5 against 27; 10368: 31.6 against 34; 20736: 41.6 against 39.6).
@@ -38,10 +39,11 @@ int split_warps(int prec, int compressed, const Geom &g) {
 // (an iteration of plain CG in double float at 46080 sites per parity 65 ->
 // 58 us, at 80000 93.5 -> 87; of mixed CG in FP32 on 12-real links at 80000
 // 59.9 -> 52.8, 128000: 69 -> 66; 64 MB and more were slower again).  A
-// single Dslash call keeps none (stag_dslash_*: its caller may well be
+// single call keeps none (stag_dslash_*, stag_apply_M: its caller may well be
 // working on several lattices in turn; three of them at 120960 sites on
-// 12-real links: 28.8 against 27.8 us a pair of calls).  The kernels that
-// load with LD_STREAM ignore it.
+// 12-real links: 28.8 against 27.8 us a pair of Dslash calls; M in FP32 at
+// 112000 sites 37.7 against 35.6 us, 331776: 112.1 against 110.1).  The
+// kernels that load with LD_STREAM ignore it.
 int link_keep_sites(int prec, int compressed) {
     const size_t site = 2 * link_parity_bytes(prec, compressed, 256) / 256;  // both parities' links
     return (int)((32u << 20) / site);

@@ -686,11 +686,13 @@ extern "C" int stag_apply_M(stag_lattice lat, stag_field out_even, const stag_fi
     STAG_TRY(ensure_cg_work(lat, prec));
     CgWork &w = lat->cg[prec];
     DslashArgs a1 = dslash_args(lat, prec, STAG_ODD, in_even->data, w.t);
+    a1.keep = 0;
     CUDA_TRY(launch_dslash(prec, EPI_NONE, a1, lat->dslash_block[prec], lat->stream));
     DslashArgs a2 = dslash_args(lat, prec, STAG_EVEN, w.t, out_even->data);
     a2.p = in_even->data;
     a2.m2 = make_dpair(mass * mass);
     a2.m2_in_args = 1;
+    a2.keep = 0;
     CUDA_TRY(launch_dslash(prec, EPI_M, a2, lat->dslash_block[prec], lat->stream));
     return STAG_OK;
 }
