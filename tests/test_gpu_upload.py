@@ -124,3 +124,20 @@ def test_su3_check_at_its_limit(dev, ok, kind):
         else:
             with pytest.raises(stag.StagError):
                 lat.upload_gauge(U, N, precisions=("f32",), compress12=True)
+
+
+# a warp of the scan takes every 97280th link from its 32 on: one link off in
+# its first, second and third chunk and at the end of either field
+@pytest.mark.parametrize("field", [0, 1])
+@pytest.mark.parametrize("link", [0, 97279, 97280, 97280 + 33, 2 * 97280 + 7, -1])
+def test_su3_check_finds_a_link_anywhere(field, link):
+    dims = (10, 14, 14, 30)
+    V = int(np.prod(dims))
+    assert 2 * 97280 + 7 < 4 * V
+    U = np.broadcast_to(np.eye(3, dtype=np.complex128), (4, V, 3, 3)).copy()
+    bad = U.copy()
+    bad.reshape(-1, 3, 3)[link] *= np.exp(1e-5j)
+    with stag.Lattice(dims) as lat:
+        lat.upload_gauge(U, U, precisions=("f32",), compress12=True)
+        with pytest.raises(stag.StagError):
+            lat.upload_gauge(*((bad, U) if field == 0 else (U, bad)), precisions=("f32",), compress12=True)
