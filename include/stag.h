@@ -322,8 +322,9 @@ int stag_cg_solve_batched_mixed(int n, stag_lattice *lats, stag_field *xs, const
  *                     register variants (regs 1: the compiler's choice,
  *                     2: capped for 768 to 1024 resident threads per SM, by
  *                     format)
- *                     and, for STAG_F16 on 12-real links with Lt a multiple
- *                     of 4 and at least 8, regs 3: two sites (x, y, z, t)
+ *                     and, for STAG_F16 with Lt a multiple of 4 and at least
+ *                     8, regs 3 (the default on 12-real links from 150000
+ *                     sites per parity on): two sites (x, y, z, t)
  *                     and (x, y, z, t + Lt/2) per thread in packed FP32x2
  *                     arithmetic (the same bits as the one-site forms), the
  *                     next hop's loads in flight through a shared-memory
@@ -339,7 +340,10 @@ int stag_cg_solve_batched_mixed(int n, stag_lattice *lats, stag_field *xs, const
  * the environment variable STAG_TUNE_CACHE names a file, the cache is read
  * from it at the first call and every new choice appended to it.  Every
  * candidate computes the same numbers (the block size only changes the order
- * of the solvers' partial sums).  Needs a gauge copy of `prec`; overwrites
+ * of the solvers' partial sums).  On small lattices (double-float up to
+ * 400000 sites per parity, FP64 36000, FP32 85000, on 12-real links 24576) the
+ * Dslash has one form without these choices, and all candidates are that form.
+ * Needs a gauge copy of `prec`; overwrites
  * the lattice's internal work vectors. */
 typedef struct {
     int kernel;    /* STAG_TUNE_DSLASH, STAG_TUNE_M or STAG_TUNE_BATCH          */
