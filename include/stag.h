@@ -149,6 +149,9 @@ int stag_lattice_set_cg_launch(stag_lattice lat, int mode, int chunk);
  *            compressed and checked (the paper's suggestion for smeared fat
  *            links, Sec. 4): 5/6 of the link bytes.
  *            A later upload replaces all copies.
+ * Device links (here, in stag_long_links_build and in stag_net_create) may
+ * start at any address that a double array may; where that is no 16-byte
+ * boundary the library works on a temporary copy.
  * Links holding a NaN, an infinity or an entry beyond the FP32 range give
  * STAG_ERR_ARG (the lattice then has no gauge field).
  * Blocks until the copies are built. */

@@ -302,6 +302,34 @@ static inline int upload_scalars(stag_lattice lat, double mass, double tol, int 
     return STAG_OK;
 }
 
+// The kernels read canonical links 16 bytes at a time (cp.async, double2).  A
+// caller's device array is taken as it is where it starts on a 16-byte
+// boundary; one that does not (any double array may), or a host array, is
+// copied into a temporary that the caller of this frees (*owned).
+static inline bool links_aligned(const void *p) { return (uintptr_t)p % 16 == 0; }
+
+static inline cudaError_t links_to_device(stag_lattice lat, const double *src, int ptr_kind, double **dev, bool *owned) {
+    *dev = (double *)src;
+    *owned = false;
+    if (ptr_kind == STAG_PTR_DEVICE && links_aligned(src))
+        return cudaSuccess;
+    const size_t bytes = 4ull * lat->V * 18 * sizeof(double);
+    cudaError_t e = cudaMalloc(dev, bytes);
+    if (e != cudaSuccess) {
+        *dev = nullptr;
+        return e;
+    }
+    e = cudaMemcpyAsync(*dev, src, bytes, ptr_kind == STAG_PTR_DEVICE ? cudaMemcpyDefault : cudaMemcpyHostToDevice,
+                        lat->stream);
+    if (e != cudaSuccess) {
+        cudaFree(*dev);
+        *dev = nullptr;
+        return e;
+    }
+    *owned = true;
+    return cudaSuccess;
+}
+
 static inline int alloc_vec(stag_lattice lat, int prec, void **p) {
     if (*p)
         return STAG_OK;

@@ -151,18 +151,10 @@ extern "C" int stag_net_create(stag_lattice lat, const double *fat, int ptr_kind
         }
     }
     // net links from the raw fat links (phases and boundary sign folded in)
-    double *fat_d = (double *)fat;
+    double *fat_d = nullptr;
     bool owned = false;
-    if (ptr_kind == STAG_PTR_HOST) {
-        const size_t bytes = 4 * V * 18 * sizeof(double);
-        if ((e = cudaMalloc(&fat_d, bytes)) != cudaSuccess)
-            return bail(e);
-        owned = true;
-        if ((e = cudaMemcpyAsync(fat_d, fat, bytes, cudaMemcpyHostToDevice, s)) != cudaSuccess) {
-            cudaFree(fat_d);
-            return bail(e);
-        }
-    }
+    if ((e = links_to_device(lat, fat, ptr_kind, &fat_d, &owned)) != cudaSuccess)
+        return bail(e);
     // the 16-bit copy's scale: the largest |re| or |im| of the field
     // (and whether they are special unitary, below)
     LinkScan *scan_d = (LinkScan *)n->scal;

@@ -232,27 +232,6 @@ static void drop_links(stag_lattice lat, unsigned prec_mask, int cmask) {
     }
 }
 
-// device copy of a canonical gauge field: returns a device pointer, allocating
-// a temporary when the source is on the host
-static int gauge_to_device(stag_lattice lat, const double *src, int ptr_kind, double **dev,
-                           bool *owned) {
-    const size_t bytes = 4ull * lat->V * 18 * sizeof(double);
-    if (ptr_kind == STAG_PTR_DEVICE) {
-        *dev = (double *)src;
-        *owned = false;
-        return STAG_OK;
-    }
-    CUDA_TRY(cudaMalloc(dev, bytes));
-    *owned = true;
-    cudaError_t e = cudaMemcpyAsync(*dev, src, bytes, cudaMemcpyHostToDevice, lat->stream);
-    if (e != cudaSuccess) {
-        cudaFree(*dev);
-        *dev = nullptr;
-        return fail(STAG_ERR_CUDA, "gauge copy to device: %s", cudaGetErrorString(e));
-    }
-    return STAG_OK;
-}
-
 extern "C" int stag_gauge_upload(stag_lattice lat, const double *fat, const double *lng, double c1,
                                  double c3, int ptr_kind, unsigned prec_mask) {
     STAG_NVTX("stag_gauge_upload");
@@ -286,9 +265,8 @@ extern "C" int stag_gauge_upload(stag_lattice lat, const double *fat, const doub
         CUDA_TRY(cudaDeviceSynchronize());
     double *fat_d = nullptr, *lng_d = nullptr;
     bool fat_owned = false, lng_owned = false;
-    int st = gauge_to_device(lat, fat, ptr_kind, &fat_d, &fat_owned);
-    if (st != STAG_OK)
-        return st;
+    int st = STAG_OK;
+    CUDA_TRY(links_to_device(lat, fat, ptr_kind, &fat_d, &fat_owned));
     auto release = [&]() {
         cudaStreamSynchronize(lat->stream);
         if (fat_owned)
@@ -297,7 +275,10 @@ extern "C" int stag_gauge_upload(stag_lattice lat, const double *fat, const doub
             cudaFree(lng_d);
     };
     if (lng) {
-        st = gauge_to_device(lat, lng, ptr_kind, &lng_d, &lng_owned);
+        const cudaError_t e = links_to_device(lat, lng, ptr_kind, &lng_d, &lng_owned);
+        if (e != cudaSuccess)
+            st = fail(e == cudaErrorMemoryAllocation ? STAG_ERR_NOMEM : STAG_ERR_CUDA, "long-link copy to device: %s",
+                      cudaGetErrorString(e));
     } else {
         cudaError_t e = cudaMalloc(&lng_d, 4ull * lat->V * 18 * sizeof(double));
         if (e == cudaSuccess) {
@@ -420,19 +401,22 @@ extern "C" int stag_long_links_build(stag_lattice lat, const double *fat, double
     const size_t bytes = 4ull * lat->V * 18 * sizeof(double);
     double *fat_d = nullptr;
     bool owned = false;
-    STAG_TRY(gauge_to_device(lat, fat, ptr_kind, &fat_d, &owned));
+    CUDA_TRY(links_to_device(lat, fat, ptr_kind, &fat_d, &owned));
     double *out_d = (double *)lng;
     cudaError_t e = cudaSuccess;
-    if (ptr_kind == STAG_PTR_HOST)
-        e = cudaMalloc(&out_d, bytes);
+    // the products are written 16 bytes at a time too
+    const bool out_owned = ptr_kind == STAG_PTR_HOST || !links_aligned(lng);
+    if (out_owned && (e = cudaMalloc(&out_d, bytes)) != cudaSuccess)
+        out_d = nullptr;
     if (e == cudaSuccess)
         e = launch_long_links(lat->geom, fat_d, out_d, lat->stream);
-    if (e == cudaSuccess && ptr_kind == STAG_PTR_HOST)
-        e = cudaMemcpyAsync(lng, out_d, bytes, cudaMemcpyDeviceToHost, lat->stream);
+    if (e == cudaSuccess && out_owned)
+        e = cudaMemcpyAsync(lng, out_d, bytes, ptr_kind == STAG_PTR_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDefault,
+                            lat->stream);
     cudaError_t e2 = cudaStreamSynchronize(lat->stream);
     if (owned)
         cudaFree(fat_d);
-    if (ptr_kind == STAG_PTR_HOST && out_d)
+    if (out_owned && out_d)
         cudaFree(out_d);
     if (e == cudaSuccess)
         e = e2;
