@@ -11,6 +11,8 @@
 
 namespace stag {
 
+constexpr int kSMs = 152;  // of a GB300
+
 // --------------------------------------------------------------------------
 // double-float: value = hi + lo, |lo| <= ulp(hi)/2.  Products use the FMA
 // error-free transformation, sums Knuth's TwoSum, so that one multiply-add

@@ -346,7 +346,7 @@ STAG_D void pair16_body(const DslashArgs &a) {
 }
 
 // One launch of the stencil.  The capped form asks for kCapThreads resident
-// threads per SM.  Left free, the compiler gives the uncompressed FP32
+// threads per SM, or 1024 where that takes a wave less (cap_blocks).  Left free, the compiler gives the uncompressed FP32
 // kernels so few registers (40) that too few loads are in flight; the
 // launcher picks the capped form for FP32 and 16-bit links (kCapped) and the
 // free one for the rest.  The free double-float kernel asks for 768 (80
@@ -366,8 +366,33 @@ __global__ void __launch_bounds__(BLOCK, P == P_DF64 ? (768 + BLOCK - 1) / BLOCK
 template <int P, int CM>
 constexpr int kCapThreads = P == P_F32 ? (CM == 3 ? 768 : 896) : P == P_F16 && CM == 3 ? 768 : 1024;
 
-template <int P, int EPI, int BLOCK, int CM>
-__global__ void __launch_bounds__(BLOCK, (kCapThreads<P, CM> + BLOCK - 1) / BLOCK) dslash_kernel_capped(DslashArgs a) {
+// Blocks per SM that the capped form of a launch of `grid` blocks asks for.
+// A block lasts as long in an almost empty last wave as in a full one, so FP32
+// takes 1024 threads per SM where that saves enough waves, and elsewhere the
+// fewer threads with more registers, whose wave is the shorter one.  D_oe at
+// 1024 against the fewer threads (waves): full links 147456 sites 25.8 / 30.7
+// us (1, 2), 278528: 46.8 / 51.2 (2, 3), 557056: 90.6 / 93.5 (4, 5), 704512:
+// 114.6 / 116.4 (5, 6), but 163840: 35.3 / 31.7 (2, 2), 851968: 139.7 / 139.6
+// (6, 7); three-link only 294912: 42.1 / 46.6 (2, 3), 163840: 31.3 / 29.2;
+// 12-real 131072: 17.2 / 20.4 (1, 2), 262144: 32.3 / 34.1 (2, 3), 606208: 68.6
+// / 70.4 (4, 6), but 163840: 27.0 / 23.6 (2, 2), 507904: 61.2 / 60.5 (4, 5).
+// In a solve, which keeps links in L2, the 12-real form gains nothing by it (an
+// iteration of mixed CG at 139264 sites 68.0 / 66.4, 253952: 101.4 / 99.7; full
+// links 139264: 76.3 / 82.1): there it holds for single calls (keep 0) only.
+template <int P, int CM> STAG_HD constexpr int cap_blocks_least(int block) {
+    return (kCapThreads<P, CM> + block - 1) / block;
+}
+template <int P, int CM> STAG_HD constexpr int cap_blocks(int block, int grid, int keep) {
+    const int least = cap_blocks_least<P, CM>(block), most = 1024 / block;
+    if (P != P_F32 || least >= most || (CM == 3 && keep > 0))
+        return least;
+    const int waves = (grid + kSMs * least - 1) / (kSMs * least);
+    const int waves1024 = (grid + kSMs * most - 1) / (kSMs * most);
+    return (CM == 3 ? 4 * waves1024 < 3 * waves : 6 * waves1024 <= 5 * waves) ? most : least;
+}
+
+template <int P, int EPI, int BLOCK, int CM, int NBLK>
+__global__ void __launch_bounds__(BLOCK, NBLK) dslash_kernel_capped(DslashArgs a) {
     dslash_body<P, EPI, BLOCK, CM>(a);
 }
 

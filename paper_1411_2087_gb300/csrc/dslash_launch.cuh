@@ -12,6 +12,18 @@ namespace stag {
 template <int P>
 constexpr bool kCapped = P == P_F16 || P == P_F32;
 
+template <int P, int EPI, int BLOCK, int CM>
+static void launch_capped(int grid, const DslashArgs &a, cudaStream_t s) {
+    constexpr int least = cap_blocks_least<P, CM>(BLOCK);
+    const int blocks = cap_blocks<P, CM>(BLOCK, grid, a.keep);
+    if constexpr (P == P_F32 && least < 1024 / BLOCK)
+        if (blocks > least) {
+            dslash_kernel_capped<P, EPI, BLOCK, CM, 1024 / BLOCK><<<grid, BLOCK, 0, s>>>(a);
+            return;
+        }
+    dslash_kernel_capped<P, EPI, BLOCK, CM, least><<<grid, BLOCK, 0, s>>>(a);
+}
+
 // The plain stencil and the M stencil with <p, Mp> partials (the solvers'
 // two kernels per iteration) are instantiated in both register variants, so
 // that the autotuner can time them; the other epilogues use the default.
@@ -22,11 +34,11 @@ static void launch_one(int grid, const DslashArgs &a, cudaStream_t s) {
                                                                                  : kCapped<P>;
     if constexpr (tunable) {
         if (capped)
-            dslash_kernel_capped<P, EPI, BLOCK, CM><<<grid, BLOCK, 0, s>>>(a);
+            launch_capped<P, EPI, BLOCK, CM>(grid, a, s);
         else
             dslash_kernel<P, EPI, BLOCK, CM><<<grid, BLOCK, 0, s>>>(a);
     } else if constexpr (kCapped<P>) {
-        dslash_kernel_capped<P, EPI, BLOCK, CM><<<grid, BLOCK, 0, s>>>(a);
+        launch_capped<P, EPI, BLOCK, CM>(grid, a, s);
     } else {
         dslash_kernel<P, EPI, BLOCK, CM><<<grid, BLOCK, 0, s>>>(a);
     }

@@ -210,7 +210,7 @@ cudaError_t launch_scan_links(const double *f0, const double *f1, long long nlin
     if (e != cudaSuccess)
         return e;
     const long long blocks = (nlinks + 127) / 128;
-    const int most = 152 * SCAN_BLOCKS_PER_SM;
+    const int most = kSMs * SCAN_BLOCKS_PER_SM;
     const dim3 grid((unsigned)(blocks < most ? blocks : most), nf);
     if (su3)
         scan_links_kernel<true><<<grid, SCAN_BLOCK, 0, s>>>((const double2 *)f0, (const double2 *)f1, nlinks, out);

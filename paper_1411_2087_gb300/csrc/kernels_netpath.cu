@@ -998,7 +998,7 @@ cudaError_t launch_net_resid_loss(const Geom &g, const NetPairs &pairs, float2 *
 }
 
 cudaError_t launch_net_dot2(int Vh, const float2 *a, int as, const float2 *b, int bs, double *out, cudaStream_t s) {
-    net_dot2_kernel<<<4 * 152, NET_SUM_BLOCK, 0, s>>>(Vh, a, as, b, bs, out);
+    net_dot2_kernel<<<4 * kSMs, NET_SUM_BLOCK, 0, s>>>(Vh, a, as, b, bs, out);
     return cudaGetLastError();
 }
 

@@ -119,7 +119,7 @@ STAG_D bool grid_sum(T v, double *partial, unsigned *ticket, double *smem, doubl
 // as long on its fence and ticket as on its loads (16-bit update at 1048576
 // sites: 25 us, now 21; a mixed solve on 48^3x96 598 -> 583 ms).  Not where
 // some threads would take two sites and most one (331776 sites: 19.3 -> 20.4).
-constexpr int SUM_BLOCKS = 8 * 152;
+constexpr int SUM_BLOCKS = 8 * kSMs;
 inline int sum_grid(int n, int block) {
     const int need = (n + block - 1) / block;
     return need <= 2 * SUM_BLOCKS ? need : SUM_BLOCKS;

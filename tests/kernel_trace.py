@@ -1,0 +1,23 @@
+"""Which kernels a call launches, by name (with template arguments), for tests
+that have to know which of several forms ran."""
+import time
+
+import pytest
+
+
+def launched(call):
+    """Names of the kernels that call() launches outside graphs, in order."""
+    import torch
+    from torch.profiler import ProfilerActivity, profile
+
+    for _ in range(3):  # the first trace of a process can come back empty
+        torch.cuda.synchronize()
+        with profile(activities=[ProfilerActivity.CUDA]) as p:
+            time.sleep(0.02)  # kernels at the very ends of a trace are dropped
+            call()
+            torch.cuda.synchronize()
+            time.sleep(0.02)
+        names = [e.name.split("(")[0].replace("stag::", "") for e in p.events() if e.name.startswith(("void stag::", "stag::"))]
+        if names:
+            return names
+    pytest.skip("no kernel trace on this machine")
