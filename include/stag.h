@@ -343,8 +343,9 @@ int stag_cg_solve_batched_mixed(int n, stag_lattice *lats, stag_field *xs, const
  * the environment variable STAG_TUNE_CACHE names a file, the cache is read
  * from it at the first call and every new choice appended to it.  Every
  * candidate computes the same numbers (the block size only changes the order
- * of the solvers' partial sums).  On small lattices (double-float up to
- * 400000 sites per parity, FP64 36000, FP32 85000, on 12-real links 24576) the
+ * of the solvers' partial sums).  On small lattices (double-float up to 70000
+ * sites per parity and from 116737 to 400000, FP64 up to 36000, FP32 up to
+ * 60000, in solves 70000 and in training 85000, on 12-real links 24576) the
  * Dslash has one form without these choices, and all candidates are that form.
  * Needs a gauge copy of `prec`; overwrites
  * the lattice's internal work vectors. */

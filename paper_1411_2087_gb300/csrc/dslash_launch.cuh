@@ -67,7 +67,7 @@ static cudaError_t launch_split_g(int epi, const DslashArgs &a, cudaStream_t s) 
 
 template <int P, int CM>
 static cudaError_t launch_split(int epi, const DslashArgs &a, cudaStream_t s) {
-    switch (split_warps(P, a.compressed, a.g)) {
+    switch (split_warps(P, a)) {
     case 4: return launch_split_g<P, 4, CM>(epi, a, s);
     case 8: return launch_split_g<P, 8, CM>(epi, a, s);
     default: return cudaErrorInvalidValue;
@@ -123,7 +123,7 @@ static cudaError_t launch_p_b(int epi, const DslashArgs &a, cudaStream_t s) {
 
 template <int P> cudaError_t launch_dslash_p(int epi, const DslashArgs &a, int block, cudaStream_t s) {
     if constexpr (P != P_F16) {
-        if (split_warps(P, a.compressed, a.g) > 0) {
+        if (split_warps(P, a) > 0) {
             if constexpr (P == P_F32) {
                 if (a.compressed == 2)
                     return launch_split<P, 2>(epi, a, s);

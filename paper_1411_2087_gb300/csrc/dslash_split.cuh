@@ -12,8 +12,9 @@
 // rather than sixteen unrolled copies: 8 KB of instructions instead of 110.
 // At 896 resident threads per SM (72 registers in double float; 768 and
 // 1024 measured slower at 32768 to 128000 sites) the finer blocks also fill
-// the last wave better, which keeps the form ahead up to 331776 sites.
-// split_warps (kernels_dslash.cu) says where it runs.
+// the last wave better, which keeps the form ahead up to 331776 sites except
+// where one thread per site takes a single, nearly full wave.  split_warps
+// (kernels_dslash.cu) says where it runs.
 #pragma once
 #include "dslash.cuh"
 

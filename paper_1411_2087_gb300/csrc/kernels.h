@@ -16,9 +16,9 @@ int dslash_default_block(int prec);
 // dslash_max_blocks of a lattice)
 int dslash_blocks(int prec, int epi, const DslashArgs &a, int block);
 inline size_t dslash_max_blocks(long long Vh) { return (size_t)(Vh + 31) / 32; }
-// warps per 32 sites of the split form (dslash_split.cuh) on this lattice;
+// warps per 32 sites of the split form (dslash_split.cuh) of this launch;
 // 0: one thread per site
-int split_warps(int prec, int compressed, const Geom &g);
+int split_warps(int prec, const DslashArgs &a);
 // DslashArgs::keep of a solver's launches
 int link_keep_sites(int prec, int compressed);
 

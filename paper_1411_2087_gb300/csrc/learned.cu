@@ -510,7 +510,9 @@ static int apply_M_f32(stag_net n, int np, const void *in, void *t, void *out, c
     const int P = STAG_F32;
     const size_t step = field_bytes(lat, P);
     // vectors per launch: the split form takes them all, the others one
-    const int per = split_warps(P, dslash_args(lat, P, STAG_ODD, in, t).compressed, lat->geom) > 0 ? np : 1;
+    DslashArgs all = dslash_args(lat, P, STAG_ODD, in, t);
+    all.nbatch = np;
+    const int per = split_warps(P, all) > 0 ? np : 1;
     for (int k = 0; k < np; k += per) {
         const char *ik = (const char *)in + k * step;
         char *tk = (char *)t + k * step, *ok = (char *)out + k * step;

@@ -4,6 +4,7 @@ import numpy as np
 import pytest
 from kernel_trace import launched
 
+import oracle
 from paper_1411_2087_gb300 import stag, synth
 
 pytestmark = pytest.mark.gpu
@@ -47,3 +48,59 @@ def test_fp32_threads_per_sm_by_waves(compress, cases):
             lat.set_tuning("f32", "dslash", 256, 2)
             lat.dslash(fo, fe)
             assert np.array_equal(fo.export(), got), Lt
+
+
+TOL = {"df64": 1e-12, "f32": 2e-6}
+TOL_M = {"df64": 1e-12, "f32": 5e-6}
+
+
+# both sides of the lines between the split form and one thread per site
+@pytest.mark.parametrize("prec,Lt,split", [("df64", 34, True), ("df64", 36, False), ("df64", 56, False),
+                                           ("df64", 58, True), ("f32", 28, True), ("f32", 30, False)])
+def test_single_calls_across_the_split_lines(prec, Lt, split):
+    dims = (16, 16, 16, Lt)
+    Vh = 2048 * Lt
+    U = links(dims, 93).cpu().numpy()
+    N = oracle.long_links(dims, U)
+    psi_e = synth.gaussian_colour_field(Vh, 94).numpy()
+    psi_o = synth.gaussian_colour_field(Vh, 95).numpy()
+    with stag.Lattice(dims) as lat:
+        lat.upload_gauge(U, N, precisions=(prec,))
+        fe, fo = lat.field(stag.EVEN, prec, psi_e), lat.field(stag.ODD, prec, psi_o)
+        oo, oe, om = lat.field(stag.ODD, prec), lat.field(stag.EVEN, prec), lat.field(stag.EVEN, prec)
+
+        def run():
+            lat.dslash(oo, fe)
+            lat.dslash(oe, fo)
+            lat.apply_M(om, fe, 0.3)
+
+        names = dslash_name(launched(run))
+        assert len(names) == 4 and all(("split" in n) == split for n in names), names
+        for got, want, tol in ((oo, oracle.dslash_parity(dims, U, N, 1, psi_e), TOL),
+                               (oe, oracle.dslash_parity(dims, U, N, 0, psi_o), TOL),
+                               (om, oracle.apply_M(dims, U, N, 0.3, psi_e), TOL_M)):
+            assert np.abs(got.export() - want).max() <= tol[prec] * np.abs(want).max()
+
+
+@pytest.mark.parametrize("inner,Lt,split", [(None, 34, True), (None, 36, False), (None, 56, False), (None, 58, True),
+                                            ("f32", 34, True), ("f32", 36, False)])
+def test_solves_across_the_split_lines(inner, Lt, split):
+    dims, mass = (16, 16, 16, Lt), 0.5
+    U = links(dims, 96).cpu().numpy()
+    N = oracle.long_links(dims, U)
+    b = synth.gaussian_colour_field(2048 * Lt, 97).numpy()
+    with stag.Lattice(dims) as lat:
+        lat.upload_gauge(U, N, precisions=("df64", "f32"))
+        fb, x = lat.field(stag.EVEN, "df64", b), lat.field(stag.EVEN, "df64")
+
+        def solve():
+            info = lat.cg_mixed(x, fb, mass, 1e-10, 2000, inner=inner) if inner else lat.cg(x, fb, mass, 1e-10, 2000)
+            assert info["return"] == stag.OK
+            r = b - oracle.apply_M(dims, U, N, mass, x.export())
+            assert np.linalg.norm(r) <= 1.05e-10 * np.linalg.norm(b)
+
+        solve()
+        lat.set_cg_launch("host")  # the same kernels, launched one by one
+        p = 1 if inner else 3
+        names = [n for n in launched(solve) if f"<{p}, " in n and "dslash" in n]
+        assert names and all(("split" in n) == split for n in names), set(names)
