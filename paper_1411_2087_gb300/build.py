@@ -2,7 +2,9 @@
 
 Every translation unit under ``csrc/`` is compiled for sm_103a in parallel,
 then linked into ``_build/libstag.so``.  A unit is recompiled when it, or any
-header it can include, is newer than its object file.
+header it can include, is newer than its object file.  The assembler's report
+(registers, spills and shared memory of each kernel) stays beside the object
+as ``_build/<unit>.ptxas``.
 """
 from __future__ import annotations
 
@@ -20,7 +22,7 @@ BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(BUILD, "libstag.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ARCH + ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC",
-                     "--expt-relaxed-constexpr", "-Xptxas", "-warn-spills"]
+                     "--expt-relaxed-constexpr", "-Xptxas", "-warn-spills,-v"]
 
 
 def nvcc() -> str:
@@ -48,13 +50,17 @@ def nccl_paths():
     return None
 
 
+def report(obj: str) -> str:
+    return os.path.splitext(obj)[0] + ".ptxas"
+
+
 def _headers():
     return (glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(CSRC, "*.h"))
             + glob.glob(os.path.join(ROOT, "include", "*.h")))
 
 
 def _stale(obj: str, src: str, newest_header: float) -> bool:
-    if not os.path.exists(obj):
+    if not os.path.exists(obj) or not os.path.exists(report(obj)):
         return True
     t = os.path.getmtime(obj)
     return t < os.path.getmtime(src) or t < newest_header
@@ -93,8 +99,10 @@ def build(verbose: bool = False, force: bool = False, jobs: int | None = None) -
         r = subprocess.run(cmd, capture_output=True, text=True)
         if r.returncode != 0:
             raise RuntimeError(f"nvcc failed on {os.path.basename(src)}:\n{r.stderr}")
+        with open(report(obj), "w") as f:
+            f.write(r.stderr)
         os.replace(tmp, obj)
-        return r.stderr
+        return "\n".join(ln for ln in r.stderr.splitlines() if "warning" in ln.lower())
 
     if todo:
         with cf.ThreadPoolExecutor(max_workers=jobs or min(len(todo), os.cpu_count() or 4)) as ex:

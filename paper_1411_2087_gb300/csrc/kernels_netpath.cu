@@ -459,16 +459,22 @@ template <> struct Chi<L12> : Chi<short2> {};
 // links' scale (1 for FP32).  The eight transported vectors go to shared
 // memory first (each thread reads back only its own), so that the loads of
 // the transport phase and the mixing's 48 live values never meet.
-// Seven resident blocks (72 registers, 28 warps per SM): a learned mixed solve
-// at 32^3x64 takes 160.9 ms at six, 160.4 at seven, 163.0 at eight, where the
-// 16-bit form spills.
+// Seven resident blocks (72 registers, 28 warps per SM) or six (80): one pass at
+// 32^3x64, 24^3x48 in us, seven against six, 16-bit input on 12-real, nine-entry
+// 16-bit links 80.5 / 86.6, 28.1 / 29.9, and 83.6 / 86.2, 28.2 / 29.0; FP32 on
+// them 81.3 / 82.1, 28.1 / 28.3, and 85.2 / 85.9; FP64 106 / 109, 39.5 / 40.9, and
+// 103 / 108, 39.6 / 41.1; FP32 links with FP32 input 124.6 / 124.0, 40.5 / 41.1, but
+// with FP64 141.0 / 138.2, 48.0 / 47.9; double-float input 87.9 / 86.1, 93.6 / 92.6
+// and, on FP32 links, 137.5 / 131.5, 45.1 / 42.6.  Eight: a learned mixed solve
+// at 32^3x64 163.0 ms against 160.4, the 16-bit form spills.
 // Q = NetPairs: the inputs of several training pairs in one launch, pair
 // blockIdx.y with the y-th part of chi (NoPairs: the one input r).
 struct NoPairs {};
-constexpr int NET_MID_MINB = 7;
+template <int P, class LT>
+constexpr int kNetMidBlocks = P == P_DF64 || (P == P_F64 && std::is_same<LT, float2>::value) ? 6 : 7;
 
 template <int P, class LT, class Q>
-__global__ void __launch_bounds__(NET_BLOCK, NET_MID_MINB)
+__global__ void __launch_bounds__(NET_BLOCK, kNetMidBlocks<P, LT>)
 net_mid_kernel(Geom g, const LT *__restrict__ NL, float ls, int bcneg, const NetPath *__restrict__ path,
                const typename Fmt<P>::Elem *__restrict__ r, int rs, void *__restrict__ chi, const int *gate,
                const __grid_constant__ Q pairs) {
@@ -580,14 +586,22 @@ net_mid_kernel(Geom g, const LT *__restrict__ NL, float ls, int bcneg, const Net
 // z(x) = c0 r(x) + sum_a (T_a chi_a)(x) on the even sites.  NET_OUT_DOTS
 // adds per-block partials of Re<z, r> (partial[blk]) and Re<z, Ap>
 // (partial[nblk + blk]; 0 without Ap) for the flexible CG.
-// Nine resident blocks (56 registers, latency-bound at eight: 66 us at
-// 32^3x64; a learned mixed solve 161.7 ms at eight, 160.9 at nine and ten,
-// 163.4 at twelve).
+// Nine resident blocks (56 registers).  Left free, the compiler gives the forms
+// without row rebuilds 40 to 48, with too few loads in flight, and the others 64:
+// one pass at 24^3x48, 32^3x64 in us, free against nine, plain on FP32 links 38.9 /
+// 36.6, 129 / 124 (16^4: 11.8 / 6.8), FP64 42.5 / 40.7, 145 / 136, eight training
+// pairs 38.7 / 36.5, 128 / 125; with the dots, 16-bit on 12-real links 25.2 / 22.4,
+// 68.8 / 66.2, on nine-entry ones 24.7 / 22.8, 78.6 / 73.7, double float 28.0 / 24.8,
+// 86.4 / 82.8 and 27.9 / 26.1, 94.4 / 89.8 (the 4 to 20 bytes that some forms spill
+// cost less).  Twelve: a learned mixed solve at 32^3x64 163.4 ms against 160.9.
+// The plain double-float form on 12-real links stays free: 18.1 / 18.1, 64.9 /
+// 65.7, at 212992 sites 12.7 / 13.2.
 enum { NET_OUT_PLAIN = 0, NET_OUT_DOTS = 1 };
-constexpr int NET_OUT_MINB = 9;
+template <int PI, class LT, int EPI>
+constexpr int kNetOutBlocks = PI == P_DF64 && EPI == NET_OUT_PLAIN && std::is_same<LT, L12>::value ? 0 : 9;
 
 template <int PI, int PO, class LT, int EPI, class Q>
-__global__ void __launch_bounds__(NET_BLOCK, NET_OUT_MINB)
+__global__ void __launch_bounds__(NET_BLOCK, kNetOutBlocks<PI, LT, EPI>)
 net_out_kernel(Geom g, const LT *__restrict__ NL, float ls, int bcneg, const NetPath *__restrict__ path,
                const void *__restrict__ chi, const typename Fmt<PI>::Elem *__restrict__ r, int rs,
                typename Fmt<PO>::Elem *__restrict__ z, int zs, const typename Fmt<PO>::Elem *__restrict__ Ap,
