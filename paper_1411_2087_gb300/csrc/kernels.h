@@ -65,10 +65,13 @@ cudaError_t launch_fold_links(const Geom &g, const double bc[4], double c1, doub
 // matrices (device; f1 may be NULL), into out[0..1] (device)
 struct LinkScan {
     unsigned long long maxbits;  // largest |re| or |im|, the double's bits
-    unsigned dev;                // largest deviation from SU(3) (with su3), the float's bits
+    unsigned dev;                // largest deviation from SU(3), the float's bits
     unsigned pad;
 };
-cudaError_t launch_scan_links(const double *f0, const double *f1, long long nlinks, bool su3, LinkScan *out,
+// deviation from SU(3): not asked for; as far as a decision at 1e-6 needs it
+// (deviations of U U^+ that FP32 shows to be below 1e-6 are left out); exact
+enum ScanSu3 { SCAN_NO_SU3, SCAN_SU3_LIMIT, SCAN_SU3_EXACT };
+cudaError_t launch_scan_links(const double *f0, const double *f1, long long nlinks, ScanSu3 su3, LinkScan *out,
                               cudaStream_t s);
 // of a scan copied to the host: the largest |entry| (infinite if the field
 // holds a NaN, an infinity or a value beyond the FP32 range), the deviation

@@ -66,8 +66,11 @@ constexpr int SCAN_BLOCK = 128;
 // of U U^+ run in FP32 first (rounding at most 8 u sum |u||v| < 4.8e-7 for
 // rows of length one); only a link that may miss 1e-6 by that repeats them in
 // double-float.  The determinant's bound in FP32 would exceed 1e-6, so it is
-// double-float always.  In FP64 this took 240 operations at 1/64 rate.
-STAG_D float su3_deviation(const double2 *A) {
+// double-float always.  In FP64 this took 240 operations at 1/64 rate.  Where
+// FP32 can tell, the products add nothing to the result, which then serves the
+// decision and is not the deviation; with EXACT they run in double-float for
+// every link.
+template <bool EXACT> STAG_D float su3_deviation(const double2 *A) {
     df re[9], im[9];
 #pragma unroll
     for (int e = 0; e < 9; e++) {
@@ -93,7 +96,7 @@ STAG_D float su3_deviation(const double2 *A) {
             const float d = fmaxf(fabsf(sr), fabsf(si));
             dev = d >= 0.f ? fmaxf(dev, d) : INFINITY;  // an overflow to NaN is no special unitary link
         }
-    if (!(dev <= 5e-7f)) {
+    if (EXACT || !(dev <= 5e-7f)) {
         dev = 0.f;
         for (int a = 0; a < 3; a++)
             for (int b = a; b < 3; b++) {
@@ -152,7 +155,7 @@ STAG_D float su3_deviation(const double2 *A) {
 // blocks hold the registers to 96; six would spill 136 bytes a thread.
 constexpr int SCAN_BLOCKS_PER_SM = 5;
 
-template <bool SU3>
+template <ScanSu3 SU3>
 __global__ void __launch_bounds__(SCAN_BLOCK, SCAN_BLOCKS_PER_SM)
 scan_links_kernel(const double2 *__restrict__ f0, const double2 *__restrict__ f1, long long nlinks, LinkScan *out) {
     __shared__ double2 tile[SCAN_BLOCK / 32][2][288];
@@ -185,8 +188,8 @@ scan_links_kernel(const double2 *__restrict__ f0, const double2 *__restrict__ f1
                 big = max(big, __double_as_longlong(A[e].x) & 0x7fffffffffffffffLL);
                 big = max(big, __double_as_longlong(A[e].y) & 0x7fffffffffffffffLL);
             }
-            if (SU3)
-                dev = fmaxf(dev, su3_deviation(A));
+            if (SU3 != SCAN_NO_SU3)
+                dev = fmaxf(dev, su3_deviation<SU3 == SCAN_SU3_EXACT>(A));
         }
         __syncwarp();
     }
@@ -198,12 +201,12 @@ scan_links_kernel(const double2 *__restrict__ f0, const double2 *__restrict__ f1
     }
     if (lane == 0) {
         atomicMax((long long *)&out[blockIdx.y].maxbits, big);
-        if (SU3)
+        if (SU3 != SCAN_NO_SU3)
             atomicMax(&out[blockIdx.y].dev, __float_as_uint(dev));
     }
 }
 
-cudaError_t launch_scan_links(const double *f0, const double *f1, long long nlinks, bool su3, LinkScan *out,
+cudaError_t launch_scan_links(const double *f0, const double *f1, long long nlinks, ScanSu3 su3, LinkScan *out,
                               cudaStream_t s) {
     const int nf = f1 ? 2 : 1;
     cudaError_t e = cudaMemsetAsync(out, 0, sizeof(LinkScan) * nf, s);
@@ -212,10 +215,12 @@ cudaError_t launch_scan_links(const double *f0, const double *f1, long long nlin
     const long long blocks = (nlinks + 127) / 128;
     const int most = kSMs * SCAN_BLOCKS_PER_SM;
     const dim3 grid((unsigned)(blocks < most ? blocks : most), nf);
-    if (su3)
-        scan_links_kernel<true><<<grid, SCAN_BLOCK, 0, s>>>((const double2 *)f0, (const double2 *)f1, nlinks, out);
-    else
-        scan_links_kernel<false><<<grid, SCAN_BLOCK, 0, s>>>((const double2 *)f0, (const double2 *)f1, nlinks, out);
+    const double2 *a = (const double2 *)f0, *b = (const double2 *)f1;
+    switch (su3) {
+    case SCAN_NO_SU3: scan_links_kernel<SCAN_NO_SU3><<<grid, SCAN_BLOCK, 0, s>>>(a, b, nlinks, out); break;
+    case SCAN_SU3_LIMIT: scan_links_kernel<SCAN_SU3_LIMIT><<<grid, SCAN_BLOCK, 0, s>>>(a, b, nlinks, out); break;
+    case SCAN_SU3_EXACT: scan_links_kernel<SCAN_SU3_EXACT><<<grid, SCAN_BLOCK, 0, s>>>(a, b, nlinks, out); break;
+    }
     return cudaGetLastError();
 }
 

@@ -160,7 +160,7 @@ extern "C" int stag_net_create(stag_lattice lat, const double *fat, int ptr_kind
     LinkScan *scan_d = (LinkScan *)n->scal;
     static_assert(sizeof(LinkScan) <= 4 * sizeof(double), "scan scratch");
     LinkScan scan = {};
-    e = launch_scan_links(fat_d, nullptr, (long long)(4 * V), true, scan_d, s);
+    e = launch_scan_links(fat_d, nullptr, (long long)(4 * V), SCAN_SU3_LIMIT, scan_d, s);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(&scan, scan_d, sizeof scan, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess)

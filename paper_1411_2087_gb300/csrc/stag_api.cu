@@ -310,14 +310,16 @@ extern "C" int stag_gauge_upload(stag_lattice lat, const double *fat, const doub
     // valid for links in SU(3) (the paper's Sec. 4 notes smeared links are not)
     float inv_scale[2] = {0.f, 0.f};
     {
-        cudaError_t e = lat->scan ? cudaSuccess : cudaMalloc(&lat->scan, 2 * sizeof(LinkScan));
         LinkScan scan[2] = {};
+        auto run_scan = [&](ScanSu3 su3) {
+            cudaError_t e = launch_scan_links(fat_d, lng_d, 4LL * lat->V, su3, lat->scan, lat->stream);
+            if (e == cudaSuccess)
+                e = cudaMemcpyAsync(scan, lat->scan, sizeof scan, cudaMemcpyDeviceToHost, lat->stream);
+            return e == cudaSuccess ? cudaStreamSynchronize(lat->stream) : e;
+        };
+        cudaError_t e = lat->scan ? cudaSuccess : cudaMalloc(&lat->scan, 2 * sizeof(LinkScan));
         if (e == cudaSuccess)
-            e = launch_scan_links(fat_d, lng_d, 4LL * lat->V, compress, lat->scan, lat->stream);
-        if (e == cudaSuccess)
-            e = cudaMemcpyAsync(scan, lat->scan, sizeof scan, cudaMemcpyDeviceToHost, lat->stream);
-        if (e == cudaSuccess)
-            e = cudaStreamSynchronize(lat->stream);
+            e = run_scan(compress ? SCAN_SU3_LIMIT : SCAN_NO_SU3);
         if (e != cudaSuccess)
             return refuse(fail(STAG_ERR_CUDA, "gauge scan: %s", cudaGetErrorString(e)));
         const double cf[2] = {std::fabs(c1), std::fabs(c3)};
@@ -332,11 +334,16 @@ extern "C" int stag_gauge_upload(stag_lattice lat, const double *fat, const doub
                 inv_scale[h] = mx > 0 ? (float)(32767.0 / mx) : 0.f;
             }
         }
-        const float dev[2] = {scan_su3_deviation(scan[0]), scan_su3_deviation(scan[1])};
-        if (compress && (((cmask & 1) && !(dev[0] <= 1e-6f)) || !(dev[1] <= 1e-6f)))
+        if (compress && (((cmask & 1) && !(scan_su3_deviation(scan[0]) <= 1e-6f)) ||
+                         !(scan_su3_deviation(scan[1]) <= 1e-6f))) {
+            e = run_scan(SCAN_SU3_EXACT);  // the message's figures
+            if (e != cudaSuccess)
+                return refuse(fail(STAG_ERR_CUDA, "gauge scan: %s", cudaGetErrorString(e)));
             return refuse(fail(STAG_ERR_ARG, "stag_gauge_upload: links deviate from SU(3) by %.2e (fat) / %.2e "
-                               "(long); 12-real compression needs special unitary links%s", dev[0], dev[1],
+                               "(long); 12-real compression needs special unitary links%s",
+                               scan_su3_deviation(scan[0]), scan_su3_deviation(scan[1]),
                                (cmask & 1) ? " (STAG_COMPRESS12_LONG compresses the long links only)" : ""));
+        }
     }
     // the copies of the last upload keep their buffers where this one has
     // the same (allocating 24^3x48 in DF64, FP32 and 16-bit anew took 1.5 ms)
