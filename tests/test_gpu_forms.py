@@ -104,3 +104,32 @@ def test_solves_across_the_split_lines(inner, Lt, split):
         p = 1 if inner else 3
         names = [n for n in launched(solve) if f"<{p}, " in n and "dslash" in n]
         assert names and all(("split" in n) == split for n in names), set(names)
+
+
+@pytest.mark.parametrize("Lt,pair", [(72, False), (76, True)])  # 147456, 155648 sites per parity
+def test_16_bit_pair_form_is_the_untuned_default(Lt, pair):
+    """16-bit D on 12-real links, nothing tuned, against the oracle (the
+    storage format's tolerance), and the bits of the one-site form."""
+    dims = (16, 16, 16, Lt)
+    Vh = 2048 * Lt
+    U = links(dims, 98).cpu().numpy()
+    N = oracle.long_links(dims, U)
+    psi_e = synth.gaussian_colour_field(Vh, 99).numpy()
+    psi_o = synth.gaussian_colour_field(Vh, 100).numpy()
+    with stag.Lattice(dims) as lat:
+        lat.upload_gauge(U, N, precisions=("f16",), compress12=True)
+        fe, fo = lat.field(stag.EVEN, "f16", psi_e), lat.field(stag.ODD, "f16", psi_o)
+        oo, oe = lat.field(stag.ODD, "f16"), lat.field(stag.EVEN, "f16")
+
+        def run():
+            lat.dslash(oo, fe)
+            lat.dslash(oe, fo)
+
+        names = dslash_name(launched(run))
+        assert len(names) == 2 and all(("pair16" in n) == pair for n in names), names
+        got = oo.export(), oe.export()
+        for g, want in zip(got, (oracle.dslash_parity(dims, U, N, 1, psi_e), oracle.dslash_parity(dims, U, N, 0, psi_o))):
+            assert np.abs(g - want).max() <= 3e-4 * np.abs(want).max()
+        lat.set_tuning("f16", "dslash", 128, 1)
+        run()
+        assert np.array_equal(oo.export(), got[0]) and np.array_equal(oe.export(), got[1])
