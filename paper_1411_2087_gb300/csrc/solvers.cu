@@ -812,9 +812,10 @@ struct BatchPlan {
 };
 
 // group systems by lattice (consecutive, at most batch_max_k per group) and
-// allocate work vectors and reduction buffers; x/b are raw buffers
+// allocate work vectors and reduction buffers; x/b are raw buffers.  lanes: the
+// Dslash of one thread per (site, system) however small the batch
 static int plan_batch(BatchPlan &P, int n, stag_lattice *lats, void *const *x, const void *const *b,
-                      int prec) {
+                      int prec, bool lanes = false) {
     // systems per group: the lattice's tuned group size, else the largest
     auto group_k = [&](stag_lattice L) { return L->batch_k[prec] > 0 ? L->batch_k[prec] : batch_max_k(prec); };
     memset(&P.a, 0, sizeof P.a);
@@ -873,7 +874,7 @@ static int plan_batch(BatchPlan &P, int n, stag_lattice *lats, void *const *x, c
     long long items = 0;
     for (int gi = 0; gi < G; gi++)
         items += (long long)P.a.grp[gi].g.Vh * P.a.grp[gi].K;
-    P.a.split = prec != STAG_F32 && items <= batch_split_items(prec);
+    P.a.split = prec != STAG_F32 && !lanes && items <= batch_split_items(prec);
     const int per = P.a.split ? SPLIT_SITES : P.block;
     for (int gi = 0; gi < G; gi++) {
         BatchGroup &gr = P.a.grp[gi];
@@ -1418,7 +1419,10 @@ static int tune_all(stag_lattice lat, int prec, std::vector<stag_tune_result> &r
     if (prec == STAG_F16)
         return STAG_OK;  // no batched kernels in 16-bit storage
     // the batched Dslash: block x systems per group, one group of K systems;
-    // the time per right-hand side decides
+    // the time per right-hand side decides.  Always the form of one thread per
+    // (site, system): a small group alone would run in split form, which has
+    // no block size to choose, and say nothing of the larger batches that it
+    // is a part of.
     const int kmax = batch_max_k(prec);
     for (int i = 0; i < kmax; i++)
         STAG_TRY(alloc_vec(lat, prec, &lat->bwork[prec][BATCH_MAX_G * BATCH_KMAX - 1 - i][0]));
@@ -1436,7 +1440,7 @@ static int tune_all(stag_lattice lat, int prec, std::vector<stag_tune_result> &r
             lat->batch_block[prec] = block;
             lat->batch_k[prec] = K;
             BatchPlan P;
-            int st = plan_batch(P, K, lats.data(), x.data(), b.data(), prec);
+            int st = plan_batch(P, K, lats.data(), x.data(), b.data(), prec, true);
             double us = 0;
             if (st == STAG_OK)
                 st = time_launch(lat, [&]() { return launch_batch(prec, BATCH_DSLASH_X, P.a, block, s); }, reps, &us);

@@ -59,3 +59,14 @@ def test_batched_forms(prec, sizes, split):
             assert r <= 1.05e-10, (dims, m, block, r)
     for lat in lats:
         lat.close()
+
+
+@pytest.mark.parametrize("prec", ["df64", "f64"])
+def test_tuner_times_the_form_with_block_sizes(prec):
+    """65536 items per group of four: alone such a group would run in split form."""
+    dims = (16, 16, 16, 8)
+    with stag.Lattice(dims) as lat:
+        lat.upload_gauge(synth.su3_field(dims, 0.3, 41).numpy(), None, precisions=(prec,))
+        names = [n for n in launched(lambda: lat.autotune_all(prec, force=True)) if "batch_dslash" in n]
+        assert names and all("batch_dslash_lanes_kernel<" in n for n in names), set(names)
+        assert {b for b in (128, 256) for n in names if f", {b}, " in n} == {128, 256}
