@@ -344,7 +344,8 @@ int stag_cg_solve_batched_mixed(int n, stag_lattice *lats, stag_field *xs, const
  * The fastest of each kind is kept for every later call on the lattice and
  * cached for the process per (dims, precision, link layout, device); when
  * the environment variable STAG_TUNE_CACHE names a file, the cache is read
- * from it at the first call and every new choice appended to it.  Every
+ * from it at the first call and every new choice appended to it; choices that
+ * a library with other kernels wrote are ignored (timed again).  Every
  * candidate computes the same numbers (the block size only changes the order
  * of the solvers' partial sums).  On small lattices (double-float up to 70000
  * sites per parity and from 116737 to 400000, FP64 up to 36000, FP32 up to

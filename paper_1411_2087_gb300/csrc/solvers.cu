@@ -1299,8 +1299,12 @@ static std::string tune_key(const stag_lattice lat, int prec) {
     return buf;
 }
 
-// the optional file cache: one line per key, "stag-tune2 <key> <six ints>"
-// (lines of other formats, such as those of earlier candidate sets, are ignored)
+// the optional file cache: one line per key, "stag-tune2 <key> <six ints>
+// <kernel set>".  Lines of other formats are ignored, and so are those of
+// another kernel set: choices timed on kernels that are no longer the ones
+// behind their numbers (none written: set 2 and before; 3: the caps by format
+// and grid, the split forms and the pair form by default).
+constexpr int kTuneKernelSet = 3;
 static const char *tune_file() { return getenv("STAG_TUNE_CACHE"); }
 
 // a choice read from the file is applied only if stag_lattice_set_tuning
@@ -1331,12 +1335,12 @@ static void tune_file_read_locked() {
         return;
     char line[512];
     while (fgets(line, sizeof line, f)) {
-        int d[4], prec, comp;
+        int d[4], prec, comp, set;
         char dev[200];
         TuneChoice c;
-        if (sscanf(line, "stag-tune2 %d %d %d %d %d %d %199s %d %d %d %d %d %d", &d[0], &d[1], &d[2], &d[3], &prec,
-                   &comp, dev, &c.dblock, &c.dregs, &c.mblock, &c.mregs, &c.bblock, &c.bk) == 13 &&
-            tune_choice_valid(prec, c)) {
+        if (sscanf(line, "stag-tune2 %d %d %d %d %d %d %199s %d %d %d %d %d %d %d", &d[0], &d[1], &d[2], &d[3], &prec,
+                   &comp, dev, &c.dblock, &c.dregs, &c.mblock, &c.mregs, &c.bblock, &c.bk, &set) == 14 &&
+            set == kTuneKernelSet && tune_choice_valid(prec, c)) {
             char key[256];
             snprintf(key, sizeof key, "%d %d %d %d %d %d %s", d[0], d[1], d[2], d[3], prec, comp, dev);
             g_tune_cache[key] = c;
@@ -1352,7 +1356,8 @@ static void tune_file_append(const std::string &key, const TuneChoice &c) {
     FILE *f = fopen(path, "a");
     if (!f)
         return;
-    fprintf(f, "stag-tune2 %s %d %d %d %d %d %d\n", key.c_str(), c.dblock, c.dregs, c.mblock, c.mregs, c.bblock, c.bk);
+    fprintf(f, "stag-tune2 %s %d %d %d %d %d %d %d\n", key.c_str(), c.dblock, c.dregs, c.mblock, c.mregs, c.bblock, c.bk,
+            kTuneKernelSet);
     fclose(f);
 }
 
