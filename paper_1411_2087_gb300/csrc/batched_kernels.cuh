@@ -17,7 +17,7 @@ STAG_D void load_active(const BatchArgs &a, const BatchGroup &G, int *act, bool 
     __syncthreads();
 }
 
-// multi-RHS Dslash: out_k = D in_k for the active systems of the group;
+// multi-RHS Dslash (FP32): out_k = D in_k for the active systems of the group;
 // EPI_M_PAP: out_k = m_k^2 p_k - D in_k and <p_k, out_k> -> alpha_k;
 // EPI_RESID: |b_k - (m_k^2 p_k - D in_k)|^2 -> true_rr_k
 template <int P, int EPI, int BLOCK, int K>
@@ -238,8 +238,8 @@ STAG_D const void *batch_lane_input(const BatchGroup &G, int k, int src_x) {
 // Lane-mapped multi-RHS Dslash (double-float and FP64): thread t of the
 // group's range handles site t / GK for system t % GK (GK = systems in the
 // group), with the single-site stencil; epilogues as batch_dslash_kernel.
-// Bound by the FMA pipe in double-float (4 x 576 multiply-adds of 12 FP32
-// operations per site).  The hops of one direction are unrolled and the four
+// Bound by the FMA pipe in double-float (4 x 576 multiply-adds of ten FP32
+// operations per site; the figures below were taken with twelve).  The hops of one direction are unrolled and the four
 // directions a loop: all sixteen unrolled are 110 KB of code, which the warps
 // of an SM, each elsewhere in it, fetch again and again.  An iteration of a
 // batched solve of four systems on 24^3x48 in double float: 1083 us unrolled
@@ -524,12 +524,17 @@ cudaError_t launch_batch_pbk(int what, const BatchArgs &a, cudaStream_t s) {
         default: break;
         }
     }
+    if constexpr (P == P_F32) {
+        switch (what) {
+        case BATCH_DSLASH_OE: batch_dslash_kernel<P, EPI_NONE, BLOCK, K><<<grid, BLOCK, 0, s>>>(a, 1, 0); return cudaGetLastError();
+        case BATCH_DSLASH_X: batch_dslash_kernel<P, EPI_NONE, BLOCK, K><<<grid, BLOCK, 0, s>>>(a, 1, 1); return cudaGetLastError();
+        case BATCH_M_PAP: batch_dslash_kernel<P, EPI_M_PAP, BLOCK, K><<<grid, BLOCK, 0, s>>>(a, 0, 0); return cudaGetLastError();
+        case BATCH_RESID: batch_dslash_kernel<P, EPI_RESID, BLOCK, K><<<grid, BLOCK, 0, s>>>(a, 0, 0); return cudaGetLastError();
+        default: break;
+        }
+    }
     switch (what) {
     case BATCH_INIT: batch_init_kernel<P, BLOCK, K><<<grid, BLOCK, 0, s>>>(a); break;
-    case BATCH_DSLASH_OE: batch_dslash_kernel<P, EPI_NONE, BLOCK, K><<<grid, BLOCK, 0, s>>>(a, 1, 0); break;
-    case BATCH_DSLASH_X: batch_dslash_kernel<P, EPI_NONE, BLOCK, K><<<grid, BLOCK, 0, s>>>(a, 1, 1); break;
-    case BATCH_M_PAP: batch_dslash_kernel<P, EPI_M_PAP, BLOCK, K><<<grid, BLOCK, 0, s>>>(a, 0, 0); break;
-    case BATCH_RESID: batch_dslash_kernel<P, EPI_RESID, BLOCK, K><<<grid, BLOCK, 0, s>>>(a, 0, 0); break;
     case BATCH_UPDATE: batch_update_kernel<P, BLOCK, K><<<grid, BLOCK, 0, s>>>(a); break;
     case BATCH_P: batch_p_kernel<P, BLOCK, K><<<grid, BLOCK, 0, s>>>(a); break;
     default: return cudaErrorInvalidValue;

@@ -90,14 +90,6 @@ STAG_D df df_add(df a, df b) {
 }
 STAG_D df df_sub(df a, df b) { return df_add(a, -b); }
 
-STAG_D df df_mul(df a, df b) {
-    const float p = __fmul_rn(a.hi, b.hi);
-    float e = __fmaf_rn(a.hi, b.hi, -p);
-    e = __fmaf_rn(a.hi, b.lo, e);
-    e = __fmaf_rn(a.lo, b.hi, e);
-    return df_norm(df_make(p, e));
-}
-
 // --------------------------------------------------------------------------
 // generic real arithmetic used by the stencil templates
 // --------------------------------------------------------------------------

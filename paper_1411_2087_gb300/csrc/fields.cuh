@@ -100,7 +100,6 @@ template <> struct Fmt<P_F64> {
     STAG_D static double2 pack(const cplx<R> &c) { return make_double2(c.re, c.im); }
     STAG_D static cplx<R> make(double re, double im) { return cplx<R>{re, im}; }
     STAG_D static cplx<R> unpack_link(double2 e, float) { return unpack(e); }
-    STAG_D static double2 pack_link(double re, double im, float) { return make_double2(re, im); }
 };
 
 template <> struct Fmt<P_DF64> {
@@ -112,7 +111,6 @@ template <> struct Fmt<P_DF64> {
         return cplx<R>{df_from_double(re), df_from_double(im)};
     }
     STAG_D static cplx<R> unpack_link(float4 e, float) { return unpack(e); }
-    STAG_D static float4 pack_link(double re, double im, float) { return pack(make(re, im)); }
 };
 
 template <> struct Fmt<P_F32> {
@@ -122,7 +120,6 @@ template <> struct Fmt<P_F32> {
     STAG_D static float2 pack(const cplx<R> &c) { return make_float2(c.re, c.im); }
     STAG_D static cplx<R> make(double re, double im) { return cplx<R>{(float)re, (float)im}; }
     STAG_D static cplx<R> unpack_link(float2 e, float) { return unpack(e); }
-    STAG_D static float2 pack_link(double re, double im, float) { return make_float2((float)re, (float)im); }
 };
 
 // 16-bit storage: signed fixed point q = round(v / scale * 32767), float
@@ -157,10 +154,6 @@ template <> struct Fmt<P_F16> {
     STAG_D static cplx<R> unpack_link(short2 e, float scale) {
         return cplx<R>{(float)e.x * scale, (float)e.y * scale};
     }
-    // inv_scale = 32767 / field max
-    STAG_D static short2 pack_link(double re, double im, float inv_scale) {
-        return make_short2(q16((float)re * inv_scale), q16((float)im * inv_scale));
-    }
 };
 
 // --------------------------------------------------------------------------
@@ -184,10 +177,6 @@ template <> struct C12<P_F32> {
             L[2 * k + 1] = cplx<float>{v.z, v.w};
         }
     }
-    STAG_D static void store(char *kind_base, size_t S, size_t idx, int e, double re, double im, float) {
-        float2 *p = (float2 *)((float4 *)kind_base + (e / 2) * S + idx) + (e % 2);
-        *p = make_float2((float)re, (float)im);
-    }
 };
 
 template <> struct C12<P_F16> {
@@ -204,10 +193,6 @@ template <> struct C12<P_F16> {
         L[3] = q(a.w, scale);
         L[4] = q(b.x, scale);
         L[5] = q(b.y, scale);
-    }
-    STAG_D static void store(char *kind_base, size_t S, size_t idx, int e, double re, double im, float inv_scale) {
-        short2 *p = e < 4 ? (short2 *)kind_base + idx * 4 + e : (short2 *)(kind_base + 16 * S) + idx * 2 + (e - 4);
-        *p = make_short2(q16((float)re * inv_scale), q16((float)im * inv_scale));
     }
 };
 
@@ -231,16 +216,8 @@ STAG_HD size_t link_kind_offset(int p, int mask, int kind, size_t S) {
 }
 STAG_HD size_t link_parity_bytes(int p, int mask, size_t S) { return link_kind_offset(p, mask, 8, S); }
 
-// the full 16-bit kind: where entry e of link idx lives, and its nine raw
-// int16 pairs in three loads
+// the full 16-bit kind: the nine raw int16 pairs of link idx in three loads
 struct L16 {
-    STAG_D static short2 *slot(char *kb, size_t S, size_t idx, int e) {
-        if (e < 4)
-            return (short2 *)kb + idx * 4 + e;
-        if (e < 8)
-            return (short2 *)(kb + 16 * S) + idx * 4 + (e - 4);
-        return (short2 *)(kb + 32 * S) + idx;
-    }
     template <int LD> STAG_D static void load(const char *kb, size_t S, int idx, l2pol pol, int w[9]) {
         const int4 a = ld_link<LD>((const int4 *)kb + idx, pol);
         const int4 b = ld_link<LD>((const int4 *)(kb + 16 * S) + idx, pol);

@@ -125,38 +125,4 @@ inline int sum_grid(int n, int block) {
     return need <= 2 * SUM_BLOCKS ? need : SUM_BLOCKS;
 }
 
-// Grid-wide sum of two values per thread (same protocol as grid_sum;
-// partial must hold 2 * gridDim.x doubles).
-template <int BLOCK, class T>
-STAG_D bool grid_sum2(T v0, T v1, double *partial, unsigned *ticket, double *smem,
-                      double &t0, double &t1) {
-    __shared__ bool last;
-    const double s0 = block_sum<BLOCK>(v0, smem);
-    const double s1 = block_sum<BLOCK>(v1, smem);
-    if (threadIdx.x == 0) {
-        partial[2 * blockIdx.x] = s0;
-        partial[2 * blockIdx.x + 1] = s1;
-        __threadfence();
-        const unsigned t = atomicAdd(ticket, 1u);
-        last = (t == gridDim.x - 1);
-    }
-    __syncthreads();
-    if (!last)
-        return false;
-    __threadfence();
-    const double a0 = block_sum<BLOCK>(partials_share<BLOCK>(partial, (int)gridDim.x, 2), smem);
-    const double a1 = block_sum<BLOCK>(partials_share<BLOCK>(partial + 1, (int)gridDim.x, 2), smem);
-    __shared__ double res[2];
-    if (threadIdx.x == 0) {
-        res[0] = a0;
-        res[1] = a1;
-        *ticket = 0u;
-    }
-    __syncthreads();
-    t0 = res[0];
-    t1 = res[1];
-    __syncthreads();
-    return true;
-}
-
 }  // namespace stag
