@@ -339,8 +339,8 @@ int stag_cg_solve_batched_mixed(int n, stag_lattice *lats, stag_field *xs, const
  *                     (group: FP32 4 or 8, F64/DF64 2 or 4; decided by the
  *                     time per right-hand side; F64/DF64: of the kernel that
  *                     batches of more than 100000/70000 sites times
- *                     right-hand sides run, smaller ones have a form without
- *                     block sizes); none in 16-bit storage
+ *                     right-hand sides run, most smaller ones have a form
+ *                     without block sizes); none in 16-bit storage
  * The fastest of each kind is kept for every later call on the lattice and
  * cached for the process per (dims, precision, link layout, device); when
  * the environment variable STAG_TUNE_CACHE names a file, the cache is read

@@ -120,9 +120,9 @@ struct BatchArgs;
 cudaError_t launch_batch(int prec, int what, const BatchArgs &a, int block, cudaStream_t s);
 int batch_max_k(int prec);
 int batch_min_k(int prec);
-// batches of at most this many (site, system) items run the lane-mapped
-// Dslash in split form
-long long batch_split_items(int prec);
+// whether a batch of `items` (site, system) pairs runs the lane-mapped Dslash
+// in split form
+bool batch_split(int prec, long long items);
 
 // record the calling thread's last error message (read back by
 // stag_last_error_message) and return `code`

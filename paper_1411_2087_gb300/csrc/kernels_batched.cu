@@ -26,10 +26,19 @@ int batch_max_k(int prec) { return prec == P_F32 ? 8 : 4; }
 int batch_min_k(int prec) { return prec == P_F32 ? 4 : 2; }
 
 // An iteration in split form against one thread per (site, system): double
-// float 4096 items 35 / 50 us, 27648: 51 / 60, 55296: 87.5 / 83.5, 65536: 80.5
-// / 83, 98304: 114 / 119, 131072: 148 / 134; FP64 4096: 44 / 82, 41472: 132 /
-// 154, 98304: 254 / 278, 131072: 326 / 323.
-long long batch_split_items(int prec) { return prec == P_F64 ? 100000 : prec == P_DF64 ? 70000 : 0; }
+// float 4096 items 35 / 50 us, 27648: 51 / 60, 61440: 83.8 / 86.4, 65536: 92.2
+// / 92.8, 73728: 94.3 / 88.0, 98304: 117.7 / 113.3; FP64 4096: 44 / 82, 41472:
+// 132 / 154, 61440: 172 / 193, 65536: 190 / 202, 73728: 204 / 196, 81920: 225 /
+// 245, 98304: 264 / 284, 114688: 288 either way.  (FP64 at 73728: the split form
+// is past two waves of 1064 blocks of 32 items, the other within one of 608
+// blocks of 128.)
+bool batch_split(int prec, long long items) {
+    switch (prec) {
+    case P_DF64: return items <= 70000;
+    case P_F64: return items <= 2 * 7 * 32 * kSMs || (items > 4 * 128 * kSMs && items <= 100000);
+    default: return false;
+    }
+}
 
 cudaError_t launch_batch(int prec, int what, const BatchArgs &a, int block, cudaStream_t s) {
     if (block != 128 && block != 256)

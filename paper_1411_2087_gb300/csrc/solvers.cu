@@ -874,7 +874,7 @@ static int plan_batch(BatchPlan &P, int n, stag_lattice *lats, void *const *x, c
     long long items = 0;
     for (int gi = 0; gi < G; gi++)
         items += (long long)P.a.grp[gi].g.Vh * P.a.grp[gi].K;
-    P.a.split = prec != STAG_F32 && !lanes && items <= batch_split_items(prec);
+    P.a.split = !lanes && batch_split(prec, items);
     const int per = P.a.split ? SPLIT_SITES : P.block;
     for (int gi = 0; gi < G; gi++) {
         BatchGroup &gr = P.a.grp[gi];

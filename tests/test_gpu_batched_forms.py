@@ -1,6 +1,6 @@
 """The two forms of the batched double-float and FP64 Dslash: one thread per
-(site, system) above 70000 (FP64: 100000) items of a batch, at both block
-sizes, and the split form below, with groups of three systems, whose blocks
+(site, system) above 70000 (FP64: 100000, and 68097 to 77824) items of a batch,
+at both block sizes, and the split form below, with groups of three systems, whose blocks
 end inside a site.  Residuals recomputed by the oracle, and the kernel that
 ran read from a trace."""
 import numpy as np
@@ -23,6 +23,8 @@ pytestmark = pytest.mark.gpu
     ("f64", [(16, 3)], True),            # 98304
     ("f64", [(6, 7), (2, 3)], True),     # 98304
     ("f64", [(18, 3)], False),           # 110592
+    ("f64", [(12, 3)], False),           # 73728: one wave of the other form
+    ("f64", [(10, 4)], True),            # 81920
     ("f64", [(8, 7), (2, 3)], False),    # 126976
 ])
 def test_batched_forms(prec, sizes, split):
