@@ -185,8 +185,10 @@ int assemble(const Domains &D, int i, const void *global) {
     return copy_slices(D, global, x.buf, x.t0 - kHalo, x.nt + 2 * kHalo);
 }
 
-// domain i's Dslash from its assembled input: the outputs of its slab
-int domain_dslash(const Domains &D, int i, int out_par, int epi, void *out, const void *p, double m2) {
+// domain i's Dslash from its assembled input: the outputs of its slab (call:
+// a Dslash call of its own, in the form of stag_dslash_*: the same bits)
+int domain_dslash(const Domains &D, int i, int out_par, int epi, void *out, const void *p, double m2,
+                  bool call = false) {
     const Domain &x = D.d[i];
     stag_lattice lat = D.lat;
     DslashArgs a = dslash_args(lat, D.prec, out_par, x.buf, out);
@@ -200,6 +202,8 @@ int domain_dslash(const Domains &D, int i, int out_par, int epi, void *out, cons
     a.sc = x.sc;
     a.m2 = make_dpair(m2);
     a.m2_in_args = 1;
+    if (call)
+        a.keep = 0;
     CUDA_TRY(launch_dslash(D.prec, epi, a, lat->dslash_block[D.prec], lat->stream));
     return STAG_OK;
 }
@@ -261,7 +265,7 @@ extern "C" int stag_dd_dslash(stag_lattice lat, int ndomains, stag_field out, co
     STAG_TRY(make_domains(D, ndomains));
     for (int i = 0; i < ndomains; i++) {
         STAG_TRY(assemble(D, i, in->data));
-        STAG_TRY(domain_dslash(D, i, out->parity, EPI_NONE, out->data, nullptr, 0.0));
+        STAG_TRY(domain_dslash(D, i, out->parity, EPI_NONE, out->data, nullptr, 0.0, true));
     }
     CUDA_TRY(cudaStreamSynchronize(lat->stream));
     return STAG_OK;

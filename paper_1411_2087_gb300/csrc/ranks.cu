@@ -344,9 +344,10 @@ static int exchange_halo(stag_ddr d, int prec, void *field, cudaStream_t s) {
 
 // the stencil on slices [t, t + n) (and [t2, t2 + n2) in the same launch)
 // of the slab, with the halo of `in` filled where they need it; EPI_M_PART
-// writes its block partials from d->partial + *np on and advances *np
+// writes its block partials from d->partial + *np on and advances *np.  call:
+// a Dslash call of its own, in the form of stag_dslash_* (the same bits)
 static int slab_range(stag_ddr d, int prec, int out_par, int epi, const void *in, void *out, const void *p,
-                      const void *b, double m2, int t, int n, int t2, int n2, int *np) {
+                      const void *b, double m2, int t, int n, int t2, int n2, int *np, bool call = false) {
     stag_lattice lat = d->lat;
     if (n <= 0)
         return STAG_OK;
@@ -356,6 +357,8 @@ static int slab_range(stag_ddr d, int prec, int out_par, int epi, const void *in
     a.cn = n * P;
     a.c0b = t2 * P;
     a.cnb = n2 > 0 ? n2 * P : 0;
+    if (call)
+        a.keep = 0;
     a.p = p;
     a.b = b;
     a.sc = d->sc;
@@ -381,25 +384,26 @@ static int slab_range(stag_ddr d, int prec, int out_par, int epi, const void *in
 // One rank owns the whole lattice: its halo is its own slices, so there is
 // nothing to exchange.
 static int slab_dslash(stag_ddr d, int prec, int out_par, int epi, const void *in, void *out, const void *p,
-                       double m2, int *np) {
+                       double m2, int *np, bool call = false) {
     stag_lattice lat = d->lat;
     cudaStream_t s = lat->stream;
     const int t0 = d->slab.t0, nt = d->slab.nt, h = kHaloSlices;
     if (np)
         *np = 0;
     if (d->comm.size == 1)
-        return slab_range(d, prec, out_par, epi, in, out, p, nullptr, m2, t0, nt, 0, 0, np);
+        return slab_range(d, prec, out_par, epi, in, out, p, nullptr, m2, t0, nt, 0, 0, np, call);
     if (nt <= 2 * h) {
         STAG_TRY(exchange_halo(d, prec, (void *)in, s));
-        return slab_range(d, prec, out_par, epi, in, out, p, nullptr, m2, t0, nt, 0, 0, np);
+        return slab_range(d, prec, out_par, epi, in, out, p, nullptr, m2, t0, nt, 0, 0, np, call);
     }
     CUDA_TRY(cudaEventRecord(d->ev_in, s));
     CUDA_TRY(cudaStreamWaitEvent(d->side, d->ev_in, 0));
-    STAG_TRY(slab_range(d, prec, out_par, epi, in, out, p, nullptr, m2, t0 + h, nt - 2 * h, 0, 0, np));
+    STAG_TRY(slab_range(d, prec, out_par, epi, in, out, p, nullptr, m2, t0 + h, nt - 2 * h, 0, 0, np,
+                        call));
     STAG_TRY(exchange_halo(d, prec, (void *)in, d->side));
     CUDA_TRY(cudaEventRecord(d->ev_halo, d->side));
     CUDA_TRY(cudaStreamWaitEvent(s, d->ev_halo, 0));
-    return slab_range(d, prec, out_par, epi, in, out, p, nullptr, m2, t0, h, t0 + nt - h, h, np);
+    return slab_range(d, prec, out_par, epi, in, out, p, nullptr, m2, t0, h, t0 + nt - h, h, np, call);
 }
 
 // sum one device double over the ranks, in place, in order on the lattice
@@ -469,7 +473,7 @@ extern "C" int stag_ddr_dslash(stag_ddr d, stag_field out, stag_field in) {
         return fail(STAG_ERR_STATE, "stag_ddr_dslash: no %s gauge copy uploaded", prec_name(prec));
     DEVICE_SCOPE(lat->device);
     STAG_TRY(put_scalars(d, 0.0, 0.0, 0.0));  // running: the stencil's gate
-    STAG_TRY(slab_dslash(d, prec, out->parity, EPI_NONE, in->data, out->data, nullptr, 0.0, nullptr));
+    STAG_TRY(slab_dslash(d, prec, out->parity, EPI_NONE, in->data, out->data, nullptr, 0.0, nullptr, true));
     CUDA_TRY(cudaStreamSynchronize(lat->stream));
     return STAG_OK;
 }

@@ -133,3 +133,24 @@ def test_16_bit_pair_form_is_the_untuned_default(Lt, pair):
         lat.set_tuning("f16", "dslash", 128, 1)
         run()
         assert np.array_equal(oo.export(), got[0]) and np.array_equal(oe.export(), got[1])
+
+
+@pytest.mark.parametrize("prec,compress,Lt", [("f32", False, 32), ("f32", True, 72), ("df64", False, 34),
+                                              ("f16", True, 76)])
+def test_decomposed_dslash_takes_the_single_calls_form(prec, compress, Lt):
+    """Between the single calls' line and the solves' (and where their launches
+    differ otherwise) the slab-decomposed Dslash keeps the single call's bits."""
+    dims = (16, 16, 16, Lt)
+    with stag.Lattice(dims) as lat:
+        lat.upload_gauge(links(dims, 101), None, precisions=(prec,), compress12=compress)
+        fe = lat.field(stag.EVEN, prec, synth.gaussian_colour_field(2048 * Lt, 102).numpy())
+        one, slabs, rank = (lat.field(stag.ODD, prec) for _ in range(3))
+        lat.dslash(one, fe)
+        lat.dd_dslash(slabs, fe, 3)
+        comm = stag.HostComm(0, 1, lambda p, n: (n, p), lambda v: v)
+        d = stag.DDRank(lat, comm)
+        d.dslash(rank, fe)
+        want = one.export()
+        assert np.array_equal(slabs.export(), want)
+        assert np.array_equal(rank.export(), want)
+        d.close()
