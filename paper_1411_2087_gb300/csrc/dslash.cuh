@@ -49,7 +49,7 @@ struct DslashArgs {
     int bc_neg[4];          // boundary sign of direction mu is -1
     int keep;               // links of checkerboard sites below keep stay in L2, the others are evicted first
     int regs;               // EPI_NONE, EPI_M_PART: REGS_* (autotuned)
-    int nbatch;             // split form, EPI_NONE and EPI_M: vectors of one launch (0: one), ...
+    int nbatch;             // training (EPI_NONE, EPI_M): vectors of one launch, in split form; 0 elsewhere: one, ...
     size_t vec_step;        // ... and the bytes between them (in, out and p)
 };
 

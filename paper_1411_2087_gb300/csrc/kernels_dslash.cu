@@ -44,7 +44,7 @@ int split_warps(int prec, const DslashArgs &a) {
     switch (prec) {
     case P_DF64: split = Vh <= 70000 || (Vh > 768 * kSMs && Vh <= 400000); break;
     case P_F64: split = Vh <= 36000; break;
-    case P_F32: split = Vh <= (a.compressed ? 24576 : a.nbatch > 1 ? 85000 : a.keep > 0 ? 70000 : 60000); break;
+    case P_F32: split = Vh <= (a.compressed ? 24576 : a.nbatch > 0 ? 85000 : a.keep > 0 ? 70000 : 60000); break;
     }
     return !split ? 0 : Vh <= 16384 ? 8 : 4;
 }

@@ -509,7 +509,8 @@ static int apply_M_f32(stag_net n, int np, const void *in, void *t, void *out, c
     stag_lattice lat = n->lat;
     const int P = STAG_F32;
     const size_t step = field_bytes(lat, P);
-    // vectors per launch: the split form takes them all, the others one
+    // vectors per launch: the split form takes them all, the others one (a
+    // pair's numbers are the same in a group and alone)
     DslashArgs all = dslash_args(lat, P, STAG_ODD, in, t);
     all.nbatch = np;
     const int per = split_warps(P, all) > 0 ? np : 1;

@@ -154,3 +154,23 @@ def test_decomposed_dslash_takes_the_single_calls_form(prec, compress, Lt):
         assert np.array_equal(slabs.export(), want)
         assert np.array_equal(rank.export(), want)
         d.close()
+
+
+def test_training_pairs_give_the_same_numbers_alone_and_in_groups():
+    """Between the solves' line and the training launches' (groups of three
+    pairs here): the kernels are the same per pair, so a group's loss and
+    gradient are the sums of its pairs' up to FP64 rounding."""
+    dims, mass = (16, 16, 16, 36), 0.1
+    U = links(dims, 103).cpu().numpy()
+    with stag.Lattice(dims) as lat:
+        lat.upload_gauge(U, None, precisions=("df64", "f32"))
+        net = stag.Net(lat, U, 8, 5)
+        net.set_loss("residual")
+        b = lat.field(stag.EVEN, "df64", synth.gaussian_colour_field(2048 * 36, 104).numpy())
+        assert net.collect_pairs(b, mass, 1e-10, 3, 4) == 4
+        loss, grads = net.loss_grad(0, 4)
+        parts = [net.loss_grad(k, 1) for k in range(4)]
+        assert abs(loss - sum(p[0] for p in parts)) <= 1e-10 * abs(loss)
+        for layer, g in enumerate(grads):
+            want = sum(p[1][layer] for p in parts)
+            assert np.abs(g - want).max() <= 1e-10 * max(np.abs(p[1][layer]).max() for p in parts)
