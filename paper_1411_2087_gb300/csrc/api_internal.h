@@ -362,7 +362,10 @@ static inline int m_block(const stag_lattice lat, int prec) {
 // iteration of plain CG, multi-shift CG in double float left to the next
 // kernel against summed by the one block: 80000 sites 84.8, 97.9 against
 // 86.0, 100.2 us, 96000: 99.2, 112.5 against 100.8, 113.0, 128000: 133, 145
-// against 126, 143).
+// against 126, 143; mixed CG at 96000 sites FP32 full links 56.9 against 56.5,
+// 12-real 51.2 / 51.6, 16-bit 44.7 / 45.3, 47.0 / 47.8, at 80000 FP32 full links
+// 53.8 / 52.3, 16-bit 44.3 / 44.1; the learned solvers at 96000 in double float
+// 129.3 / 131.6, with FP32 iterations 84.9 / 84.6, 16-bit 72.1 / 72.5).
 constexpr int kSmallVh = 100000;
 
 // the M Dslash Ap = m^2 p - D_eo t of an iteration (skip_if_done: it returns

@@ -154,6 +154,8 @@ template <bool EXACT> STAG_D float su3_deviation(const double2 *A) {
 // for its own loads at 4 blocks per SM, 2.2 ms as four passes in FP64.  Five
 // blocks hold the registers to 96; six would spill 136 bytes a thread.
 constexpr int SCAN_BLOCKS_PER_SM = 5;
+static_assert(kSMs * SCAN_BLOCKS_PER_SM * SCAN_BLOCK == 97280,
+              "tests/test_gpu_upload.py puts its wrong links at multiples of the links of one sweep");
 
 template <ScanSu3 SU3>
 __global__ void __launch_bounds__(SCAN_BLOCK, SCAN_BLOCKS_PER_SM)

@@ -339,7 +339,7 @@ cudaError_t launch_net_path_coef(int C, const float *w32, const int off[3], int 
 // dL/dc0* (C holomorphic in W: dL/dW* = sum conj(dC/dW) dL/dC*); added to
 // grad.  One warp per weight, the paths it lies on across the lanes (one
 // thread per weight took 240 us, the 64 paths of the first layer's identity
-// weights one after the other in FP64; now 13).
+// weights one after the other in FP64; now 11 to 12).
 constexpr int NET_MAX_W = 9 * (2 * 8 + 8 * 8);
 constexpr int CHAIN_BLOCK = 128;
 
