@@ -135,8 +135,10 @@ struct stag_lattice_s {
     double *staging = nullptr;             // canonical [Vh][3] complex128 for host import/export
     float link_scale[2] = {0.f, 0.f};      // 16-bit links: field max / 32767 (one-link, three-link)
     float *xs = nullptr;                   // F32 correction x_sloppy of the mixed solver
-    unsigned *absmax = nullptr;            // scratch of the field checks
-    LinkScan *scan = nullptr;              // scratch of a gauge upload (two fields)
+    // scratch behind *sc, of a gauge upload's scan (two fields) and of the
+    // field checks: read back before the call that uses it returns
+    LinkScan *scan = nullptr;
+    unsigned *absmax = nullptr;
     struct MixedGraph {
         cudaGraphExec_t exec = nullptr;
         cudaGraph_t graph = nullptr;

@@ -95,13 +95,15 @@ extern "C" int stag_lattice_create(stag_lattice *out, const int dims[4], const d
     }
     const size_t nblk = dslash_max_blocks(Vh) + (size_t)(Vh + 127) / 128 + 1;
     if ((e = cudaMalloc(&lat->partial, sizeof(double) * nblk)) != cudaSuccess ||
-        (e = cudaMalloc(&lat->sc, sizeof(CgScalars))) != cudaSuccess ||
+        (e = cudaMalloc(&lat->sc, sizeof(CgScalars) + 2 * sizeof(LinkScan))) != cudaSuccess ||
         (e = cudaMemset(lat->sc, 0, sizeof(CgScalars))) != cudaSuccess ||
         (e = cudaMallocHost(&lat->sc_host, sizeof(CgScalars))) != cudaSuccess ||
         (e = cudaEventCreate(&lat->ev0)) != cudaSuccess ||
         (e = cudaEventCreate(&lat->ev1)) != cudaSuccess)
         return cleanup(fail(STAG_ERR_NOMEM, "stag_lattice_create: %s", cudaGetErrorString(e)));
     memset(lat->sc_host, 0, sizeof(CgScalars));
+    lat->scan = (LinkScan *)(lat->sc + 1);
+    lat->absmax = (unsigned *)lat->scan;
     *out = lat;
     return STAG_OK;
 }
@@ -160,10 +162,6 @@ extern "C" int stag_lattice_destroy(stag_lattice lat) {
     }
     if (lat->ms_blo)
         cudaFree(lat->ms_blo);
-    if (lat->absmax)
-        cudaFree(lat->absmax);
-    if (lat->scan)
-        cudaFree(lat->scan);
     for (int h = 0; h < 4; h++)
         for (int l = 0; l < 4; l++) {
             if (lat->mixed[h][l].exec)
@@ -317,9 +315,7 @@ extern "C" int stag_gauge_upload(stag_lattice lat, const double *fat, const doub
                 e = cudaMemcpyAsync(scan, lat->scan, sizeof scan, cudaMemcpyDeviceToHost, lat->stream);
             return e == cudaSuccess ? cudaStreamSynchronize(lat->stream) : e;
         };
-        cudaError_t e = lat->scan ? cudaSuccess : cudaMalloc(&lat->scan, 2 * sizeof(LinkScan));
-        if (e == cudaSuccess)
-            e = run_scan(compress ? SCAN_SU3_LIMIT : SCAN_NO_SU3);
+        cudaError_t e = run_scan(compress ? SCAN_SU3_LIMIT : SCAN_NO_SU3);
         if (e != cudaSuccess)
             return refuse(fail(STAG_ERR_CUDA, "gauge scan: %s", cudaGetErrorString(e)));
         const double cf[2] = {std::fabs(c1), std::fabs(c3)};
@@ -551,11 +547,8 @@ static int field_io(stag_field f, const double *src, double *dst, int ptr_kind) 
     }
     if (e == cudaSuccess && src && f->prec != STAG_F64) {
         // the float-based formats hold entries up to the FP32 range only
-        if (!lat->absmax)
-            e = cudaMalloc(&lat->absmax, 2 * sizeof(unsigned));
         unsigned flag = 0;
-        if (e == cudaSuccess)
-            e = launch_finite_overflow(canon, (long long)lat->Vh * 6, lat->absmax, lat->stream);
+        e = launch_finite_overflow(canon, (long long)lat->Vh * 6, lat->absmax, lat->stream);
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(&flag, lat->absmax, sizeof flag, cudaMemcpyDeviceToHost, lat->stream);
         if (e == cudaSuccess)
@@ -836,8 +829,6 @@ int rhs_scale_begin(const stag_field b, RhsScale *rs) {
         return STAG_OK;  // FP64 has the range; 16-bit fields carry a norm per site
     stag_lattice lat = b->lat;
     DEVICE_SCOPE(lat->device);
-    if (!lat->absmax)
-        CUDA_TRY(cudaMalloc(&lat->absmax, 2 * sizeof(unsigned)));
     unsigned bits = 0;
     CUDA_TRY(launch_field_absmax(b->prec, lat->geom, b->data, lat->absmax, lat->stream));
     CUDA_TRY(cudaMemcpyAsync(&bits, lat->absmax, sizeof bits, cudaMemcpyDeviceToHost, lat->stream));
