@@ -260,7 +260,9 @@ struct FoldArgs {
 // per request), and the 32 sites of one parity are written as whole segments
 // of each plane.  Bound by HBM: 24^3x48 into DF64, FP32, 16-bit and the two
 // 12-real copies moves 2.5 GB in 367 us, 6.8 TB/s (2.2 ms in one launch per
-// copy with a thread reading its own link).
+// copy with a thread reading its own link).  Plain stores: copies that fit the L2
+// wait there for the first application (D_oe and D_eo on new 12-real FP32 links
+// at 120960 sites 52 us, 59 with streaming stores, which move no less).
 constexpr int FOLD_BLOCK = 128;
 constexpr int FOLD_LINKS = 64;
 
@@ -312,28 +314,27 @@ fold_kernel(const __grid_constant__ FoldArgs fa, const double *__restrict__ fat,
             const double2 v = L[e];
             const double re = coef * v.x, im = coef * v.y;
             if (fa.out.full[P_F64])
-                __stcs((double2 *)((char *)fa.out.full[P_F64] + par * half) + at + e * S, make_double2(re, im));
+                *((double2 *)((char *)fa.out.full[P_F64] + par * half) + at + e * S) = make_double2(re, im);
             const df dr = df_split(re), di = df_split(im);
             if (fa.out.full[P_DF64])
-                __stcs((float4 *)((char *)fa.out.full[P_DF64] + par * half) + at + e * S,
-                       make_float4(dr.hi, dr.lo, di.hi, di.lo));
+                *((float4 *)((char *)fa.out.full[P_DF64] + par * half) + at + e * S) = make_float4(dr.hi, dr.lo, di.hi, di.lo);
             f[e] = make_float2(dr.hi, di.hi);
         }
         if (fa.out.full[P_F32])
 #pragma unroll
             for (int e = 0; e < 9; e++)
-                __stcs((float2 *)((char *)fa.out.full[P_F32] + par * (half / 2)) + at + e * S, f[e]);
+                *((float2 *)((char *)fa.out.full[P_F32] + par * (half / 2)) + at + e * S) = f[e];
         if (fa.out.c12[P_F32]) {
             char *kb = (char *)fa.out.c12[P_F32] + par * link_parity_bytes(P_F32, mask, S) +
                        link_kind_offset(P_F32, mask, kind, S);
             if (c12) {
 #pragma unroll
                 for (int k = 0; k < 3; k++)
-                    __stcs((float4 *)kb + k * S + cb, make_float4(f[2 * k].x, f[2 * k].y, f[2 * k + 1].x, f[2 * k + 1].y));
+                    *((float4 *)kb + k * S + cb) = make_float4(f[2 * k].x, f[2 * k].y, f[2 * k + 1].x, f[2 * k + 1].y);
             } else {
 #pragma unroll
                 for (int e = 0; e < 9; e++)
-                    __stcs((float2 *)kb + e * S + cb, f[e]);
+                    *((float2 *)kb + e * S + cb) = f[e];
             }
         }
         if (!fa.out.full[P_F16])
@@ -349,12 +350,12 @@ fold_kernel(const __grid_constant__ FoldArgs fa, const double *__restrict__ fat,
                 break;
             const int m = copy ? mask : 0;
             char *kb = base + par * link_parity_bytes(P_F16, m, S) + link_kind_offset(P_F16, m, kind, S);
-            __stcs((int4 *)kb + cb, make_int4(q[0], q[1], q[2], q[3]));
+            *((int4 *)kb + cb) = make_int4(q[0], q[1], q[2], q[3]);
             if (copy && c12) {
-                __stcs((int2 *)(kb + 16 * S) + cb, make_int2(q[4], q[5]));
+                *((int2 *)(kb + 16 * S) + cb) = make_int2(q[4], q[5]);
             } else {
-                __stcs((int4 *)(kb + 16 * S) + cb, make_int4(q[4], q[5], q[6], q[7]));
-                __stcs((int *)(kb + 32 * S) + cb, q[8]);
+                *((int4 *)(kb + 16 * S) + cb) = make_int4(q[4], q[5], q[6], q[7]);
+                *((int *)(kb + 32 * S) + cb) = q[8];
             }
         }
     }
