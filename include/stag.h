@@ -530,7 +530,8 @@ int stag_cg_solve_learned_mixed(stag_net n, stag_field x_even, const stag_field 
  *   fat, lng   complex128 [4][V][3][3] raw links (c1, c3, phases and
  *              boundary signs are applied by the kernel)
  *   in_even    complex128 [Vh][3], out_even complex128 [Vh][3] (distinct)
- * All four must be device memory of the current CUDA device; dims and bc as
+ * All four must be device memory of the current CUDA device, 16-byte aligned
+ * (else STAG_ERR_ARG: nothing could be copied); dims and bc as
  * for stag_lattice_create (bc NULL = {+1,+1,+1,-1}).  FP64 arithmetic.
  *
  * Limit: Vh = V/2 <= 65536 (e.g. 16^4, 16^3 x 32); larger lattices return

@@ -171,10 +171,13 @@ extern "C" int stag_apply_M_noalloc(const int dims[4], const double bc[4], doubl
         return stag::set_error(STAG_ERR_ARG, "stag_apply_M_noalloc: c1, c3, mass must be finite");
     if (in_even == out_even)
         return stag::set_error(STAG_ERR_ARG, "stag_apply_M_noalloc: in and out must differ");
+    const void *ptrs[4] = {fat, lng, in_even, out_even};
+    for (const void *p : ptrs)  // the kernel reads and writes complex numbers 16 bytes at a time
+        if ((uintptr_t)p % 16)
+            return stag::set_error(STAG_ERR_ARG, "stag_apply_M_noalloc: every buffer must be 16-byte aligned");
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64)
         return stag::set_error(STAG_ERR_CUDA, "stag_apply_M_noalloc: no current CUDA device");
-    const void *ptrs[4] = {fat, lng, in_even, out_even};
     for (const void *p : ptrs)
         if (!is_device_pointer_of(p, dev))
             return stag::set_error(STAG_ERR_ARG,
